@@ -1,11 +1,14 @@
 // engine_fp64.cu -- FP64 evaluation of the Stokes single- and double-layer
 // sums (Eq. "sl_stokes", the double-layer kernel of Sec. 2.1, summed as in
-// Sec. 3.1).  Same work items as the mixed engine: a warp holds up to 128
-// targets (T per lane) and walks the item's source segments; sources are
-// 96-byte FP64 records read with warp-uniform (broadcast) loads.  On GB300
-// the FP64 pipe issues about 1/64 of the FP32 rate, so this path is bound by
-// DFMA throughput; it is the accuracy reference form on the GPU.
+// Sec. 3.1).  Same work items as the mixed engine: a warp takes up to 128
+// targets against the item's source segments, read with warp-uniform
+// (broadcast) loads.  On GB300 the FP64 pipe runs at about 1/64 of the FP32
+// rate, so a pair written in FP64 alone is bound by it: k_engine_fp64, which
+// remains for inputs that fixed point does not fit.  k_engine_fx evaluates the
+// differences, dot products and reciprocals in fixed point (fixed_pair.cuh).
+// Both are launched; the packing decides on the device which of them works.
 #include "common.cuh"
+#include "fixed_pair.cuh"
 #include "prep.cuh"
 
 namespace stk {
@@ -99,7 +102,8 @@ __device__ void run_item64(const EngineParams &P, const Item &it, int b, int lan
   }
 }
 
-__global__ void __launch_bounds__(kWarpsPerCta *kWarp, 4) k_engine_fp64(EngineParams P) {
+__global__ void __launch_bounds__(kWarpsPerCta *kWarp, 4) k_engine_fp64(EngineParams P, FxParams F) {
+  if (fx_use(*F.state, F.ns)) return;  // k_engine_fx does the call
   const int lane = threadIdx.x & (kWarp - 1);
   const int n_items = *P.n_items;
   while (true) {
@@ -138,14 +142,243 @@ __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 4) k_engine_fp64(EnginePa
   }
 }
 
-cudaError_t launch_engine_fp64(const EngineParams &P, int grid, cudaStream_t stream) {
-  k_engine_fp64<<<grid, kWarpsPerCta * kWarp, 0, stream>>>(P);
+// ------------------------------------------------------------ fixed point
+// The FP64 form of a pair that fixed point cannot hold; n and psi from their
+// fixed point parts (61 bits on the vector's own exponent).
+template <int KIND>
+__device__ __noinline__ void fx_slow(const double *xp, const double *yp, const SrcFx *S,
+                                     double *acc) {
+  const double dx = xp[0] - yp[0], dy = xp[1] - yp[1], dz = xp[2] - yp[2];
+  const double r2 = dx * dx + dy * dy + dz * dz;
+  if (!(r2 > 0.0)) return;  // zero-distance pair contributes nothing
+  const double ri = rsqrt(r2), ri2 = ri * ri;
+  double c = 0.0;
+  if (KIND & K_DL) {
+    double n[3], p[3];
+    for (int k = 0; k < 3; ++k) {
+      n[k] = ldexp((double)(((int64_t)S->nh[k] << 30) + S->nl[k]), -60);
+      p[k] = ldexp((double)(((int64_t)S->ph[k] << 30) + S->pl[k]), S->epn - 60);
+    }
+    c = (dx * p[0] + dy * p[1] + dz * p[2]) * (dx * n[0] + dy * n[1] + dz * n[2]);
+  }
+  const double d[3] = {dx, dy, dz};
+  if (KIND & K_SL) {
+    c = (dx * S->q[0] + dy * S->q[1] + dz * S->q[2] + c * ri2) * ri2;
+    for (int k = 0; k < 3; ++k) acc[k] += (S->q[k] + d[k] * c) * ri;
+  } else {
+    c *= ri2 * ri2 * ri;
+    for (int k = 0; k < 3; ++k) acc[k] += d[k] * c;
+  }
+}
+
+template <int KIND>
+__device__ __forceinline__ void seg_fx(const EngineParams &P, const SrcFx *__restrict__ rec, int64_t s, int64_t e, int b, int E,
+                                       const int64_t (&X)[3], int32_t xflag, const double *xp,
+                                       double (&acc)[3]) {
+  for (int64_t k = s; k < e; k += b) {
+    const SrcFx &S = rec[k];
+    if (!fx_pair<KIND>(X, xflag, E, S, acc)) {
+      double a[3] = {acc[0], acc[1], acc[2]};
+      fx_slow<KIND>(xp, P.src64 + 3 * (size_t)k, &S, a);
+      acc[0] = a[0];
+      acc[1] = a[1];
+      acc[2] = a[2];
+    }
+  }
+}
+
+// An item's tn targets and b source slices make tn b columns, one per lane,
+// 32 to a pass over the item's sources; b is chosen so that the last pass is
+// nearly full (a pair costs some 700 cycles of a warp, its loads nothing).  The
+// slices' sums meet in shared memory and are added in slice order.
+constexpr int kFxCols = 256, kFxSlices = 16;
+
+//
+// Bound: the FP64 pipe, 9 instructions of about 68 cycles per warp and SL + DL
+// pair, with some 190 integer and FP32 instructions beside them (six CTAs per
+// SM so that one warp's integer part overlaps another's FP64 part).  SL + DL of
+// 34,816 points on themselves: 71.5 -> 19.9 ms (k_engine_fp64 -> this), near
+// field of 262,096 points: 44.3 -> 7.5 ms (24.2 ms with items of 128 targets,
+// whose last round left the GPU idle).
+template <int KMODE>
+__global__ void __launch_bounds__(kWarpsPerCta *kWarp, 6) k_engine_fx(EngineParams P, FxParams F) {
+  __shared__ double sums[kWarpsPerCta][3][kFxCols];
+  const FxState fs = *F.state;
+  if (!fx_use(fs, F.ns)) return;  // k_engine_fp64 does the call
+  const int E = fx_exp(fs);
+  double(*R)[kFxCols] = sums[threadIdx.x / kWarp];
+  const int lane = threadIdx.x & (kWarp - 1);
+  const int n_items = *P.n_items;
+  while (true) {
+    int idx = 0;
+    if (lane == 0) idx = atomicAdd(P.item_counter, 1);
+    idx = __shfl_sync(kFull, idx, 0);
+    if (idx >= n_items) break;
+    const Item it = P.items[P.item_order ? P.item_order[idx] : idx];
+    const int tn = it.tn_part & 0xFF, part = it.tn_part >> 8;
+    // slices: fewest lanes idle, at most kFxCols columns
+    int b = 1;
+    for (int c = 2, idle = ((tn + 31) & ~31) - tn, cols = tn;
+         c <= kFxSlices && idle * 16 > cols && c * tn <= kFxCols; ++c) {
+      const int n = c * tn, w = ((n + 31) & ~31) - n;
+      if (w * cols < idle * n) {
+        idle = w;
+        cols = n;
+        b = c;
+      }
+    }
+    const int ncol = b * tn;
+    for (int c0 = 0; c0 < ncol; c0 += kWarp) {
+      const int col = min(c0 + lane, ncol - 1);
+      const int sl = col / tn, t = it.t0 + col % tn;
+      const double *xp = P.trg64 + 3 * (size_t)(P.tperm ? P.tperm[t] : t);
+      int64_t X[3];
+      int32_t xflag = 0;
+      double acc[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        X[k] = fx_coord(xp[k], E, xflag);
+        acc[k] = 0.0;
+      }
+      for (int e = it.seg0; e < it.seg1; ++e) {
+        int sid = P.seg_list ? P.seg_list[e] : e;
+        const int64_t s = P.range_ptr[sid] + sl;
+        int64_t en = P.range_ptr[sid + 1];
+        if (KMODE && P.seg_list)  // contiguous segments as one, so that slices come out even
+          while (e + 1 < it.seg1 && P.range_ptr[sid = P.seg_list[e + 1]] == en) {
+            en = P.range_ptr[sid + 1];
+            ++e;
+          }
+        if (KMODE ? KMODE == K_SL : !(sid & 1))
+          seg_fx<K_SL>(P, F.rec, s, en, b, E, X, xflag, xp, acc);
+        else if (KMODE ? KMODE == K_DL : true)
+          seg_fx<K_DL>(P, F.rec, s, en, b, E, X, xflag, xp, acc);
+        else
+          seg_fx<K_SLDL>(P, F.rec, s, en, b, E, X, xflag, xp, acc);
+      }
+      if (c0 + lane < ncol)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) R[k][col] = acc[k];
+    }
+    __syncwarp();
+    double *out = P.part_out + ((size_t)part * (size_t)P.nt + (size_t)it.t0) * 3;
+    for (int v = lane; v < 3 * tn; v += kWarp) {
+      const int t = v / 3, k = v % 3;
+      double a = R[k][t];
+      for (int sl = 1; sl < b; ++sl) a += R[k][sl * tn + t];
+      out[v] = a;
+    }
+    __syncwarp();
+  }
+}
+
+// Largest coordinate exponent of the sources and (when they differ) targets.
+__global__ void k_fx_range(int64_t ns, const double *__restrict__ src, int64_t nt,
+                           const double *__restrict__ trg, FxState *__restrict__ st) {
+  const int64_t n = 3 * ns, m = n + 3 * nt;
+  int f = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
+       i += (int64_t)gridDim.x * blockDim.x)
+    f = max(f, fx_field(i < n ? src[i] : trg[i - n]));
+  f = __reduce_max_sync(kFull, f);
+  if ((threadIdx.x & 31) == 0) atomicMax(&st->field, f);
+}
+
+__global__ void k_pack_fx(int64_t ns, const double *__restrict__ src, const double *__restrict__ f,
+                          const double *__restrict__ nrm, const double *__restrict__ phi,
+                          const double *__restrict__ w, double csl, double cdl,
+                          FxState *__restrict__ st, SrcFx *__restrict__ rec) {
+  const int E = st->field - 1022;
+  if (E > kFxMaxExp || E < -kFxMaxExp) return;
+  int bad = 0, inexact = 0;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
+       j += (int64_t)gridDim.x * blockDim.x) {
+    SrcFx R;
+    const double wj = w ? w[j] : 1.0;
+    double n[3], p[3];
+    R.flag = 0;
+    for (int k = 0; k < 3; ++k) {
+      R.y[k] = fx_coord(src[3 * j + k], E, R.flag);
+      R.q[k] = f ? wj * csl * f[3 * j + k] : 0.0;
+      n[k] = phi ? nrm[3 * j + k] : 0.0;
+      p[k] = phi ? wj * cdl * phi[3 * j + k] : 0.0;
+    }
+    const int eq = fx_block(R.q, R.qh, R.ql), en = fx_block(n, R.nh, R.nl),
+              ep = fx_block(p, R.ph, R.pl);
+    const bool ok = eq <= kFxMaxExp && eq >= -kFxMaxExp && en <= kFxMaxExp && en >= -kFxMaxExp &&
+                    ep <= kFxMaxExp && ep >= -kFxMaxExp;
+    R.eq = (int16_t)eq;
+    R.epn = (int16_t)(en + ep);
+    bad |= !ok;
+    inexact += R.flag;
+    rec[j] = R;
+  }
+  if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) st->bad = 1;
+  inexact = __reduce_add_sync(kFull, inexact);
+  if (inexact && (threadIdx.x & 31) == 0) atomicAdd(&st->inexact, inexact);
+}
+
+__global__ void k_pack_fp64(int64_t ns, const double *__restrict__ src,
+                            const double *__restrict__ f, const double *__restrict__ nrm,
+                            const double *__restrict__ phi, const double *__restrict__ w,
+                            double csl, double cdl, const FxState *__restrict__ fx,
+                            SrcRec64 *__restrict__ rec) {
+  if (fx && fx_use(*fx, ns)) return;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
+       j += (int64_t)gridDim.x * blockDim.x) {
+    SrcRec64 R;
+    const double wj = w ? w[j] : 1.0;
+    for (int k = 0; k < 3; ++k) {
+      R.y[k] = src[3 * j + k];
+      R.q[k] = f ? wj * csl * f[3 * j + k] : 0.0;
+      R.n[k] = phi ? nrm[3 * j + k] : 0.0;
+      R.p[k] = phi ? wj * cdl * phi[3 * j + k] : 0.0;
+    }
+    rec[j] = R;
+  }
+}
+
+static int pack_grid(int64_t n) {
+  int64_t g = (n + 255) / 256;
+  return (int)(g < 1 ? 1 : g > 4096 ? 4096 : g);
+}
+
+void launch_pack_fp64(int64_t ns, const double *src, const double *f, const double *nrm,
+                      const double *phi, const double *w, double csl, double cdl, SrcRec64 *rec,
+                      cudaStream_t st) {
+  k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, nullptr, rec);
   count_launches(1);
+}
+
+void launch_pack_fx(int64_t ns, const double *src, int64_t nt, const double *trg, const double *f,
+                    const double *nrm, const double *phi, const double *w, double csl, double cdl,
+                    FxState *fx, SrcFx *recfx, SrcRec64 *rec, cudaStream_t st) {
+  k_fx_range<<<pack_grid(3 * ns + 3 * nt), 256, 0, st>>>(ns, src, nt, trg, fx);
+  k_pack_fx<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, fx, recfx);
+  k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, fx, rec);
+  count_launches(3);
+}
+
+cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,
+                               cudaStream_t stream) {
+  if (P.kind_alternating)
+    k_engine_fx<0><<<grid_fx, kWarpsPerCta * kWarp, 0, stream>>>(P, F);
+  else if (P.kind == K_SL)
+    k_engine_fx<K_SL><<<grid_fx, kWarpsPerCta * kWarp, 0, stream>>>(P, F);
+  else if (P.kind == K_DL)
+    k_engine_fx<K_DL><<<grid_fx, kWarpsPerCta * kWarp, 0, stream>>>(P, F);
+  else
+    k_engine_fx<K_SLDL><<<grid_fx, kWarpsPerCta * kWarp, 0, stream>>>(P, F);
+  k_engine_fp64<<<grid, kWarpsPerCta * kWarp, 0, stream>>>(P, F);
+  count_launches(2);
   return cudaGetLastError();
 }
 
-cudaError_t engine_fp64_occupancy(int *blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_engine_fp64,
+cudaError_t engine_fp64_occupancy(int *blocks_per_sm, int *blocks_per_sm_fx) {
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_engine_fp64,
+                                                                kWarpsPerCta * kWarp, 0);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm_fx, k_engine_fx<K_SLDL>,
                                                        kWarpsPerCta * kWarp, 0);
 }
 

@@ -59,24 +59,6 @@ __global__ void k_pack_mixed(int64_t ns, const double *__restrict__ src,
   }
 }
 
-__global__ void k_pack_fp64(int64_t ns, const double *__restrict__ src,
-                            const double *__restrict__ f, const double *__restrict__ nrm,
-                            const double *__restrict__ phi, const double *__restrict__ w,
-                            double csl, double cdl, SrcRec64 *__restrict__ rec) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    SrcRec64 R;
-    const double wj = w ? w[j] : 1.0;
-    for (int k = 0; k < 3; ++k) {
-      R.y[k] = src[3 * j + k];
-      R.q[k] = f ? wj * csl * f[3 * j + k] : 0.0;
-      R.n[k] = phi ? nrm[3 * j + k] : 0.0;
-      R.p[k] = phi ? wj * cdl * phi[3 * j + k] : 0.0;
-    }
-    rec[j] = R;
-  }
-}
-
 // ---------------------------------------------------------------- bbox
 constexpr int kRedThreads = 256;
 
@@ -508,13 +490,6 @@ void launch_pack_mixed(int64_t ns, const double *src, const double *f, const dou
                        double csl, double cdl, const double *cen, SrcRec *rec, cudaStream_t st) {
   k_pack_mixed<<<grid_for(ns, 256), 256, 0, st>>>(ns, src, f, nrm, phi, w, h, alpha, csl, cdl,
                                                   cen ? cen : src, rec);
-  count_launches(1);
-}
-
-void launch_pack_fp64(int64_t ns, const double *src, const double *f, const double *nrm,
-                      const double *phi, const double *w, double csl, double cdl, SrcRec64 *rec,
-                      cudaStream_t st) {
-  k_pack_fp64<<<grid_for(ns, 256), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, rec);
   count_launches(1);
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "fixed_pair.cuh"
 
 namespace stk {
 
@@ -15,6 +16,12 @@ void launch_pack_mixed(int64_t ns, const double *src, const double *f, const dou
 void launch_pack_fp64(int64_t ns, const double *src, const double *f, const double *nrm,
                       const double *phi, const double *w, double csl, double cdl, SrcRec64 *rec,
                       cudaStream_t st);
+// Records of both FP64 engines (engine_fp64.cu): the fixed point form's, and
+// the plain ones where it does not fit; *fx is zero before the call.  trg: the
+// targets where they are not the sources (nt = 0 otherwise).
+void launch_pack_fx(int64_t ns, const double *src, int64_t nt, const double *trg, const double *f,
+                    const double *nrm, const double *phi, const double *w, double csl, double cdl,
+                    FxState *fx, SrcFx *recfx, SrcRec64 *rec, cudaStream_t st);
 int bbox_partial_blocks(int64_t n);
 void launch_bbox(int64_t n, const double *pts, double *partial, double *box, cudaStream_t st);
 void launch_morton(int64_t n, const double *pts, const double *box, const int64_t *group_ptr,
@@ -84,7 +91,9 @@ void launch_adj_finish(bool src_major, int64_t n, int32_t nsplit, const double *
 size_t engine_mixed_smem_bytes();
 cudaError_t launch_engine_mixed(const EngineParams &P, int grid, cudaStream_t stream);
 cudaError_t engine_mixed_occupancy(int *blocks_per_sm);
-cudaError_t launch_engine_fp64(const EngineParams &P, int grid, cudaStream_t stream);
-cudaError_t engine_fp64_occupancy(int *blocks_per_sm);
+// Launches both FP64 engines (grids of resident CTAs); *F.state picks one.
+cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,
+                               cudaStream_t stream);
+cudaError_t engine_fp64_occupancy(int *blocks_per_sm, int *blocks_per_sm_fx);
 
 }  // namespace stk

@@ -68,6 +68,7 @@ struct DevInfo {
   int sms = 0;
   int occ_mixed = 0;
   int occ_fp64 = 0;
+  int occ_fx = 0;
 };
 
 cudaError_t dev_info(DevInfo &di) {
@@ -84,10 +85,11 @@ cudaError_t dev_info(DevInfo &di) {
     if (e != cudaSuccess) return e;
     e = engine_mixed_occupancy(&n.occ_mixed);
     if (e != cudaSuccess) return e;
-    e = engine_fp64_occupancy(&n.occ_fp64);
+    e = engine_fp64_occupancy(&n.occ_fp64, &n.occ_fx);
     if (e != cudaSuccess) return e;
     if (n.occ_mixed < 1) n.occ_mixed = 1;
     if (n.occ_fp64 < 1) n.occ_fp64 = 1;
+    if (n.occ_fx < 1) n.occ_fx = 1;
     c = n;
   }
   di = c;
@@ -119,7 +121,7 @@ struct Plan {
   bool small = false;  // the one-launch small direct form (direct_small.cu)
   int32_t ngroup = 0;
   // offsets (the counters always sit at offset 0 of the aligned workspace)
-  size_t counters, rec, keys_a, keys_b, vals_a, vals_b, ikeys_a, ikeys_b, ivals_a, ivals_b, hist,
+  size_t counters, rec, recfx = 0, keys_a, keys_b, vals_a, vals_b, ikeys_a, ikeys_b, ivals_a, ivals_b, hist,
       hist_scan, bbox_part, bbox, items, range, cnt, offs, part, frames = 0, xloc = 0,
       cand_list = 0, cand_cnt = 0, total;
 };
@@ -127,13 +129,26 @@ struct Plan {
 // Candidate sources the engine lists per item for k_near (items with more are
 // rescanned by k_near).
 constexpr int32_t kCandCap = 512;
+// Counters at the head of the workspace: items, engine queue, error word, near
+// queue, then the FP64 form's FxState.
+constexpr int kCounters = 8;
+constexpr int kFxCounter = 4;
 
-int auto_splits(int64_t nt, int64_t ns, const DevInfo &di, int occ) {
-  const int64_t chunks = (nt + kItemMax - 1) / kItemMax;
+// The FP64 form's items are an eighth of the mixed form's: a pair costs some
+// 700 cycles of a warp there against some 25, an item's set-up and loads are
+// nothing beside it, and the last items of a launch have to be short (262,096
+// points' near field: 24.2 ms with items of 128 targets, see engine_fp64.cu).
+constexpr int kFp64ItemDiv = 8;
+
+// Splits of a direct sum's sources.  The mixed engine takes two items per
+// resident warp, the FP64 form eight.
+int auto_splits(int64_t nt, int64_t ns, const DevInfo &di, bool mixed, int item_max) {
+  const int64_t chunks = (nt + item_max - 1) / item_max;
   if (chunks <= 0) return 1;
-  const int64_t warps = (int64_t)di.sms * occ * kWarpsPerCta;
-  int64_t s = (2 * warps + chunks - 1) / chunks;
-  const int64_t cap = ns / 64 > 1 ? ns / 64 : 1;  // at least 64 sources per split
+  const int64_t warps = (int64_t)di.sms * (mixed ? di.occ_mixed : di.occ_fx) * kWarpsPerCta;
+  int64_t s = ((mixed ? 2 : 8) * warps + chunks - 1) / chunks;
+  const int64_t least = mixed ? 64 : 32;  // sources per split
+  const int64_t cap = ns / least > 1 ? ns / least : 1;
   if (s > cap) s = cap;
   if (s > 64) s = 64;
   if (s < 1) s = 1;
@@ -142,7 +157,7 @@ int auto_splits(int64_t nt, int64_t ns, const DevInfo &di, int occ) {
 
 void layout(Plan &p) {
   Alloc a;
-  p.counters = a.take(sizeof(int32_t) * 4);
+  p.counters = a.take(sizeof(int32_t) * kCounters);
   if (p.small) {  // partial results per source split and a counter per target block
     p.cnt = a.take(sizeof(int32_t) * (size_t)direct_small_blocks(p.nt));
     p.part = a.take(sizeof(double) * 3 * (size_t)p.nt * (size_t)p.nsplit);
@@ -150,6 +165,7 @@ void layout(Plan &p) {
     return;
   }
   p.rec = a.take((size_t)p.ns * (p.mixed ? sizeof(SrcRec) : sizeof(SrcRec64)));
+  if (!p.mixed) p.recfx = a.take((size_t)p.ns * sizeof(SrcFx));
   const int64_t nsort = p.sort_targets ? p.nt : 0;
   const int64_t nitem = p.sort_items ? p.max_items : 0;
   p.keys_a = a.take(sizeof(uint64_t) * (size_t)nsort);
@@ -180,12 +196,20 @@ void layout(Plan &p) {
   p.total = a.off + 256;  // slack for re-alignment of an unaligned base
 }
 
+TileConfig form_tile(const stk_opts *o) {
+  TileConfig t = tile_config(o->tile_config < 0 ? 0 : o->tile_config);
+  if (o->precision != STK_MIXED) t.item_max /= kFp64ItemDiv;
+  return t;
+}
+// The smallest item size of a precision: bounds the item count of any tile.
+int least_item(bool mixed) { return mixed ? kMinItemMax : kMinItemMax / kFp64ItemDiv; }
+
 stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
   DevInfo di;
   CU(dev_info(di));
   p.form = F_DIRECT;
   p.mixed = o->precision == STK_MIXED;
-  p.tile = tile_config(o->tile_config < 0 ? 0 : o->tile_config);
+  p.tile = form_tile(o);
   p.ns = ns;
   p.nt = nt;
   // small mixed sums with the default options: one launch and the finish
@@ -196,11 +220,12 @@ stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
     layout(p);
     return STK_OK;
   }
-  const int occ = p.mixed ? di.occ_mixed : di.occ_fp64;
-  p.nsplit = o->source_splits > 0 ? o->source_splits : auto_splits(nt, ns, di, occ);
+  p.nsplit = o->source_splits > 0
+                 ? o->source_splits
+                 : auto_splits(nt, ns, di, p.mixed, p.mixed ? kItemMax : p.tile.item_max);
   if (p.nsplit > ns && ns > 0) p.nsplit = (int32_t)ns;
   if (p.nsplit < 1) p.nsplit = 1;
-  p.max_items = ((nt + kMinItemMax - 1) / kMinItemMax) * p.nsplit;
+  p.max_items = ((nt + least_item(p.mixed) - 1) / least_item(p.mixed)) * p.nsplit;
   p.nseg_ranges = p.nsplit;
   p.sort_targets = p.mixed;
   p.sort_items = false;
@@ -212,10 +237,10 @@ stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
 stk_status plan_p2p(int64_t n, int32_t nleaf, const stk_opts *o, Plan &p) {
   p.form = F_P2P;
   p.mixed = o->precision == STK_MIXED;
-  p.tile = tile_config(o->tile_config < 0 ? 0 : o->tile_config);
+  p.tile = form_tile(o);
   p.ns = p.nt = n;
   p.nsplit = 1;
-  p.max_items = (int64_t)nleaf + n / kMinItemMax + 1;
+  p.max_items = (int64_t)nleaf + n / least_item(p.mixed) + 1;
   p.nseg_ranges = nleaf;
   p.sort_targets = false;
   p.sort_items = true;
@@ -227,10 +252,10 @@ stk_status plan_p2p(int64_t n, int32_t nleaf, const stk_opts *o, Plan &p) {
 stk_status plan_batched(int64_t n, int32_t nsusp, const stk_opts *o, Plan &p) {
   p.form = F_BATCHED;
   p.mixed = o->precision == STK_MIXED;
-  p.tile = tile_config(o->tile_config < 0 ? 0 : o->tile_config);
+  p.tile = form_tile(o);
   p.ns = p.nt = n;
   p.nsplit = 1;
-  p.max_items = (int64_t)nsusp + n / kMinItemMax + 1;
+  p.max_items = (int64_t)nsusp + n / least_item(p.mixed) + 1;
   p.nseg_ranges = 2 * nsusp;
   p.sort_targets = p.mixed;
   p.sort_items = true;
@@ -360,7 +385,11 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
     CU(launch_engine_mixed(P, (int)grid, st));
   } else {
     P.rec64 = at<SrcRec64>(ws, p.rec);
-    CU(launch_engine_fp64(P, (int)grid, st));
+    const FxParams F{at<SrcFx>(ws, p.recfx), reinterpret_cast<const FxState *>(counters + kFxCounter),
+                     p.ns};
+    int64_t grid_fx = (int64_t)di.sms * di.occ_fx;
+    if (grid_fx > need) grid_fx = need;
+    CU(launch_engine_fp64(P, F, (int)grid, (int)(grid_fx < 1 ? 1 : grid_fx), st));
   }
   if (g_ev_start && g_ev_stop) CU(cudaEventRecord(g_ev_stop, st));
   if (p.mixed) {
@@ -371,14 +400,16 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
 }
 
 stk_status pack(const Plan &p, void *ws, const double *src, const double *f, const double *nrm,
-                const double *phi, const double *w, const double *h, double mu, double alpha,
-                cudaStream_t st) {
+                const double *phi, const double *w, const double *h, const double *trg, double mu,
+                double alpha, cudaStream_t st) {
   const double csl = 1.0 / (8.0 * kPi * mu), cdl = 6.0 / (8.0 * kPi);
   if (p.mixed)
     launch_pack_mixed(p.ns, src, f, nrm, phi, w, h, alpha, csl, cdl, src, at<SrcRec>(ws, p.rec),
                       st);
   else
-    launch_pack_fp64(p.ns, src, f, nrm, phi, w, csl, cdl, at<SrcRec64>(ws, p.rec), st);
+    launch_pack_fx(p.ns, src, trg == src ? 0 : p.nt, trg, f, nrm, phi, w, csl, cdl,
+                   reinterpret_cast<FxState *>(at<int32_t>(ws, p.counters) + kFxCounter),
+                   at<SrcFx>(ws, p.recfx), at<SrcRec64>(ws, p.rec), st);
   CU(cudaGetLastError());
   return STK_OK;
 }
@@ -457,9 +488,9 @@ stk_status direct_common(int32_t kinds, const double *src, const double *f, cons
                            at<int32_t>(ws, p.cnt), out, st));
     return STK_OK;
   }
-  launch_zero_ints(at<int32_t>(ws, p.counters), 4, st);
+  launch_zero_ints(at<int32_t>(ws, p.counters), kCounters, st);
   s = pack(p, ws, src, (kinds & K_SL) ? f : nullptr, nrm, (kinds & K_DL) ? phi : nullptr, w, h,
-           (kinds & K_SL) ? mu : 1.0, o->near_ratio, st);
+           trg, (kinds & K_SL) ? mu : 1.0, o->near_ratio, st);
   if (s != STK_OK) return s;
   EngineParams P;
   std::memset(&P, 0, sizeof(P));
@@ -674,11 +705,11 @@ stk_status stokes_p2p_leaflists(const double *pts, const double *f, const double
   if (s != STK_OK) return s;
   if (!workspace || workspace_bytes < p.total) return fail(STK_ENOMEM, "workspace too small");
   void *ws = align_ws(workspace);
-  launch_zero_ints(at<int32_t>(ws, p.counters), 4, st);
+  launch_zero_ints(at<int32_t>(ws, p.counters), kCounters, st);
   // the packing runs beside the item build (they meet at the engine)
   SideStream *sd = fork_side(st);
   s = pack(p, ws, pts, (kernels & K_SL) ? f : nullptr, nrm, (kernels & K_DL) ? phi : nullptr, w,
-           h, (kernels & K_SL) ? mu : 1.0, opts->near_ratio, sd ? sd->s : st);
+           h, pts, (kernels & K_SL) ? mu : 1.0, opts->near_ratio, sd ? sd->s : st);
   if (s != STK_OK) return s;
   if (sd) CU(cudaEventRecord(sd->join, sd->s));
   int64_t *range = at<int64_t>(ws, p.range);
@@ -745,8 +776,8 @@ stk_status stokes_batched_eval(const double *pts, const double *f, const double 
   if (s != STK_OK) return s;
   if (!workspace || workspace_bytes < p.total) return fail(STK_ENOMEM, "workspace too small");
   void *ws = align_ws(workspace);
-  launch_zero_ints(at<int32_t>(ws, p.counters), 4, st);
-  s = pack(p, ws, pts, f, nrm, phi, w, h, mu, opts->near_ratio, st);
+  launch_zero_ints(at<int32_t>(ws, p.counters), kCounters, st);
+  s = pack(p, ws, pts, f, nrm, phi, w, h, pts, mu, opts->near_ratio, st);
   if (s != STK_OK) return s;
   EngineParams P;
   std::memset(&P, 0, sizeof(P));
