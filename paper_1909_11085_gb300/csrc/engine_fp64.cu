@@ -173,11 +173,11 @@ __device__ __noinline__ void fx_slow(const double *xp, const double *yp, const S
 
 template <int KIND>
 __device__ __forceinline__ void seg_fx(const EngineParams &P, const SrcFx *__restrict__ rec, int64_t s, int64_t e, int b, int E,
-                                       const int64_t (&X)[3], int32_t xflag, const double *xp,
+                                       const int64_t (&X)[3], uint32_t xthr, const double *xp,
                                        double (&acc)[3]) {
   for (int64_t k = s; k < e; k += b) {
     const SrcFx &S = rec[k];
-    if (!fx_pair<KIND>(X, xflag, E, S, acc)) {
+    if (!fx_pair<KIND>(X, xthr, E, S, acc)) {
       double a[3] = {acc[0], acc[1], acc[2]};
       fx_slow<KIND>(xp, P.src64 + 3 * (size_t)k, &S, a);
       acc[0] = a[0];
@@ -233,11 +233,11 @@ __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 6) k_engine_fx(EnginePara
       const int sl = col / tn, t = it.t0 + col % tn;
       const double *xp = P.trg64 + 3 * (size_t)(P.tperm ? P.tperm[t] : t);
       int64_t X[3];
-      int32_t xflag = 0;
+      uint32_t xthr = kFxExact;
       double acc[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        X[k] = fx_coord(xp[k], E, xflag);
+        X[k] = fx_coord(xp[k], E, xthr);
         acc[k] = 0.0;
       }
       for (int e = it.seg0; e < it.seg1; ++e) {
@@ -250,11 +250,11 @@ __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 6) k_engine_fx(EnginePara
             ++e;
           }
         if (KMODE ? KMODE == K_SL : !(sid & 1))
-          seg_fx<K_SL>(P, F.rec, s, en, b, E, X, xflag, xp, acc);
+          seg_fx<K_SL>(P, F.rec, s, en, b, E, X, xthr, xp, acc);
         else if (KMODE ? KMODE == K_DL : true)
-          seg_fx<K_DL>(P, F.rec, s, en, b, E, X, xflag, xp, acc);
+          seg_fx<K_DL>(P, F.rec, s, en, b, E, X, xthr, xp, acc);
         else
-          seg_fx<K_SLDL>(P, F.rec, s, en, b, E, X, xflag, xp, acc);
+          seg_fx<K_SLDL>(P, F.rec, s, en, b, E, X, xthr, xp, acc);
       }
       if (c0 + lane < ncol)
 #pragma unroll
@@ -296,9 +296,9 @@ __global__ void k_pack_fx(int64_t ns, const double *__restrict__ src, const doub
     SrcFx R;
     const double wj = w ? w[j] : 1.0;
     double n[3], p[3];
-    R.flag = 0;
+    R.thr = kFxExact;
     for (int k = 0; k < 3; ++k) {
-      R.y[k] = fx_coord(src[3 * j + k], E, R.flag);
+      R.y[k] = fx_coord(src[3 * j + k], E, R.thr);
       R.q[k] = f ? wj * csl * f[3 * j + k] : 0.0;
       n[k] = phi ? nrm[3 * j + k] : 0.0;
       p[k] = phi ? wj * cdl * phi[3 * j + k] : 0.0;
@@ -310,7 +310,7 @@ __global__ void k_pack_fx(int64_t ns, const double *__restrict__ src, const doub
     R.eq = (int16_t)eq;
     R.epn = (int16_t)(en + ep);
     bad |= !ok;
-    inexact += R.flag;
+    inexact += R.thr != kFxExact;
     rec[j] = R;
   }
   if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) st->bad = 1;

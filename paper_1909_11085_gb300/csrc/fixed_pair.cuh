@@ -112,10 +112,16 @@ FX_HD double fx_fma(double a, double b, double c) {
 // ------------------------------------------------------------------- storage
 constexpr uint32_t kFxLow = 0x3fffffffu;  // the low part: 30 bits
 
+// A pair whose largest |d_k| has a high word below both points' thresholds
+// takes the FP64 form.
+constexpr uint32_t kFxExact = 1u;          // exact coordinates: |d| < 2^32 quanta
+constexpr uint32_t kFxInexact = 1u << 22;  // an inexact coordinate: |d| < 2^54 quanta
+constexpr uint32_t kFxNever = ~0u;         // nothing of the point fits
+
 // Positions on the grid, and block fixed point vectors (value = (h 2^30 + l) 2^(e - 60)).
 struct alignas(16) SrcFx {
   int64_t y[3];
-  int32_t flag;      // 1: a coordinate is inexact
+  uint32_t thr;      // threshold (above)
   int16_t eq, epn;   // exponent of q; of psi and n together
   double q[3];
   int32_t qh[3], ql[3], nh[3], nl[3], ph[3], pl[3];
@@ -148,27 +154,33 @@ FX_HD bool fx_use(const FxState &s, int64_t ns) {
 }
 
 // A coordinate on the grid of exponent E (|v| < 2^E, kFxMaxExp >= |E|),
-// rounded to nearest; inexact is set when bits are dropped.
-FX_HD int64_t fx_coord(double v, int E, int32_t &inexact) {
+// rounded to nearest; thr is raised when bits are dropped.
+FX_HD int64_t fx_coord(double v, int E, uint32_t &thr) {
   const uint64_t u = fx_to_bits(v);
   const int ef = (int)((u >> 52) & 0x7ff);
   if (ef == 0) {  // zero or far below the quantum
-    if (u << 1) inexact = 1;
+    if ((u << 1) && thr < kFxInexact) thr = kFxInexact;
     return 0;
   }
   const uint64_t m = (u & 0xfffffffffffffull) | (1ull << 52);
   const int s = ef - 1013 - E;  // m 2^(ef - 1075) = m 2^s quanta
   uint64_t a;
+  if (s > 9) {  // outside the grid (the engine's never are)
+    thr = kFxNever;
+    return 0;
+  }
+  bool inexact = false;
   if (s >= 0) {
-    a = m << s;  // s <= 9
+    a = m << s;
   } else if (s < -54) {
-    inexact = 1;
+    inexact = true;
     a = 0;
   } else {
     const int r = -s;
-    if (m & ((1ull << r) - 1)) inexact = 1;
+    inexact = (m & ((1ull << r) - 1)) != 0;
     a = (m + (1ull << (r - 1))) >> r;
   }
+  if (inexact && thr < kFxInexact) thr = kFxInexact;
   return (u >> 63) ? -(int64_t)a : (int64_t)a;
 }
 
@@ -286,13 +298,15 @@ FX_HD uint64_t fx_rsqrt(int64_t W, int &b) {
 }
 
 // ----------------------------------------------------------------------- pair
-// What one pair needs besides the source: returns false when the pair has to
-// take the FP64 form, else adds it to acc.
-//   SL:   q/r + d (d.q)/r^3,  DL: d (d.psi)(d.n)/r^5
+// Returns false when the pair has to take the FP64 form, else adds it to acc.
+//   SL: q/r + d (d.q)/r^3,  DL: d (d.psi)(d.n)/r^5,  K_EQ: SL + s d/r^3 (an
+//   equivalent density's force and point source)
 // With d = 2^a D, R = |D|: the sums are 2^-a [q + D ((D.q) + 2^-a (D.psi)(D.n)
 // /R^2) /R^2] /R for both layers (q = 0 and the first dot left out for DL).
+constexpr int K_EQ = 4 | K_SL;
 template <int KIND>
-FX_HD bool fx_pair(const int64_t (&x)[3], int32_t xflag, int E, const SrcFx &S, double (&acc)[3]) {
+FX_HD bool fx_pair(const int64_t (&x)[3], uint32_t xthr, int E, const SrcFx &S, double (&acc)[3],
+                   double s0 = 0.0) {
   int64_t d[3];
   uint32_t any = 0u;
   for (int k = 0; k < 3; ++k) {
@@ -300,8 +314,7 @@ FX_HD bool fx_pair(const int64_t (&x)[3], int32_t xflag, int E, const SrcFx &S, 
     const int32_t hi = (int32_t)(d[k] >> 32);
     any |= (uint32_t)(hi ^ (hi >> 31));
   }
-  // |d| < 2^32 quanta, or an inexact coordinate and |d| < 2^54 quanta
-  if (any < ((xflag | S.flag) ? (1u << 22) : 1u)) return false;
+  if (any < xthr || any < S.thr) return false;
   const int s = fx_clz(any) - 1;  // left-justified: |D| in [2^62, 2^63)
   int32_t dh[3], dl[3];
   double D[3];
@@ -336,7 +349,9 @@ FX_HD bool fx_pair(const int64_t (&x)[3], int32_t xflag, int E, const SrcFx &S, 
       c = (dp * dn) * (ri2 * ri2);
     }
   } else {
-    c = fx_to_double(fx_dot(dh, dl, S.qh, S.ql), 1026 + S.eq) * ri2;
+    c = fx_to_double(fx_dot(dh, dl, S.qh, S.ql), 1026 + S.eq);
+    if (KIND == K_EQ) c = fx_fma(s0, fx_bits((uint32_t)(1023 - a) << 20, 0u), c);
+    c *= ri2;
   }
   if (KIND & K_SL) {
     for (int k = 0; k < 3; ++k) acc[k] = fx_fma(fx_fma(D[k], c, S.q[k]), ria, acc[k]);

@@ -1,13 +1,15 @@
 // fmm.cu -- the far field of the kernel-independent FMM on the GPU (Sec. 3.1,
-// "Far evaluation"): the passes of fmm_passes.cuh, one grid-stride launch per
-// pass and depth on the caller's stream, in FP64 or in the mixed form (FP32
-// evaluations and spectra, double-FP32 check-to-equivalent products), with M2L
-// dense or in Fourier space.  The near field is the U-list P2P sum
+// "Far evaluation") on the caller's stream, with M2L dense or in Fourier space:
+// the blocked FP64 form (fmm_fp64.cu), the blocked mixed form (fmm_fast.cu: FP32
+// evaluations and spectra, double-FP32 check-to-equivalent products), and for
+// mixed calls outside that form's limits the passes of fmm_passes.cuh, one
+// grid-stride launch per pass and depth.  The near field is the U-list P2P sum
 // (stokes_p2p_leaflists); the two together are the FMM.
 #include <cmath>
 
 #include "../../include/stokesgpu.h"
 #include "fmm_fast.cuh"
+#include "fmm_fp64.cuh"
 #include "prep.cuh"
 
 namespace stk {
@@ -28,9 +30,7 @@ __global__ void __launch_bounds__(256) k_fmm_pass(Pass P, int64_t n) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) F()(P, e);
 }
 
-__global__ void k_fmm_setup(Pass P) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) stk::fmm::fill_setup(P);
-}
+__global__ void k_fmm_setup(Pass P) { stk::fmm::fill_setup(P, threadIdx.x, blockDim.x); }
 
 struct DeviceExec {
   cudaStream_t st;
@@ -176,7 +176,12 @@ stk_status stokes_fmm_far_eval(const double *pts, const double *f, const double 
 
   if (cudaMemsetAsync(ws + L.counters, 0, sizeof(int32_t) * 4, st) != cudaSuccess)
     return report_error(STK_ECUDA, "cannot clear the error word");
-  k_fmm_setup<<<1, 32, 0, st>>>(P);
+  if (!mixed) {
+    const cudaError_t e = stk::fmm::far_field_fp64(P, tree->depth_ptr, tree->max_depth, sms, st);
+    if (e != cudaSuccess) return report_error(STK_ECUDA, cudaGetErrorString(e));
+    return STK_OK;
+  }
+  k_fmm_setup<<<1, 256, 0, st>>>(P);
   if (cudaGetLastError() != cudaSuccess) return report_error(STK_ECUDA, "set-up launch failed");
   stk::count_launches(1);
   // the CTA-blocked mixed kernels (their spectral products need the colleague table)
@@ -187,7 +192,7 @@ stk_status stokes_fmm_far_eval(const double *pts, const double *f, const double 
     return STK_OK;
   }
   DeviceExec ex{st, (int64_t)sms * 8};
-  stk::fmm::far_field(ex, P, tree->depth_ptr, tree->max_depth);
+  stk::fmm::far_field_mixed(ex, P, tree->depth_ptr, tree->max_depth);
   if (ex.err != cudaSuccess) return report_error(STK_ECUDA, cudaGetErrorString(ex.err));
   return STK_OK;
 }

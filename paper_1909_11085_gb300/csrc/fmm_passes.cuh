@@ -96,6 +96,15 @@ struct Tree {
   double root_size;
 };
 
+struct alignas(8) int2_t {
+  int32_t h, l;
+};
+constexpr int kTableMaxP = 6;  // orders whose M2L kernel table (33 MB at p = 6) is built
+constexpr int32_t kBadExp = 0x7fffffff;
+// Lattice displacements of a box pair, padded to whole 16-byte units per plane.
+FMM_HD int table_entries(int p) { return (2 * p - 1) * (2 * p - 1) * (2 * p - 1); }
+FMM_HD int table_pad(int p) { return (table_entries(p) + 1) & ~1; }
+
 // Everything one pass reads and writes.
 struct Pass {
   Tree t;
@@ -160,49 +169,21 @@ struct Pass {
                        // fmm_fast.cu)
   int32_t *vpar;       // [26][nbox] plist position of the neighbour in each direction of the
                        // parent at each plist position (-1 where it has no children)
+  // the blocked FP64 form (fmm_fp64.cu), dense M2L: kernel table and densities in
+  // fixed point
+  int2_t *ktab;        // [343][9][mpad] (high, low)
+  int32_t *kexp;       // [343] exponents
+  int2_t *edens;       // [nbox][ns][4]
+  int32_t *eexp;       // [nbox] exponents (kBadExp: not finite)
   // work items of the blocked L2T (fmm_fast.cu): per leaf the item count,
   // log2 of the points per item and the exclusive scan of the counts; the
   // items as (leaf, block | log2 << 24) pairs
   int32_t *icnt, *ipb, *ioff, *items;
 };
 
-// Boundary points of the p^3 grid on [-1, 1]^3, i slowest, k fastest.
-FMM_HD void fill_surface(int p, double *s) {
-  int m = 0;
-  for (int i = 0; i < p; ++i)
-    for (int j = 0; j < p; ++j)
-      for (int k = 0; k < p; ++k) {
-        if (!(i == 0 || j == 0 || k == 0 || i == p - 1 || j == p - 1 || k == p - 1)) continue;
-        s[3 * m + 0] = -1.0 + 2.0 * i / (p - 1);
-        s[3 * m + 1] = -1.0 + 2.0 * j / (p - 1);
-        s[3 * m + 2] = -1.0 + 2.0 * k / (p - 1);
-        ++m;
-      }
-}
-
 FMM_HD int surface_count(int p) { return p * p * p - (p - 2) * (p - 2) * (p - 2); }
 
 FMM_HD int freq_count(int p) { return 4 * p * p * (p + 1); }
-
-// Lattice indices of the surface points (the order of fill_surface) and the
-// twiddles of the G-point DFT.
-FMM_HD void fill_lattice(int p, int32_t *sidx, double *tw) {
-  int m = 0;
-  for (int i = 0; i < p; ++i)
-    for (int j = 0; j < p; ++j)
-      for (int k = 0; k < p; ++k) {
-        if (!(i == 0 || j == 0 || k == 0 || i == p - 1 || j == p - 1 || k == p - 1)) continue;
-        sidx[3 * m + 0] = i;
-        sidx[3 * m + 1] = j;
-        sidx[3 * m + 2] = k;
-        ++m;
-      }
-  const int G = 2 * p;
-  for (int t = 0; t < G; ++t) {
-    tw[2 * t + 0] = cos(2.0 * kPi * t / G);
-    tw[2 * t + 1] = sin(2.0 * kPi * t / G);
-  }
-}
 
 // Centre and half-width of box b (depth d).
 FMM_HD void box_geom(const Tree &t, int32_t b, int32_t d, double c[3], double &r) {
@@ -959,6 +940,7 @@ struct Layout {
   size_t child8, bflag, bpos, plist, ftab, fitab, vpar, uhh, uhl, btab;
   int64_t uslots;
   size_t icnt, ipb, ioff, items;
+  size_t ktab, kexp, edens, eexp;
   size_t total;
 };
 
@@ -1004,6 +986,7 @@ inline Layout layout(int64_t nbox, int p, int nc, bool fft, bool mixed, int64_t 
       none;
   L.uslots = spectrum_slots(depth_ptr, max_depth);
   L.icnt = L.ipb = L.ioff = L.items = none;
+  L.ktab = L.kexp = L.edens = L.eexp = none;
   if (!mixed) {
     L.chk = take(sizeof(double) * 3 * ns * B);
     L.up = take(sizeof(double) * nc * ns * B);
@@ -1013,6 +996,12 @@ inline Layout layout(int64_t nbox, int p, int nc, bool fft, bool mixed, int64_t 
       L.uhat = take(sizeof(double) * 2 * nf * nc * B);
       L.chat = take(sizeof(double) * 2 * nf * 3 * B);
       L.m2l = take(sizeof(double) * 3 * ns * B);
+    }
+    if (p <= kTableMaxP) {  // with spectra too: the two forms differ by the spectra alone
+      L.ktab = take(sizeof(int2_t) * 343 * 9 * (size_t)table_pad(p));
+      L.kexp = take(sizeof(int32_t) * 343);
+      L.edens = take(sizeof(int2_t) * 4 * ns * B);
+      L.eexp = take(sizeof(int32_t) * B);
     }
   } else {
     const size_t nops = (size_t)(op_entries(p, nc, max_depth, true) +
@@ -1071,7 +1060,12 @@ inline void bind(Pass &P, char *ws, const Layout &L, bool fft, bool mixed) {
   P.tw = mixed ? nullptr : d(L.tw);
   P.uhat = (fft && !mixed) ? d(L.uhat) : nullptr;
   P.chat = (fft && !mixed) ? d(L.chat) : nullptr;
+  const bool table = !fft && !mixed && P.p <= kTableMaxP;
   P.m2l = (fft && !mixed) ? d(L.m2l) : nullptr;
+  P.ktab = table ? reinterpret_cast<int2_t *>(ws + L.ktab) : nullptr;
+  P.kexp = table ? reinterpret_cast<int32_t *>(ws + L.kexp) : nullptr;
+  P.edens = table ? reinterpret_cast<int2_t *>(ws + L.edens) : nullptr;
+  P.eexp = table ? reinterpret_cast<int32_t *>(ws + L.eexp) : nullptr;
   P.ploc = mixed ? f(L.ploc) : nullptr;
   P.qf = (mixed && P.f) ? f(L.qf) : nullptr;
   P.pf = (mixed && P.phi) ? f(L.pf) : nullptr;
@@ -1103,17 +1097,32 @@ inline void bind(Pass &P, char *ws, const Layout &L, bool fft, bool mixed) {
   P.items = mixed ? i32(L.items) : nullptr;
 }
 
-// Surface points, lattice indices and twiddles (one thread; set-up of a call).
-FMM_HD void fill_setup(const Pass &P) {
-  fill_surface(P.p, P.surf);
-  double tw[2 * 2 * 12];  // G = 2p <= 24 twiddles
-  fill_lattice(P.p, P.sidx, tw);
-  for (int t = 0; t < 2 * 2 * P.p; ++t) {
-    if (P.tw) P.tw[t] = tw[t];
-    if (P.tw32) P.tw32[t] = (float)tw[t];
+// Surface points, lattice indices and twiddles (set-up of a call), by thread
+// `tid` of `nthreads`: point m is the m-th boundary point of the p^3 grid on
+// [-1, 1]^3 (i slowest, k fastest).  On
+// one thread its divisions and cosines in a row took 55-75 us of a call.
+FMM_HD void fill_setup(const Pass &P, int tid = 0, int nthreads = 1) {
+  const int p = P.p, G = 2 * p;
+  for (int m = tid; m < P.ns; m += nthreads) {
+    int seen = 0, at = -1;
+    for (int e = 0; e < p * p * p && at < 0; ++e) {
+      const int i = e / (p * p), j = (e / p) % p, k = e % p;
+      if (i == 0 || j == 0 || k == 0 || i == p - 1 || j == p - 1 || k == p - 1)
+        if (seen++ == m) at = e;
+    }
+    const int idx[3] = {at / (p * p), (at / p) % p, at % p};
+    for (int q = 0; q < 3; ++q) {
+      const double x = -1.0 + 2.0 * idx[q] / (p - 1);
+      P.surf[3 * m + q] = x;
+      P.sidx[3 * m + q] = idx[q];
+      if (P.surf32) P.surf32[3 * m + q] = (float)x;
+    }
   }
-  if (P.surf32)
-    for (int q = 0; q < 3 * P.ns; ++q) P.surf32[q] = (float)P.surf[q];
+  for (int t = tid; t < 2 * G; t += nthreads) {
+    const double a = 2.0 * kPi * (t / 2) / G, v = (t & 1) ? sin(a) : cos(a);
+    if (P.tw) P.tw[t] = v;
+    if (P.tw32) P.tw32[t] = (float)v;
+  }
 }
 
 // The spectral products of one depth: blocked by parent when the colleague
@@ -1129,60 +1138,73 @@ void m2l_products(Exec &ex, Pass P, const int32_t *depth_ptr, int64_t per_box_co
   }
 }
 
-// The pass sequence; Exec::run<F>(P, count) calls F on every output of a pass
+// The pass sequences; Exec::run<F>(P, count) calls F on every output of a pass
 // (a kernel launch on the GPU).  depth_ptr is the host copy of the depth
-// ranges of the boxes.
+// ranges of the boxes.  The FP64 one is the reference the blocked FP64 kernels
+// (fmm_fp64.cu) are checked against on the host.
 template <class Exec>
-void far_field(Exec &ex, Pass P, const int32_t *depth_ptr, int32_t max_depth) {
+void far_field_mixed(Exec &ex, Pass P, const int32_t *depth_ptr, int32_t max_depth) {
   const int64_t ns = P.ns;
-  const bool mixed = P.mixed != 0;
-  if (mixed) {
-    ex.template run<PACK>(P, P.n);
-    ex.template run<OPSPLIT>(P, P.n_uc2e + P.n_dc2e);
-    if (P.spec) ex.template run<SPEC32>(P, (int64_t)343 * freq_count(P.p) * 3 * P.nc * 2);
-    ex.template run<S2MF>(P, (int64_t)P.t.nleaf * ns);
-  } else {
-    ex.template run<S2M>(P, (int64_t)P.t.nleaf * ns);
-  }
-  for (int32_t d = max_depth; d >= kFirstDepth; --d) {
+  auto at_depth = [&](int32_t d) {
     P.depth = d;
     P.box0 = depth_ptr[d];
     P.box1 = depth_ptr[d + 1];
-    const int64_t nb = P.box1 - P.box0;
-    if (mixed) {
-      if (d < max_depth) ex.template run<M2MF>(P, nb * ns);
-      ex.template run<UC2EF>(P, nb * P.nc * ns);
-    } else {
-      if (d < max_depth) ex.template run<M2M>(P, nb * ns);
-      ex.template run<UC2E>(P, nb * P.nc * ns);
-    }
+    return (int64_t)(P.box1 - P.box0);
+  };
+  ex.template run<PACK>(P, P.n);
+  ex.template run<OPSPLIT>(P, P.n_uc2e + P.n_dc2e);
+  if (P.spec) ex.template run<SPEC32>(P, (int64_t)343 * freq_count(P.p) * 3 * P.nc * 2);
+  ex.template run<S2MF>(P, (int64_t)P.t.nleaf * ns);
+  for (int32_t d = max_depth; d >= kFirstDepth; --d) {
+    const int64_t nb = at_depth(d);
+    if (d < max_depth) ex.template run<M2MF>(P, nb * ns);
+    ex.template run<UC2EF>(P, nb * P.nc * ns);
   }
   for (int32_t d = kFirstDepth; d <= max_depth; ++d) {
+    const int64_t nb = at_depth(d), nf = freq_count(P.p);
+    if (P.spec) {
+      ex.template run<UFFTT<float>>(P, nb * nf * P.nc);
+      m2l_products<Exec, float>(ex, P, depth_ptr, nb * nf);
+      ex.template run<IFFTT<float>>(P, nb * ns);
+    }
+    ex.template run<DCHKF>(P, nb * ns);
+    ex.template run<DC2EF>(P, nb * 3 * ns);
+  }
+  ex.template run<L2TF>(P, P.n);
+}
+
+template <class Exec>
+void far_field_fp64_passes(Exec &ex, Pass P, const int32_t *depth_ptr, int32_t max_depth) {
+  const int64_t ns = P.ns;
+  auto at_depth = [&](int32_t d) {
     P.depth = d;
     P.box0 = depth_ptr[d];
     P.box1 = depth_ptr[d + 1];
-    const int64_t nb = P.box1 - P.box0;
-    const int64_t nf = freq_count(P.p);
-    if (mixed) {
-      if (P.spec) {
-        ex.template run<UFFTT<float>>(P, nb * nf * P.nc);
-        m2l_products<Exec, float>(ex, P, depth_ptr, nb * nf);
-        ex.template run<IFFTT<float>>(P, nb * ns);
-      }
-      ex.template run<DCHKF>(P, nb * ns);
-      ex.template run<DC2EF>(P, nb * 3 * ns);
-    } else {
-      if (P.spec) {
-        ex.template run<UFFT>(P, nb * nf * P.nc);
-        m2l_products<Exec, double>(ex, P, depth_ptr, nb * nf);
-        ex.template run<IFFT>(P, nb * ns);
-      }
-      ex.template run<DCHK>(P, nb * ns);
-      ex.template run<DC2E>(P, nb * 3 * ns);
-    }
+    return (int64_t)(P.box1 - P.box0);
+  };
+  ex.template run<S2M>(P, (int64_t)P.t.nleaf * ns);
+  for (int32_t d = max_depth; d >= kFirstDepth; --d) {
+    const int64_t nb = at_depth(d);
+    if (d < max_depth) ex.template run<M2M>(P, nb * ns);
+    ex.template run<UC2E>(P, nb * P.nc * ns);
   }
-  if (mixed) ex.template run<L2TF>(P, P.n);
-  else ex.template run<L2T>(P, P.n);
+  for (int32_t d = kFirstDepth; d <= max_depth; ++d) {
+    const int64_t nb = at_depth(d), nf = freq_count(P.p);
+    if (P.spec) {
+      ex.template run<UFFT>(P, nb * nf * P.nc);
+      m2l_products<Exec, double>(ex, P, depth_ptr, nb * nf);
+      ex.template run<IFFT>(P, nb * ns);
+    }
+    ex.template run<DCHK>(P, nb * ns);
+    ex.template run<DC2E>(P, nb * 3 * ns);
+  }
+  ex.template run<L2T>(P, P.n);
+}
+
+template <class Exec>
+void far_field(Exec &ex, Pass P, const int32_t *depth_ptr, int32_t max_depth) {
+  if (P.mixed) far_field_mixed(ex, P, depth_ptr, max_depth);
+  else far_field_fp64_passes(ex, P, depth_ptr, max_depth);
 }
 
 }  // namespace fmm

@@ -73,12 +73,12 @@ static void run(int count, double size, double shift, double sep, int planar, do
     }
     g_est = (float)(2.4e-7 * U(g));
     SrcFx S;
-    S.flag = 0;
-    int32_t xf = 0;
+    S.thr = kFxExact;
+    uint32_t xf = kFxExact;
     int64_t X[3];
     for (int k = 0; k < 3; ++k) {
       X[k] = fx_coord(x[k], E, xf);
-      S.y[k] = fx_coord(y[k], E, S.flag);
+      S.y[k] = fx_coord(y[k], E, S.thr);
       S.q[k] = q[k];
     }
     S.eq = (int16_t)fx_block(q, S.qh, S.ql);
@@ -153,11 +153,11 @@ extern "C" int fixed_coord_check(int count, int E, double *worst) {
   for (int i = 0; i < count; ++i) {
     const double v = i == 0 ? 0.0 : i == 1 ? 5e-324 : i == 2 ? -std::ldexp(1 - 1e-16, E)
                                                    : std::ldexp(U(g), E - (int)(g() % 80));
-    int32_t f = 0;
+    uint32_t f = kFxExact;
     const int64_t X = fx_coord(v, E, f);
     const Q e = fabsl((Q)X - (Q)v * ldexpl(1, 62 - E));
     *worst = std::fmax(*worst, (double)e);
-    if (e != 0 && !f) ++lies;
+    if (e != 0 && f == kFxExact) ++lies;
   }
   return lies;
 }
