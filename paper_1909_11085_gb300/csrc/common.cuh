@@ -89,6 +89,9 @@ struct EngineParams {
   int32_t *cand_list;        // MIXED: per item, up to cand_cap candidate sources (index | kind << 30)
   int32_t *cand_cnt;         // MIXED: per item, candidates listed (-1: more than cand_cap)
   int32_t cand_cap;
+  int32_t *over_list;        // MIXED: the items whose list overflowed (any order),
+  int32_t *over_cnt;         //   their count and k_near's queue head over them (both
+  int32_t *over_head;        //   zeroed before the engine's launch)
   int32_t *err_flag;         // device error word
   int64_t spin_limit;        // bounded mbarrier waits, in SM clock cycles
   int64_t drain_limit;       // bound of the wait for a warp's own copy after an expiry

@@ -595,7 +595,10 @@ __device__ bool run_item(const EngineParams &P, const Item &it, int id, WarpSmem
     s_cur = s_next;
   }
   if (!ok) return false;
-  if (lane == 0) P.cand_cnt[id] = ccount <= P.cand_cap ? ccount : -1;
+  if (lane == 0) {
+    P.cand_cnt[id] = ccount <= P.cand_cap ? ccount : -1;
+    if (ccount > P.cand_cap) P.over_list[atomicAdd(P.over_cnt, 1)] = id;
+  }
   float hi[T][3], lo[T][3];
 #pragma unroll
   for (int t = 0; t < T; ++t)

@@ -123,16 +123,17 @@ struct Plan {
   // offsets (the counters always sit at offset 0 of the aligned workspace)
   size_t counters, rec, recfx = 0, keys_a, keys_b, vals_a, vals_b, ikeys_a, ikeys_b, ivals_a, ivals_b, hist,
       hist_scan, bbox_part, bbox, items, range, cnt, offs, part, frames = 0, xloc = 0,
-      cand_list = 0, cand_cnt = 0, total;
+      cand_list = 0, cand_cnt = 0, over = 0, total;
 };
 
 // Candidate sources the engine lists per item for k_near (items with more are
 // rescanned by k_near).
 constexpr int32_t kCandCap = 512;
 // Counters at the head of the workspace: items, engine queue, error word, near
-// queue, then the FP64 form's FxState.
+// queue, then the FP64 form's FxState or the mixed form's overflowed items and
+// their queue.
 constexpr int kCounters = 8;
-constexpr int kFxCounter = 4;
+constexpr int kFxCounter = 4, kOverCounter = 4;
 
 // The FP64 form's items are an eighth of the mixed form's: a pair costs some
 // 700 cycles of a warp there against some 25, an item's set-up and loads are
@@ -192,6 +193,7 @@ void layout(Plan &p) {
     p.xloc = a.take(sizeof(float) * 3 * (size_t)(p.nt > 0 ? p.nt : 1));
     p.cand_list = a.take(sizeof(int32_t) * (size_t)kCandCap * mi);
     p.cand_cnt = a.take(sizeof(int32_t) * mi);
+    p.over = a.take(sizeof(int32_t) * mi);
   }
   p.total = a.off + 256;  // slack for re-alignment of an unaligned base
 }
@@ -382,6 +384,9 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
     P.cand_list = at<int32_t>(ws, p.cand_list);
     P.cand_cnt = at<int32_t>(ws, p.cand_cnt);
     P.cand_cap = kCandCap;
+    P.over_list = at<int32_t>(ws, p.over);
+    P.over_cnt = counters + kOverCounter;
+    P.over_head = counters + kOverCounter + 1;
     CU(launch_engine_mixed(P, (int)grid, st));
   } else {
     P.rec64 = at<SrcRec64>(ws, p.rec);
