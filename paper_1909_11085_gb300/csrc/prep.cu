@@ -89,15 +89,31 @@ __global__ void k_bbox_partial(int64_t n, const double *__restrict__ pts, double
     for (int k = 0; k < 6; ++k) part[6 * blockIdx.x + k] = sm[k][0];
 }
 
-__global__ void k_bbox_final(int nblk, const double *__restrict__ part, double *__restrict__ box) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// One block over the partial boxes (one thread took 60 to 420 us for up to 1,024).
+__global__ void __launch_bounds__(kRedThreads) k_bbox_final(int nblk, const double *__restrict__ part,
+                                                            double *__restrict__ box) {
+  __shared__ double sm[6][kRedThreads / kWarp];
   double b[6] = {DBL_MAX, DBL_MAX, DBL_MAX, -DBL_MAX, -DBL_MAX, -DBL_MAX};
-  for (int i = 0; i < nblk; ++i)
-    for (int k = 0; k < 3; ++k) {
-      b[k] = fmin(b[k], part[6 * i + k]);
-      b[3 + k] = fmax(b[3 + k], part[6 * i + 3 + k]);
+  for (int i = threadIdx.x; i < nblk; i += kRedThreads)
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      b[k] = k < 3 ? fmin(b[k], part[6 * i + k]) : fmax(b[k], part[6 * i + k]);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double v = __shfl_xor_sync(kFull, b[k], o);
+      b[k] = k < 3 ? fmin(b[k], v) : fmax(b[k], v);
     }
-  for (int k = 0; k < 6; ++k) box[k] = b[k];
+    if (threadIdx.x % kWarp == 0) sm[k][threadIdx.x / kWarp] = b[k];
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    const int k = threadIdx.x;
+    double v = sm[k][0];
+    for (int w = 1; w < kRedThreads / kWarp; ++w) v = k < 3 ? fmin(v, sm[k][w]) : fmax(v, sm[k][w]);
+    box[k] = v;
+  }
 }
 
 // ---------------------------------------------------------------- Morton keys
@@ -221,15 +237,63 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t *__r
   hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// Stable scatter: keys of equal digit keep their order.
+// Exclusive scan of each digit's row of block counts (a block per digit); the
+// row's total goes to its first count.  One block scanning all rows took 9 us
+// for 35 thousand keys and 75 us for 1.3 million.
+__global__ void __launch_bounds__(kSortThreads) k_radix_rows(int nblk, int32_t *__restrict__ hist,
+                                                             int32_t *__restrict__ rows) {
+  __shared__ int32_t wsum[kSortThreads / kWarp];
+  int32_t *in = hist + (int64_t)blockIdx.x * nblk, *out = rows + (int64_t)blockIdx.x * nblk;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int32_t carry = 0;
+  for (int base = 0; base < nblk; base += kSortThreads) {
+    const int i = base + threadIdx.x;
+    const int32_t v = i < nblk ? in[i] : 0;
+    int32_t t = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(kFull, t, o);
+      if (lane >= o) t += y;
+    }
+    if (lane == 31) wsum[wid] = t;
+    __syncthreads();
+    int32_t before = carry, all = 0;
+#pragma unroll
+    for (int w = 0; w < kSortThreads / kWarp; ++w) {
+      before += w < wid ? wsum[w] : 0;
+      all += wsum[w];
+    }
+    if (i < nblk) out[i] = before + t - v;
+    carry += all;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) in[0] = carry;
+}
+
+// Stable scatter: keys of equal digit keep their order.  rows: this block's
+// offset within each digit; hist: the digits' totals, scanned here.
 __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     const uint64_t *__restrict__ kin, const int32_t *__restrict__ vin, int64_t n, int shift,
-    int nblk, const int32_t *__restrict__ offs, uint64_t *__restrict__ kout,
-    int32_t *__restrict__ vout) {
+    int nblk, const int32_t *__restrict__ hist, const int32_t *__restrict__ rows,
+    uint64_t *__restrict__ kout, int32_t *__restrict__ vout) {
   __shared__ int32_t running[256];
   __shared__ int32_t cnt[kSortThreads / kWarp][256];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  running[threadIdx.x] = offs[(int64_t)threadIdx.x * nblk + blockIdx.x];
+  {
+    const int32_t v = hist[(int64_t)threadIdx.x * nblk];
+    int32_t t = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(kFull, t, o);
+      if (lane >= o) t += y;
+    }
+    if (lane == 31) cnt[0][wid] = t;
+    __syncthreads();
+    int32_t before = 0;
+    for (int w = 0; w < wid; ++w) before += cnt[0][w];
+    running[threadIdx.x] = before + t - v + rows[(int64_t)threadIdx.x * nblk + blockIdx.x];
+    __syncthreads();
+  }
   const int64_t base = (int64_t)blockIdx.x * kSortTile;
   const unsigned lt = (1u << lane) - 1u;
   for (int r = 0; r < kSortRounds; ++r) {
@@ -265,6 +329,30 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
   }
 }
 
+// Stable sort of a few keys in one launch: a key's place is the number of keys
+// before it, counted by its thread.
+constexpr int kRankTile = 1024;
+__global__ void __launch_bounds__(kSortThreads) k_rank_sort(const uint64_t *__restrict__ kin,
+                                                            const int32_t *__restrict__ vin, int n,
+                                                            uint64_t *__restrict__ kout,
+                                                            int32_t *__restrict__ vout) {
+  __shared__ uint64_t s[kRankTile];
+  const int i = blockIdx.x * kSortThreads + threadIdx.x;
+  const uint64_t key = i < n ? kin[i] : 0;
+  int rank = 0;
+  for (int base = 0; base < n; base += kRankTile) {
+    const int m = min(kRankTile, n - base);
+    __syncthreads();
+    for (int t = threadIdx.x; t < m; t += kSortThreads) s[t] = kin[base + t];
+    __syncthreads();
+    for (int t = 0; t < m; ++t) rank += s[t] < key || (s[t] == key && base + t < i);
+  }
+  if (i < n) {
+    kout[rank] = key;
+    vout[rank] = vin[i];
+  }
+}
+
 size_t radix_hist_entries(int64_t n) {
   const int64_t nblk = (n + kSortTile - 1) / kSortTile;
   return (size_t)(256 * (nblk > 0 ? nblk : 1));
@@ -275,6 +363,15 @@ size_t radix_hist_entries(int64_t n) {
 int radix_sort(uint64_t *ka, int32_t *va, uint64_t *kb, int32_t *vb, int64_t n, int bits,
                int32_t *hist, int32_t *hist_scan, cudaStream_t st) {
   if (n <= 1) return 0;
+  // up to 8,192 keys: as many compares a thread (some 25 us at the most) against
+  // three launches per 8 bits (24 launches and 190 us for a near-zone search's
+  // 2,560 keys of 64 bits, 12 and some 60 us for 4,352 Morton keys)
+  if (n <= 8192) {
+    k_rank_sort<<<(int)((n + kSortThreads - 1) / kSortThreads), kSortThreads, 0, st>>>(
+        ka, va, (int)n, kb, vb);
+    count_launches(1);
+    return 1;
+  }
   const int nblk = (int)((n + kSortTile - 1) / kSortTile);
   int cur = 0;
   for (int shift = 0; shift < bits; shift += 8) {
@@ -282,9 +379,9 @@ int radix_sort(uint64_t *ka, int32_t *va, uint64_t *kb, int32_t *vb, int64_t n, 
     int32_t *vi = cur ? vb : va, *vo = cur ? va : vb;
     k_radix_hist<<<nblk, kSortThreads, 0, st>>>(ki, n, shift, nblk, hist);
     count_launches(1);
-    k_scan_excl<<<1, kScanThreads, 0, st>>>(hist, (int64_t)256 * nblk, hist_scan, nullptr);
+    k_radix_rows<<<256, kSortThreads, 0, st>>>(nblk, hist, hist_scan);
     count_launches(1);
-    k_radix_scatter<<<nblk, kSortThreads, 0, st>>>(ki, vi, n, shift, nblk, hist_scan, ko, vo);
+    k_radix_scatter<<<nblk, kSortThreads, 0, st>>>(ki, vi, n, shift, nblk, hist, hist_scan, ko, vo);
     count_launches(1);
     cur ^= 1;
   }
@@ -499,7 +596,7 @@ void launch_bbox(int64_t n, const double *pts, double *partial, double *box, cud
   const int nb = bbox_partial_blocks(n);
   k_bbox_partial<<<nb, kRedThreads, 0, st>>>(n, pts, partial);
   count_launches(1);
-  k_bbox_final<<<1, 32, 0, st>>>(nb, partial, box);
+  k_bbox_final<<<1, kRedThreads, 0, st>>>(nb, partial, box);
   count_launches(1);
 }
 
