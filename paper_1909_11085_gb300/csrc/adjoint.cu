@@ -95,128 +95,250 @@ struct NAcc {
 };
 
 // ---------------------------------------------------------------- FP32 pass
-template <bool SRC>
-__global__ void __launch_bounds__(kAdjThreads) k_adj_mixed(AdjParams A) {
+// Two output points per thread, one in each half of the packed FP32
+// instructions (an input's values are duplicated into both halves), 128 output
+// points per CTA of 64 threads.  One output per thread issued 81% of its slots
+// at 63% of the FMA pipe; packed, the pipe is the bound (81 of its operations
+// per source-major pair, 65 per target-major one).  Per half the operations,
+// their order and their rounding are those the scalar form compiled to (which
+// product of a sum is fused differs between the passes: FIRST), so the sums are
+// what one output per thread gave, bit for bit.
+// 34,816 points on themselves: source-major 4.01 -> 3.03 ms, target-major
+// 3.46 -> 2.55 ms (FMA pipe 83% and 81% of its cycles).
+constexpr int kAdjPack = kAdjThreads / 2;  // threads of a packed CTA
+
+__device__ __forceinline__ float2 a2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 m2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+// a b + c d, the first or the second product fused into the sum
+template <bool FIRST>
+__device__ __forceinline__ float2 sum2(float2 a, float2 b, float2 c, float2 d) {
+  return FIRST ? f2(a, b, m2(c, d)) : f2(c, d, m2(a, b));
+}
+template <bool FIRST>
+__device__ __forceinline__ float2 dot2(const float2 (&a)[3], const float2 (&b)[3]) {
+  return f2(a[2], b[2], sum2<FIRST>(a[0], b[0], a[1], b[1]));
+}
+
+template <bool SRC, int KIND>
+__device__ __forceinline__ void adj_pair2(const float2 (&d)[3], float2 ri, const float2 (&g)[3],
+                                          const float2 (&q)[3], const float2 (&p)[3],
+                                          const float2 (&n)[3], float2 *acc) {
+  const float2 ri2 = m2(ri, ri), ri3 = m2(ri, ri2), ri5 = m2(ri3, ri2);
+  const float2 dg = dot2<true>(d, g);
+  float2 gx[3] = {both(0.f), both(0.f), both(0.f)};
+  if (KIND & K_SL) {
+    const float2 dq = dot2<SRC>(d, q), gq = dot2<SRC>(g, q);
+    const float2 a = m2(dq, ri3), b = m2(dg, ri3);
+    if (SRC)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) acc[k] = a2(acc[k], f2(g[k], ri, m2(d[k], b)));
+    const float2 t = m2(m2(both(3.f), dg), dq);
+    const float2 cd = f2(neg2(t), ri5, m2(neg2(gq), ri3));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gx[k] = f2(d[k], cd, sum2<SRC>(g[k], a, q[k], b));
+  }
+  if (KIND & K_DL) {
+    const float2 dp = dot2<true>(d, p), dn = dot2<true>(d, n);
+    const float2 a = m2(m2(dg, dn), ri5), b = m2(m2(dg, dp), ri5);
+    if (SRC)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        acc[3 + k] = f2(d[k], a, acc[3 + k]);
+        acc[6 + k] = f2(d[k], b, acc[6 + k]);
+      }
+    const float2 e = m2(m2(dp, dn), ri5), t5 = m2(m2(m2(both(5.f), b), dn), ri2), mt5 = neg2(t5);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float2 w = f2(d[k], mt5, f2(n[k], b, sum2<SRC>(g[k], e, p[k], a)));
+      gx[k] = a2(gx[k], w);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    if (SRC) acc[9 + k] = a2(acc[9 + k], neg2(gx[k]));
+    else acc[k] = a2(acc[k], gx[k]);
+}
+
+template <bool SRC, int KIND>
+__global__ void __launch_bounds__(kAdjPack, SRC ? 8 : 12) k_adj_mixed(AdjParams A) {
   constexpr int NA = NAcc<SRC>::value;
   __shared__ float4 sP[kAdjThreads];   // local position, hh
   __shared__ float4 sG[kAdjThreads];   // g (src-major) or q (trg-major)
-  __shared__ float4 sN[kAdjThreads];   // n (trg-major)
-  __shared__ float4 sPs[kAdjThreads];  // psi (trg-major)
+  __shared__ float4 sN[SRC ? 1 : kAdjThreads];   // n (trg-major)
+  __shared__ float4 sPs[SRC ? 1 : kAdjThreads];  // psi (trg-major)
   __shared__ int32_t sI[kAdjThreads];  // caller index
-  __shared__ float red[6][kAdjThreads];
+  __shared__ float sums[2 * NA][kAdjThreads];  // compensated sums (hi, lo)
+  __shared__ float red[6][kAdjPack / kWarp];
   const SrcRec *orec = reinterpret_cast<const SrcRec *>(A.out_rec);
   const SrcRec *irec = reinterpret_cast<const SrcRec *>(A.in_rec);
   const int tid = threadIdx.x;
-  const int64_t o_sorted = (int64_t)blockIdx.x * kAdjThreads + tid;
-  const bool valid = o_sorted < A.nout;
-  const int64_t oc = valid ? A.operm[o_sorted] : A.operm[(int64_t)blockIdx.x * kAdjThreads];
+  const int64_t o0 = (int64_t)blockIdx.x * kAdjThreads;
+  bool valid[2];
+  int64_t oc[2];
+  SrcRec Ro[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    valid[h] = o0 + tid + h * kAdjPack < A.nout;
+    oc[h] = A.operm[valid[h] ? o0 + tid + h * kAdjPack : o0];
+    Ro[h] = orec[oc[h]];
+  }
 
   // CTA origin: centre of the output points' bounding box, as hi/lo splits
-  const SrcRec Ro = orec[oc];
-  const SrcRec R0 = orec[A.operm[(int64_t)blockIdx.x * kAdjThreads]];
-  {
-    const float r[3] = {(Ro.yh.x - R0.yh.x) + (Ro.q.w - R0.q.w),
-                        (Ro.yh.y - R0.yh.y) + (Ro.n.w - R0.n.w),
-                        (Ro.yh.z - R0.yh.z) + (Ro.p.w - R0.p.w)};
-    for (int k = 0; k < 3; ++k) {
-      red[k][tid] = valid ? r[k] : INFINITY;
-      red[3 + k][tid] = valid ? r[k] : -INFINITY;
-    }
-  }
-  __syncthreads();
-  for (int s = kAdjThreads / 2; s > 0; s >>= 1) {
-    if (tid < s)
-      for (int k = 0; k < 3; ++k) {
-        red[k][tid] = fminf(red[k][tid], red[k][tid + s]);
-        red[3 + k][tid] = fmaxf(red[3 + k][tid], red[3 + k][tid + s]);
-      }
-    __syncthreads();
-  }
+  const SrcRec R0 = orec[A.operm[o0]];
   float oh[3], ol[3];
   {
-    const double o[3] = {(double)R0.yh.x + (double)R0.q.w + 0.5 * ((double)red[0][0] + red[3][0]),
-                         (double)R0.yh.y + (double)R0.n.w + 0.5 * ((double)red[1][0] + red[4][0]),
-                         (double)R0.yh.z + (double)R0.p.w + 0.5 * ((double)red[2][0] + red[5][0])};
-    for (int k = 0; k < 3; ++k) split_hl(o[k], oh[k], ol[k]);
-  }
-  __syncthreads();
-  const float ox = to_local(Ro.yh.x, Ro.q.w, oh[0], ol[0]);
-  const float oy = to_local(Ro.yh.y, Ro.n.w, oh[1], ol[1]);
-  const float oz = to_local(Ro.yh.z, Ro.p.w, oh[2], ol[2]);
-  const float own_hh = Ro.yh.w;
-  if (valid && blockIdx.y == 0) {  // the frame, for a rescan of an overflowing list
-    float *fr = A.oframe + 9 * (size_t)oc;
-    fr[0] = ox; fr[1] = oy; fr[2] = oz;
-    fr[3] = oh[0]; fr[4] = oh[1]; fr[5] = oh[2];
-    fr[6] = ol[0]; fr[7] = ol[1]; fr[8] = ol[2];
-  }
-  const float ov1[3] = {Ro.q.x, Ro.q.y, Ro.q.z};  // g (trg-major) or q (src-major)
-  const float on[3] = {Ro.n.x, Ro.n.y, Ro.n.z};
-  const float op[3] = {Ro.p.x, Ro.p.y, Ro.p.z};
-
-  float hi[NA], lo[NA], ps[NA];
+    float mn[3], mx[3];  // (an invalid half repeats the first point)
 #pragma unroll
-  for (int a = 0; a < NA; ++a) hi[a] = lo[a] = ps[a] = 0.f;
+    for (int k = 0; k < 3; ++k) mn[k] = INFINITY, mx[k] = -INFINITY;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float r[3] = {(Ro[h].yh.x - R0.yh.x) + (Ro[h].q.w - R0.q.w),
+                          (Ro[h].yh.y - R0.yh.y) + (Ro[h].n.w - R0.n.w),
+                          (Ro[h].yh.z - R0.yh.z) + (Ro[h].p.w - R0.p.w)};
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        mn[k] = fminf(mn[k], r[k]);
+        mx[k] = fmaxf(mx[k], r[k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        mn[k] = fminf(mn[k], __shfl_xor_sync(kFull, mn[k], o));
+        mx[k] = fmaxf(mx[k], __shfl_xor_sync(kFull, mx[k], o));
+      }
+      if (tid % kWarp == 0) {
+        red[k][tid / kWarp] = mn[k];
+        red[3 + k][tid / kWarp] = mx[k];
+      }
+    }
+    __syncthreads();
+    const float first[3] = {R0.yh.x, R0.yh.y, R0.yh.z}, low[3] = {R0.q.w, R0.n.w, R0.p.w};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float lo = fminf(red[k][0], red[k][1]), hi = fmaxf(red[3 + k][0], red[3 + k][1]);
+      split_hl((double)first[k] + (double)low[k] + 0.5 * ((double)lo + hi), oh[k], ol[k]);
+    }
+  }
+  float2 own[3], v1[3], on[3], op[3];  // position; g (trg-major) or q; n; psi
+  float2 own_hh;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float o[3] = {to_local(Ro[h].yh.x, Ro[h].q.w, oh[0], ol[0]),
+                        to_local(Ro[h].yh.y, Ro[h].n.w, oh[1], ol[1]),
+                        to_local(Ro[h].yh.z, Ro[h].p.w, oh[2], ol[2])};
+    if (valid[h] && blockIdx.y == 0) {  // the frame, for a rescan of an overflowing list
+      float *fr = A.oframe + 9 * (size_t)oc[h];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        fr[k] = o[k];
+        fr[3 + k] = oh[k];
+        fr[6 + k] = ol[k];
+      }
+    }
+    const float q[3] = {Ro[h].q.x, Ro[h].q.y, Ro[h].q.z}, n[3] = {Ro[h].n.x, Ro[h].n.y, Ro[h].n.z},
+                p[3] = {Ro[h].p.x, Ro[h].p.y, Ro[h].p.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      (h ? own[k].y : own[k].x) = o[k];
+      (h ? v1[k].y : v1[k].x) = q[k];
+      (h ? on[k].y : on[k].x) = n[k];
+      (h ? op[k].y : op[k].x) = p[k];
+    }
+    (h ? own_hh.y : own_hh.x) = Ro[h].yh.w;
+  }
 
-  const int64_t i0 = A.nin * blockIdx.y / A.nsplit, i1 = A.nin * (blockIdx.y + 1) / A.nsplit;
+  float2 ps[NA];
+#pragma unroll
+  for (int a = 0; a < NA; ++a) {
+    ps[a] = both(0.f);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      sums[a][tid + h * kAdjPack] = sums[NA + a][tid + h * kAdjPack] = 0.f;
+  }
+
+  // the tiles of split y / nsub, its part y % nsub
+  const int64_t split = blockIdx.y / A.nsub, sub = blockIdx.y % A.nsub;
+  const int64_t s0 = A.nin * split / A.nsplit, s1 = A.nin * (split + 1) / A.nsplit;
+  const int64_t tiles = (s1 - s0 + kAdjThreads - 1) / kAdjThreads;
+  const int64_t i0 = s0 + kAdjThreads * (tiles * sub / A.nsub);
+  const int64_t i1 = min(s1, s0 + kAdjThreads * (tiles * (sub + 1) / A.nsub));
   for (int64_t tb = i0; tb < i1; tb += kAdjThreads) {
-    const int64_t k = tb + tid;
-    if (k < i1) {
-      const int32_t ic = A.iperm[k];
-      const SrcRec R = irec[ic];
-      sP[tid] = make_float4(to_local(R.yh.x, R.q.w, oh[0], ol[0]),
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int s = tid + h * kAdjPack;
+      if (tb + s < i1) {
+        const int32_t ic = A.iperm[tb + s];
+        const SrcRec R = irec[ic];
+        sP[s] = make_float4(to_local(R.yh.x, R.q.w, oh[0], ol[0]),
                             to_local(R.yh.y, R.n.w, oh[1], ol[1]),
                             to_local(R.yh.z, R.p.w, oh[2], ol[2]), R.yh.w);
-      sG[tid] = make_float4(R.q.x, R.q.y, R.q.z, 0.f);
-      sN[tid] = make_float4(R.n.x, R.n.y, R.n.z, 0.f);
-      sPs[tid] = make_float4(R.p.x, R.p.y, R.p.z, 0.f);
-      sI[tid] = ic;
+        sG[s] = make_float4(R.q.x, R.q.y, R.q.z, 0.f);
+        if (!SRC) {
+          sN[s] = make_float4(R.n.x, R.n.y, R.n.z, 0.f);
+          sPs[s] = make_float4(R.p.x, R.p.y, R.p.z, 0.f);
+        }
+        sI[s] = ic;
+      }
     }
     __syncthreads();
     const int m = (int)min((int64_t)kAdjThreads, i1 - tb);
-    if (valid) {
-      for (int kk = 0; kk < m; ++kk) {
-        const float4 P = sP[kk];
-        // d = x - y: source-major: x = input, y = own; target-major: x = own, y = input
-        const float dx = SRC ? P.x - ox : ox - P.x, dy = SRC ? P.y - oy : oy - P.y,
-                    dz = SRC ? P.z - oz : oz - P.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float hh = SRC ? own_hh : P.w;
-        const bool near = r2 < hh;
-        const float ri = near ? 0.f : rsqrt_ftz(r2);
-        const float4 G = sG[kk];
-        float g[3], q[3], pp[3], nn[3];
-        if (SRC) {
-          g[0] = G.x; g[1] = G.y; g[2] = G.z;
-          q[0] = ov1[0]; q[1] = ov1[1]; q[2] = ov1[2];
-          pp[0] = op[0]; pp[1] = op[1]; pp[2] = op[2];
-          nn[0] = on[0]; nn[1] = on[1]; nn[2] = on[2];
-        } else {
-          const float4 N = sN[kk], Ps = sPs[kk];
-          g[0] = ov1[0]; g[1] = ov1[1]; g[2] = ov1[2];
-          q[0] = G.x; q[1] = G.y; q[2] = G.z;
-          pp[0] = Ps.x; pp[1] = Ps.y; pp[2] = Ps.z;
-          nn[0] = N.x; nn[1] = N.y; nn[2] = N.z;
-        }
-        adj_pair<float, SRC>(dx, dy, dz, ri, g, q, pp, nn, A.has_sl, A.has_dl, ps);
-        if (near) {  // listed for the FP64 pass
-          const int slot = atomicAdd(A.near_cnt + oc, 1);
-          if (slot < A.near_cap) A.near_idx[(size_t)oc * A.near_cap + slot] = sI[kk];
-        }
-      }
+    for (int kk = 0; kk < m; ++kk) {
+      const float4 P = sP[kk], G = sG[kk];
+      const float2 in[3] = {both(P.x), both(P.y), both(P.z)};
+      const float2 gi[3] = {both(G.x), both(G.y), both(G.z)};
+      float2 d[3];  // x - y: the target is the input (src-major) or the own point
 #pragma unroll
-      for (int a = 0; a < NA; ++a) {
-        two_sum_acc(hi[a], lo[a], ps[a]);
-        ps[a] = 0.f;
+      for (int k = 0; k < 3; ++k) d[k] = SRC ? a2(in[k], neg2(own[k])) : a2(own[k], neg2(in[k]));
+      const float2 r2 = f2(d[0], d[0], f2(d[1], d[1], m2(d[2], d[2])));
+      const bool near0 = r2.x < (SRC ? own_hh.x : P.w), near1 = r2.y < (SRC ? own_hh.y : P.w);
+      const float2 ri = make_float2(near0 ? 0.f : rsqrt_ftz(r2.x), near1 ? 0.f : rsqrt_ftz(r2.y));
+      if (SRC) {
+        adj_pair2<SRC, KIND>(d, ri, gi, v1, op, on, ps);
+      } else {
+        float2 n2[3], p2[3];
+        if (KIND & K_DL) {
+          const float4 N = sN[kk], Q = sPs[kk];
+          n2[0] = both(N.x), n2[1] = both(N.y), n2[2] = both(N.z);
+          p2[0] = both(Q.x), p2[1] = both(Q.y), p2[2] = both(Q.z);
+        }
+        adj_pair2<SRC, KIND>(d, ri, v1, gi, p2, n2, ps);
+      }
+      if (near0 || near1) {  // listed for the FP64 pass
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if ((h ? near1 : near0) && valid[h]) {
+            const int slot = atomicAdd(A.near_cnt + oc[h], 1);
+            if (slot < A.near_cap) A.near_idx[(size_t)oc[h] * A.near_cap + slot] = sI[kk];
+          }
       }
     }
-    __syncthreads();
-  }
-  if (valid) {
-    double *out = A.partial + ((size_t)blockIdx.y * (size_t)A.nout + (size_t)oc) * NA;
 #pragma unroll
-    for (int a = 0; a < NA; ++a) out[a] = (double)hi[a] + (double)lo[a];
+    for (int a = 0; a < NA; ++a) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int s = tid + h * kAdjPack;
+        float hi = sums[a][s], lo = sums[NA + a][s];
+        two_sum_acc(hi, lo, h ? ps[a].y : ps[a].x);
+        sums[a][s] = hi;
+        sums[NA + a][s] = lo;
+      }
+      ps[a] = both(0.f);
+    }
   }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (valid[h]) {
+      const int s = tid + h * kAdjPack;
+      double *out = A.partial + ((size_t)blockIdx.y * (size_t)A.nout + (size_t)oc[h]) * NA;
+#pragma unroll
+      for (int a = 0; a < NA; ++a) out[a] = (double)sums[a][s] + (double)sums[NA + a][s];
+    }
 }
 
 // ---------------------------------------------------------------- near pairs
@@ -387,17 +509,25 @@ __global__ void k_adj_finish_trg(int64_t nt, int32_t nsplit, const double *__res
   }
 }
 
+template <bool SRC>
+static void launch_adj_mixed(const AdjParams &A, dim3 grid, cudaStream_t st) {
+  if (!A.has_dl) k_adj_mixed<SRC, K_SL><<<grid, kAdjPack, 0, st>>>(A);
+  else if (!A.has_sl) k_adj_mixed<SRC, K_DL><<<grid, kAdjPack, 0, st>>>(A);
+  else k_adj_mixed<SRC, K_SLDL><<<grid, kAdjPack, 0, st>>>(A);
+}
+
 cudaError_t launch_adjoint(bool mixed, bool src_major, const AdjParams &A, cudaStream_t st) {
   dim3 grid((unsigned)((A.nout + kAdjThreads - 1) / kAdjThreads), (unsigned)A.nsplit);
   if (mixed) {
+    grid.y *= (unsigned)A.nsub;
     cudaMemsetAsync(A.near_cnt, 0, sizeof(int32_t) * (size_t)A.nout, st);
     int64_t gn = (A.nout + kAdjThreads - 1) / kAdjThreads;
     if (gn > 65535) gn = 65535;
     if (src_major) {
-      k_adj_mixed<true><<<grid, kAdjThreads, 0, st>>>(A);
+      launch_adj_mixed<true>(A, grid, st);
       k_adj_near<true><<<(int)gn, kAdjThreads, 0, st>>>(A);
     } else {
-      k_adj_mixed<false><<<grid, kAdjThreads, 0, st>>>(A);
+      launch_adj_mixed<false>(A, grid, st);
       k_adj_near<false><<<(int)gn, kAdjThreads, 0, st>>>(A);
     }
     count_launches(1);

@@ -71,10 +71,11 @@ struct AdjParams {
   const int32_t *iperm;    // sorted -> caller index of the input points
   int64_t nout, nin;
   int32_t nsplit;
+  int32_t nsub;            // mixed form: parts of a split, at tile boundaries
   int32_t has_sl, has_dl;
   const double *out64;     // caller FP64 positions of the output points
   const double *in64;      // caller FP64 positions of the input points
-  double *partial;         // [nsplit][nout][12 or 3], caller order
+  double *partial;         // [nsplit nsub][nout][12 or 3], caller order
   // mixed form: near pairs per output point (caller order), filled by the FP32
   // pass and evaluated in FP64 by k_adj_near
   int32_t *near_cnt;       // [nout], zeroed before the FP32 pass

@@ -525,6 +525,7 @@ struct GradPlan {
   bool mixed;
   int64_t ns, nt;
   int32_t nsplit_src, nsplit_trg;
+  int32_t nsub_src = 1, nsub_trg = 1;
   size_t srec, trec, ska, skb, sva, svb, tka, tkb, tva, tvb, hist, hist_scan, bbox_part, bbox,
       part_src, part_trg, counters, near_cnt = 0, near_idx = 0, oframe = 0, total;
 };
@@ -539,6 +540,19 @@ int32_t adj_splits(int64_t nout, int64_t nin, const DevInfo &di) {
   return (int32_t)(s < 1 ? 1 : s);
 }
 
+// Parts a split of the mixed form is cut into, at tile boundaries (the sums of a
+// tile, and so the results to FP64 rounding, do not depend on it): CTAs for
+// eight rounds of eight per SM, of at least two tiles each.
+int32_t adj_parts(int64_t nout, int64_t nin, int32_t nsplit, const DevInfo &di) {
+  const int64_t ctas = ((nout + 127) / 128) * nsplit, tiles = (nin / nsplit + 127) / 128;
+  if (ctas <= 0) return 1;
+  int64_t s = ((int64_t)di.sms * 64 + ctas - 1) / ctas;
+  if (s > tiles / 2) s = tiles / 2;
+  if (s > 16) s = 16;
+  if (s * nsplit > 65535) s = 65535 / nsplit;
+  return (int32_t)(s < 1 ? 1 : s);
+}
+
 stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
   DevInfo di;
   CU(dev_info(di));
@@ -547,6 +561,10 @@ stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
   p.nt = nt;
   p.nsplit_src = adj_splits(ns, nt, di);
   p.nsplit_trg = adj_splits(nt, ns, di);
+  if (p.mixed) {
+    p.nsub_src = adj_parts(ns, nt, p.nsplit_src, di);
+    p.nsub_trg = adj_parts(nt, ns, p.nsplit_trg, di);
+  }
   Alloc a;
   p.counters = a.take(sizeof(int32_t) * 4);
   const size_t rb = p.mixed ? sizeof(SrcRec) : sizeof(SrcRec64);
@@ -565,8 +583,8 @@ stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
   p.hist_scan = a.take(4 * (he + 1));
   p.bbox_part = a.take(sizeof(double) * 6 * 1024);
   p.bbox = a.take(sizeof(double) * 6);
-  p.part_src = a.take(sizeof(double) * 12 * (size_t)ns * (size_t)p.nsplit_src);
-  p.part_trg = a.take(sizeof(double) * 3 * (size_t)nt * (size_t)p.nsplit_trg);
+  p.part_src = a.take(sizeof(double) * 12 * (size_t)ns * (size_t)(p.nsplit_src * p.nsub_src));
+  p.part_trg = a.take(sizeof(double) * 3 * (size_t)nt * (size_t)(p.nsplit_trg * p.nsub_trg));
   if (p.mixed) {  // near-pair lists of one pass at a time (the larger point set)
     const size_t nmax = (size_t)(ns > nt ? ns : nt);
     p.near_cnt = a.take(sizeof(int32_t) * nmax);
@@ -891,12 +909,13 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
     A.nout = ns;
     A.nin = nt;
     A.nsplit = p.nsplit_src;
+    A.nsub = p.nsub_src;
     A.out64 = src;
     A.in64 = trg;
     A.partial = at<double>(ws, p.part_src);
     if (g_ev_start && g_ev_stop) CU(cudaEventRecord(g_ev_start, st));
     CU(launch_adjoint(p.mixed, true, A, st));
-    launch_adj_finish(true, ns, p.nsplit_src, A.partial, w, csl, cdl, grad_f, grad_phi, grad_n,
+    launch_adj_finish(true, ns, p.nsplit_src * p.nsub_src, A.partial, w, csl, cdl, grad_f, grad_phi, grad_n,
                       grad_y, nullptr, st);
   }
   if (grad_x) {
@@ -907,12 +926,13 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
     A.nout = nt;
     A.nin = ns;
     A.nsplit = p.nsplit_trg;
+    A.nsub = p.nsub_trg;
     A.out64 = trg;
     A.in64 = src;
     A.partial = at<double>(ws, p.part_trg);
     CU(launch_adjoint(p.mixed, false, A, st));
     if (g_ev_start && g_ev_stop) CU(cudaEventRecord(g_ev_stop, st));
-    launch_adj_finish(false, nt, p.nsplit_trg, A.partial, nullptr, 0.0, 0.0, nullptr, nullptr,
+    launch_adj_finish(false, nt, p.nsplit_trg * p.nsub_trg, A.partial, nullptr, 0.0, 0.0, nullptr, nullptr,
                       nullptr, nullptr, grad_x, st);
   } else if (g_ev_start && g_ev_stop) {
     CU(cudaEventRecord(g_ev_stop, st));
