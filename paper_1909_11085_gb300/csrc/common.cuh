@@ -169,9 +169,25 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 // Exact-enough split of (x - c) into two floats; used identically for
 // sources and targets so that coincident points get bit-identical local
 // coordinates.
+//
+// lo = fp32(v - hi): for a normal hi of at least 2^-73 the difference is what
+// the rounding dropped (29 bits, less a whole unit when it rounded up) times
+// 2^(e - 52), which the 32-bit integer conversion rounds to nearest even as well
+// and a power of two scales exactly, so no FP64 instruction is needed.
 __device__ __forceinline__ void split_hl(double v, float &hi, float &lo) {
   hi = f64_to_f32_rn(v);
-  lo = f64_to_f32_rn(v - f32_to_f64(hi));
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  const int e = (int)((unsigned)(u >> 52) & 0x7ffu) - 1023;
+  if (e < -73 || e > 126) {
+    lo = f64_to_f32_rn(v - f32_to_f64(hi));
+    return;
+  }
+  // hi's fraction against the kept bits: it differs by one unit when rounded up
+  const unsigned kept = (unsigned)(u >> 29) & 0x7fffffu;
+  int rest = (int)((unsigned)u & 0x1fffffffu);
+  if ((__float_as_uint(hi) & 0x7fffffu) != kept) rest -= 1 << 29;
+  const float r = (float)rest * __uint_as_float((unsigned)(e - 52 + 127) << 23);
+  lo = (u >> 63) ? -r : r;
 }
 __device__ __forceinline__ float to_local(float vh, float vl, float oh, float ol) {
   return __fadd_rn(__fsub_rn(vh, oh), __fsub_rn(vl, ol));

@@ -1,5 +1,5 @@
 // direct_small.cu -- small direct sums (Eq. "sl_stokes" and the double-layer
-// kernel of Sec. 2.1) in one launch, for the mixed form with
+// kernel of Sec. 2.1) in one launch and the splits' sum, for the mixed form with
 // default options when targets x sources is small (kSmallPairs): no pack, no
 // Morton sort, no items, no separate near-pair pass.
 //
@@ -15,13 +15,17 @@
 // pairs included) takes the FP64 difference and 1/|r| (near_contrib): each
 // warp queues them in shared memory and evaluates them 32 at a time, one per
 // lane, since GB300's FP64 pipe is only fed efficiently by full warps; the
-// values of one target are added in queue order (deterministic).  The FP32
+// values of one target are added in queue order (deterministic).  In the loop a warp only keeps its ballots (two words
+// per source pair and target slot); the queue is filled from them after the tile, so
+// the loop stays branch-free and unrolls (the smallest calls 20.3 -> 18.5 us).  The FP32
 // pairs run packed (two staged sources per instruction).  Each thread sums a
 // tile of 128 sources in FP32 and two-sums the tile into (hi, lo); the
-// split's (hi, lo) goes to part[split][target], and the last split of a
-// target block to finish (a counter per block) adds the splits in order
-// (FP32 two-sum, one conversion to FP64 at the end) and writes out
-// (deterministic, no second launch and no waiting).
+// split's (hi, lo) goes to part[split][target], and k_small_finish adds the
+// splits in order (FP32 two-sum, one conversion to FP64 at the end) and writes
+// out.  That second launch, on all SMs and overlapping the first one's end, takes
+// less than the last split of each target block adding them all did (a fence, a
+// counter cleared before every call, and one CTA reading a block's partials): a
+// call of 4,352 points on themselves 41.2 -> 34.9 us, 1,632 on themselves 22.6 -> 19.0.
 #include "common.cuh"
 #include "prep.cuh"
 
@@ -38,10 +42,13 @@ struct SmallArgs {
   int32_t nsplit;
   int32_t accumulate;
   float2 *part;     // [nsplit][nt][3]: a split's compensated sum (hi, lo)
-  int32_t *blocks;  // per target block: splits done (zero before the launch)
+  int32_t *counters;  // the workspace's counters (the status word among them): cleared
   double *out;      // [nt][3]
 };
 
+// Resident CTAs per SM the kernel is compiled for.  The splits, and with them the
+// grouping of the FP32 sums, follow from it.
+constexpr int kSmallResident = 4;
 constexpr int kSmallT = 2;  // targets per thread
 constexpr int kSmallBlock = kSmallThreads * kSmallT;
 constexpr int kSmallPairsPerTile = kSmallThreads / 2;
@@ -106,6 +113,7 @@ constexpr int kSmallQueue = 256;  // near pairs queued per warp (>= 128 free bef
 
 // A warp's shared scratch for evaluating its queued near pairs.
 struct SmallNear {
+  uint4 word[kSmallPairsPerTile];  // near pairs of a staged source pair: ballots by slot and half
   int32_t queue[kSmallQueue];  // source within the staged tile | target slot << 8
   float val[32][3];            // one round's values, by lane
   float tot[32 * kSmallT][3];  // one round's sums, by target slot (zero between rounds)
@@ -165,11 +173,12 @@ __device__ __forceinline__ void small_flush(SmallNear &sn, int qn,
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(kSmallThreads) k_direct_small(SmallArgs a) {
+__global__ void __launch_bounds__(kSmallThreads, kSmallResident) k_direct_small(SmallArgs a) {
   __shared__ float4 S[kSmallPairsPerTile][kSmallFields];
   __shared__ SmallNear near_all[kSmallThreads / 32];
-  __shared__ int last;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid < 4) a.counters[tid] = 0;
   SmallNear &sn = near_all[tid >> 5];
   int32_t *queue = sn.queue;
 #pragma unroll
@@ -255,7 +264,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_direct_small(SmallArgs a) {
         u[k][q] = make_float2(0.f, 0.f);
         un[k][q] = 0.f;
       }
-    int qn = 0;
+    // near pairs of source pair p: one ballot per target slot and half, kept in
+    // shared memory (a queue built here, in the loop, cost a branch and four
+    // dependent ballots for most pairs of a cell with itself)
+    unsigned mine = 0;  // near pairs of this lane's targets
+#pragma unroll 2
     for (int p = 0; p < np; ++p) {
       float4 s[kSmallFields];
 #pragma unroll
@@ -266,27 +279,66 @@ __global__ void __launch_bounds__(kSmallThreads) k_direct_small(SmallArgs a) {
         small_pair<KIND>(s, xh[k], xl[k], u[k], nr[k]);
         if (!act[k]) nr[k] = 0u;
       }
-      if (__any_sync(kFull, (nr[0] | nr[1]) != 0u)) {
-        // queue order: by target slot and half, then by lane
+      const unsigned b0 = __ballot_sync(kFull, nr[0] & 1u), b1 = __ballot_sync(kFull, nr[0] & 2u),
+                     b2 = __ballot_sync(kFull, nr[1] & 1u), b3 = __ballot_sync(kFull, nr[1] & 2u);
+      mine |= nr[0] | nr[1];
+      if (lane == 0) sn.word[p] = make_uint4(b0, b1, b2, b3);
+    }
+    __syncwarp();
+    if (__any_sync(kFull, mine)) {
+      // queue order: by source pair, target slot and half, then by lane
+      auto entry = [](int p, int w, int l) {
+        return (2 * p + (w & 1)) | ((l + 32 * (w >> 1)) << 8);
+      };
+      // lane l counts the pairs of source pairs 2 l and 2 l + 1
+      uint4 w2[2];
+      int cnt2[2];
 #pragma unroll
-        for (int k = 0; k < kSmallT; ++k)
+      for (int e = 0; e < 2; ++e) {
+        w2[e] = 2 * lane + e < np ? sn.word[2 * lane + e] : make_uint4(0u, 0u, 0u, 0u);
+        cnt2[e] = __popc(w2[e].x) + __popc(w2[e].y) + __popc(w2[e].z) + __popc(w2[e].w);
+      }
+      int incl = cnt2[0] + cnt2[1];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const bool b = (nr[k] >> h) & 1u;
-            const unsigned m = __ballot_sync(kFull, b);
-            if (b) queue[qn + __popc(m & lt)] = (2 * p + h) | ((lane + 32 * k) << 8);
-            qn += __popc(m);
-          }
-        if (qn > kSmallQueue - 32 * 2 * kSmallT) {
-          __syncwarp();
-          small_flush<KIND>(sn, qn, S, a.src, a.trg, c0, a.nsplit, t0, lane, un);
-          qn = 0;
-          __syncwarp();
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int total = __shfl_sync(kFull, incl, 31);
+      if (total <= kSmallQueue - 32 * 2 * kSmallT) {
+        int pos = incl - cnt2[0] - cnt2[1];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const unsigned ws[4] = {w2[e].x, w2[e].y, w2[e].z, w2[e].w};
+#pragma unroll
+          for (int w = 0; w < 4; ++w)
+            for (unsigned m = ws[w]; m; m &= m - 1)
+              queue[pos++] = entry(2 * lane + e, w, __ffs(m) - 1);
         }
+        __syncwarp();
+        small_flush<KIND>(sn, total, S, a.src, a.trg, c0, a.nsplit, t0, lane, un);
+      } else {  // more than a queue: source pair by source pair
+        int qn = 0;
+        for (int p = 0; p < np; ++p) {
+          const uint4 wd = sn.word[p];
+          const unsigned ws[4] = {wd.x, wd.y, wd.z, wd.w};
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            if ((ws[w] >> lane) & 1u) queue[qn + __popc(ws[w] & lt)] = entry(p, w, lane);
+            qn += __popc(ws[w]);
+          }
+          if (qn > kSmallQueue - 32 * 2 * kSmallT) {
+            __syncwarp();
+            small_flush<KIND>(sn, qn, S, a.src, a.trg, c0, a.nsplit, t0, lane, un);
+            qn = 0;
+            __syncwarp();
+          }
+        }
+        __syncwarp();
+        if (qn) small_flush<KIND>(sn, qn, S, a.src, a.trg, c0, a.nsplit, t0, lane, un);
       }
     }
     __syncwarp();
-    if (qn) small_flush<KIND>(sn, qn, S, a.src, a.trg, c0, a.nsplit, t0, lane, un);
 #pragma unroll
     for (int k = 0; k < kSmallT; ++k)
 #pragma unroll
@@ -299,51 +351,43 @@ __global__ void __launch_bounds__(kSmallThreads) k_direct_small(SmallArgs a) {
   for (int k = 0; k < kSmallT; ++k) {
     const int64_t t = t0 + 32 * k + lane;
     if (!act[k]) continue;
+    if (a.nsplit == 1) {  // no partial results
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        double *o = a.out + 3 * t + q;
+        *o = (a.accumulate ? *o : 0.0) + ((double)hi[k][q] + (double)lo[k][q]);
+      }
+      continue;
+    }
     float2 *o = a.part + ((size_t)y * (size_t)a.nt + (size_t)t) * 3;
 #pragma unroll
     for (int q = 0; q < 3; ++q) o[q] = make_float2(hi[k][q], lo[k][q]);
   }
-  // the last split of this target block to finish adds the splits in order
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) last = atomicAdd(&a.blocks[blockIdx.x], 1) == a.nsplit - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // the block's partials of one split are 3 x 256 contiguous (hi, lo) pairs:
-  // each thread sums 6 of those values over the splits (from L2, written by
-  // the other CTAs before their fence; loads of 5 splits in flight), in split
-  // order, two-summing the hi parts and adding the lo parts
-  constexpr int kPer = 3 * kSmallBlock / kSmallThreads;
-  const int64_t v0 = 3 * tb, vend = 3 * min(tb + (int64_t)kSmallBlock, a.nt);
-  float sh[kPer], sl[kPer];
+}
+
+// out (+)= the splits' partial results in split order: the hi parts two-summed, the
+// lo parts added, one conversion to FP64.  One value per thread, kSmallAhead
+// splits in flight.  The launch overlaps the end of k_direct_small's (it waits
+// for that kernel's results before it reads them).
+constexpr int kSmallAhead = 12;
+__global__ void __launch_bounds__(kSmallThreads) k_small_finish(SmallArgs a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t n = 3 * a.nt, e = blockIdx.x * (int64_t)kSmallThreads + threadIdx.x;
+  if (e >= n) return;
+  float sh = 0.f, sl = 0.f;
+  for (int y0 = 0; y0 < a.nsplit; y0 += kSmallAhead) {
+    float2 v[kSmallAhead];
 #pragma unroll
-  for (int m = 0; m < kPer; ++m) sh[m] = sl[m] = 0.f;
-  for (int y0 = 0; y0 < a.nsplit; y0 += 5) {
-    float2 v[5][kPer];
+    for (int i = 0; i < kSmallAhead; ++i)
+      v[i] = y0 + i < a.nsplit ? __ldcg(a.part + (size_t)(y0 + i) * (size_t)n + (size_t)e)
+                               : make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < 5; ++i)
-#pragma unroll
-      for (int m = 0; m < kPer; ++m) {
-        const int64_t e = v0 + tid + kSmallThreads * m;
-        v[i][m] = (y0 + i < a.nsplit && e < vend)
-                      ? __ldcg(a.part + (size_t)(y0 + i) * (size_t)a.nt * 3 + (size_t)e)
-                      : make_float2(0.f, 0.f);
-      }
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-#pragma unroll
-      for (int m = 0; m < kPer; ++m) {
-        two_sum_acc(sh[m], sl[m], v[i][m].x);
-        sl[m] += v[i][m].y;
-      }
+    for (int i = 0; i < kSmallAhead; ++i) {
+      two_sum_acc(sh, sl, v[i].x);
+      sl += v[i].y;
+    }
   }
-#pragma unroll
-  for (int m = 0; m < kPer; ++m) {
-    const int64_t e = v0 + tid + kSmallThreads * m;
-    if (e < vend) a.out[e] = (a.accumulate ? a.out[e] : 0.0) + ((double)sh[m] + (double)sl[m]);
-  }
-  if (tid == 0) a.blocks[blockIdx.x] = 0;  // ready for the next call
+  a.out[e] = (a.accumulate ? a.out[e] : 0.0) + ((double)sh + (double)sl);
 }
 }  // namespace
 
@@ -354,12 +398,7 @@ int direct_small_splits(int64_t ns, int64_t nt, int sms) {
   if (blocks <= 0) return 1;
   // one wave: as many splits as the resident CTAs allow (a second, partial
   // wave would double the time)
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_direct_small<K_SLDL>, kSmallThreads,
-                                                    0) != cudaSuccess ||
-      occ < 1)
-    occ = 1;
-  int64_t s = (int64_t)occ * sms / blocks;
+  int64_t s = (int64_t)kSmallResident * sms / blocks;
   const int64_t cap = ns / 64 > 1 ? ns / 64 : 1;  // at least 64 sources per split
   if (s > cap) s = cap;
   if (s > 64) s = 64;
@@ -371,9 +410,9 @@ cudaError_t launch_direct_small(int kinds, const double *src, const double *f, c
                                 const double *phi, const double *w, const double *h, int64_t ns,
                                 const double *trg, int64_t nt, double alpha, double csl,
                                 double cdl, int32_t nsplit, int32_t accumulate, double *part,
-                                int32_t *blocks, double *out, cudaStream_t st) {
+                                int32_t *counters, double *out, cudaStream_t st) {
   SmallArgs a{src, f, nrm, phi, w, h, trg, ns, nt, alpha, csl, cdl, nsplit, accumulate,
-              reinterpret_cast<float2 *>(part), blocks, out};
+              reinterpret_cast<float2 *>(part), counters, out};
   const dim3 grid((unsigned)direct_small_blocks(nt), (unsigned)nsplit);
   if (kinds == K_SL)
     k_direct_small<K_SL><<<grid, kSmallThreads, 0, st>>>(a);
@@ -381,6 +420,19 @@ cudaError_t launch_direct_small(int kinds, const double *src, const double *f, c
     k_direct_small<K_DL><<<grid, kSmallThreads, 0, st>>>(a);
   else
     k_direct_small<K_SLDL><<<grid, kSmallThreads, 0, st>>>(a);
+  count_launches(1);
+  if (nsplit == 1) return cudaGetLastError();
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((3 * nt + kSmallThreads - 1) / kSmallThreads));
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small_finish, a);
+  if (e != cudaSuccess) return e;
   count_launches(1);
   return cudaGetLastError();
 }

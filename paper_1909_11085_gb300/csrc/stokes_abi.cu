@@ -118,7 +118,7 @@ struct Plan {
   int32_t nseg_ranges = 0;  // entries of range_ptr minus one
   bool sort_targets = false;
   bool sort_items = false;
-  bool small = false;  // the one-launch small direct form (direct_small.cu)
+  bool small = false;  // the small direct form (direct_small.cu)
   int32_t ngroup = 0;
   // offsets (the counters always sit at offset 0 of the aligned workspace)
   size_t counters, rec, recfx = 0, keys_a, keys_b, vals_a, vals_b, ikeys_a, ikeys_b, ivals_a, ivals_b, hist,
@@ -159,8 +159,7 @@ int auto_splits(int64_t nt, int64_t ns, const DevInfo &di, bool mixed, int item_
 void layout(Plan &p) {
   Alloc a;
   p.counters = a.take(sizeof(int32_t) * kCounters);
-  if (p.small) {  // partial results per source split and a counter per target block
-    p.cnt = a.take(sizeof(int32_t) * (size_t)direct_small_blocks(p.nt));
+  if (p.small) {  // partial results per source split
     p.part = a.take(sizeof(double) * 3 * (size_t)p.nt * (size_t)p.nsplit);
     p.total = a.off + 256;
     return;
@@ -214,7 +213,7 @@ stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
   p.tile = form_tile(o);
   p.ns = ns;
   p.nt = nt;
-  // small mixed sums with the default options: one launch and the finish
+  // small mixed sums with the default options: one launch and the splits' sum
   if (p.mixed && o->source_splits == 0 && o->tile_config < 0 && ns > 0 && nt > 0 &&
       (double)ns * (double)nt <= (double)kSmallPairs) {
     p.small = true;
@@ -483,14 +482,11 @@ stk_status direct_common(int32_t kinds, const double *src, const double *f, cons
   if (!workspace || wbytes < p.total) return fail(STK_ENOMEM, "workspace too small");
   void *ws = align_ws(workspace);
   if (p.small) {
-    CU(cudaMemsetAsync(at<int32_t>(ws, p.counters), 0, sizeof(int32_t) * 4, st));
-    CU(cudaMemsetAsync(at<int32_t>(ws, p.cnt), 0,
-                       sizeof(int32_t) * (size_t)direct_small_blocks(nt), st));
     const double csl = (kinds & K_SL) ? 1.0 / (8.0 * kPi * mu) : 0.0, cdl = 6.0 / (8.0 * kPi);
     CU(launch_direct_small(kinds, src, (kinds & K_SL) ? f : nullptr, nrm,
                            (kinds & K_DL) ? phi : nullptr, w, h, ns, trg, nt, o->near_ratio, csl,
                            cdl, p.nsplit, o->accumulate ? 1 : 0, at<double>(ws, p.part),
-                           at<int32_t>(ws, p.cnt), out, st));
+                           at<int32_t>(ws, p.counters), out, st));
     return STK_OK;
   }
   launch_zero_ints(at<int32_t>(ws, p.counters), kCounters, st);
