@@ -209,7 +209,8 @@ stk_status stokes_graph_destroy(void *graph_exec);
  * pairs with |r| < near_ratio * h_j are listed per output point (up to 32;
  * a point with more is rescanned over all inputs, one thread per such point,
  * so inputs where most points are near each other are slow) and evaluated in
- * FP64 by a second pass, in input order, so results are deterministic.  FP64: all double.  The
+ * FP64 by a second pass, in input order, so results are deterministic.  FP64: to double
+ * accuracy, the pairs partly in 64-bit fixed point where the inputs' range allows it.  The
  * workspace (stokes_grad_workspace_size) holds the packed records, the
  * Morton orders, the per-split partial gradients and, for MIXED, the near-pair
  * lists.

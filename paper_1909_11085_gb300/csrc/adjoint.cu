@@ -24,8 +24,9 @@
 // input order and adds them to the point's partial.  Keeping FP64 out of the
 // FP32 pass keeps its registers, and so its occupancy, those of FP32 code.
 // An output point with more near pairs than the list holds is rescanned by
-// k_adj_near with the FP32 pass's own frame and test.  The FP64 form does all
-// of it in double.
+// k_adj_near with the FP32 pass's own frame and test.  The FP64 form evaluates
+// the differences, dot products and reciprocals of a pair in fixed point
+// (fixed_pair.cuh) where its inputs fit, and in double otherwise.
 #include <cfloat>
 
 #include "common.cuh"
@@ -416,6 +417,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_near(AdjParams A) {
 // ---------------------------------------------------------------- FP64 pass
 template <bool SRC>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_fp64(AdjParams A) {
+  if (fx_adj_use(*A.fx, A.nout + A.nin)) return;  // k_adj_fx does the call
   constexpr int NA = NAcc<SRC>::value;
   __shared__ double sP[kAdjThreads][3];
   __shared__ double sA[kAdjThreads][3];
@@ -432,7 +434,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_fp64(AdjParams A) {
   double acc[NA];
 #pragma unroll
   for (int a = 0; a < NA; ++a) acc[a] = 0.0;
-  const int64_t i0 = A.nin * blockIdx.y / A.nsplit, i1 = A.nin * (blockIdx.y + 1) / A.nsplit;
+  const int64_t parts = (int64_t)A.nsplit * A.nsub;
+  const int64_t i0 = A.nin * blockIdx.y / parts, i1 = A.nin * (blockIdx.y + 1) / parts;
   for (int64_t tb = i0; tb < i1; tb += kAdjThreads) {
     const int64_t k = tb + tid;
     if (k < i1) {
@@ -479,6 +482,152 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_fp64(AdjParams A) {
   }
 }
 
+// ------------------------------------------------ FP64 pass in fixed point
+// The FP64 form of a pair that fixed point cannot hold.
+template <bool SRC>
+__device__ __noinline__ void adj_fx_slow(const SrcRec64 *T, const SrcRec64 *S, int has_sl,
+                                         int has_dl, double *acc) {
+  const double dx = T->y[0] - S->y[0], dy = T->y[1] - S->y[1], dz = T->y[2] - S->y[2];
+  const double r2 = dx * dx + dy * dy + dz * dz;
+  if (!(r2 > 0.0)) return;  // zero-distance pair contributes nothing
+  const double g[3] = {T->q[0], T->q[1], T->q[2]}, q[3] = {S->q[0], S->q[1], S->q[2]},
+               p[3] = {S->p[0], S->p[1], S->p[2]}, n[3] = {S->n[0], S->n[1], S->n[2]};
+  adj_pair<double, SRC>(dx, dy, dz, rsqrt(r2), g, q, p, n, has_sl, has_dl, acc);
+}
+
+// Exponents of the sources' normals (fx_block's), which their records only hold
+// added to those of psi.
+__global__ void k_adj_nexp(int64_t ns, const double *__restrict__ nrm,
+                           int32_t *__restrict__ nexp) {
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
+       j += (int64_t)gridDim.x * blockDim.x) {
+    const int f = max(fx_field(nrm[3 * j]), max(fx_field(nrm[3 * j + 1]), fx_field(nrm[3 * j + 2])));
+    nexp[j] = f ? f - 1022 : 0;
+  }
+}
+
+// One output point per thread; the inputs' records are read with warp-uniform
+// loads.  With c = (d.g)/r^3, t = (d.g)/r^5, w = d.q + (d.psi)(d.n)/r^2:
+//   ds/dq = g/r + c d,  dt/dpsi = a d,  dt/dn = b d,  a = t (d.n),  b = t (d.psi)
+//   d(s+t)/dd = g w/r^3 + q c + psi a + n b - d [(g.q)/r^3 + t (3 d.q + 5 (d.psi)(d.n)/r^2)]
+// The terms along the own point's vectors only need the sums of their scalars
+// (own: q c + psi a + n b source-major, g w/r^3 target-major); the vectors are
+// multiplied in once at the end.
+//
+// Bound: the FP64 pipe, 31 (source-major) and 23 (target-major) instructions of
+// about 68 cycles per warp and pair of both layers, where k_adj_fp64, with the
+// differences, dot products and the reciprocal square root in FP64 as well,
+// takes about 100 and 80.  34,816 points on themselves, both passes: 365 -> 118 ms
+// (double layer 235 -> 89, single layer 218 -> 67); 1,088 points 1.86 -> 0.42 ms, with
+// splits of at least 32 inputs.  Error against 64 bits (extended precision sums,
+// 544 points): at most 6.5e-16 where k_adj_fp64's is 9.6e-16.
+template <bool SRC, int KIND>
+__global__ void __launch_bounds__(kAdjThreads, 4) k_adj_fx(AdjParams A) {
+  constexpr int NA = NAcc<SRC>::value;
+  const FxState fs = *A.fx;
+  if (!fx_adj_use(fs, A.nout + A.nin)) return;  // k_adj_fp64 does the call
+  const int E = fx_exp(fs);
+  const int64_t o_sorted = (int64_t)blockIdx.x * kAdjThreads + threadIdx.x;
+  if (o_sorted >= A.nout) return;
+  const int64_t oc = A.operm[o_sorted];
+  const SrcRec64 *orec = reinterpret_cast<const SrcRec64 *>(A.out_rec);
+  const SrcRec64 *irec = reinterpret_cast<const SrcRec64 *>(A.in_rec);
+  const SrcFx own = A.out_fx[oc];
+  const int own_en = SRC && (KIND & K_DL) ? A.nexp[oc] : 0;
+  double acc[NA], sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < NA; ++i) acc[i] = 0.0;
+  const int64_t parts = (int64_t)A.nsplit * A.nsub;
+  const int64_t i0 = A.nin * blockIdx.y / parts, i1 = A.nin * (blockIdx.y + 1) / parts;
+  for (int64_t k = i0; k < i1; ++k) {
+    const int32_t ic = A.iperm[k];
+    const SrcFx &in = A.in_fx[ic];
+    const SrcFx &T = SRC ? in : own, &S = SRC ? own : in;
+    int64_t J[3];
+    int32_t dh[3], dl[3];
+    int ea, eb, z, z3;
+    if (!fx_diff(T.y, S.y, T.thr, S.thr, E, J, dh, dl, ea)) {
+      double s[NA];
+      for (int i = 0; i < NA; ++i) s[i] = acc[i];
+      adj_fx_slow<SRC>(SRC ? irec + ic : orec + oc, SRC ? orec + oc : irec + ic, KIND & K_SL,
+                       KIND & K_DL, s);
+      for (int i = 0; i < NA; ++i) acc[i] = s[i];
+      continue;
+    }
+    double d[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) d[i] = fx_to_double(J[i], 1023 + ea);
+    const uint64_t Y = fx_rsqrt(fx_norm2(dh, dl), eb);  // 2^ea / r = Y 2^(eb - 62)
+    const uint64_t Z = fx_mul62(Y, Y, z), W = fx_mul62(Z, Y, z3);
+    const double i1r = fx_round(Y, 1022 + eb - ea), i2r = fx_round(Z, 1022 + 2 * (eb - ea) - z);
+    const double i3r = fx_round(W, 1022 + 3 * (eb - ea) - z - z3);
+    // dots in units of 2^(e - 60): field 1086 + e - 60
+    const double dg = fx_to_double(fx_dot(dh, dl, T.qh, T.ql), 1026 + T.eq + ea);
+    const double c = dg * i3r, t = c * i2r;
+    double e, cd, a = 0.0, b = 0.0, pd = 0.0;  // cd: the bracket above
+    if (KIND & K_DL) {
+      const int en = SRC ? own_en : A.nexp[ic];
+      const double dp = fx_to_double(fx_dot(dh, dl, S.ph, S.pl), 1026 + S.epn - en + ea);
+      const double dn = fx_to_double(fx_dot(dh, dl, S.nh, S.nl), 1026 + en + ea);
+      a = t * dn;
+      b = t * dp;
+      pd = dp * dn;
+    }
+    if (KIND & K_SL) {
+      const double dq = fx_to_double(fx_dot(dh, dl, S.qh, S.ql), 1026 + S.eq + ea);
+      const double gq = fx_to_double(fx_dot(T.qh, T.ql, S.qh, S.ql), 1026 + T.eq + S.eq);
+      const double w = KIND & K_DL ? fx_fma(pd, i2r, dq) : dq;
+      e = i3r * w;
+      // 3 d.q + 5 (w - d.q)
+      const double v = KIND & K_DL ? fx_fma(5.0, w, -2.0 * dq) : 3.0 * dq;
+      cd = fx_fma(t, v, i3r * gq);
+    } else {
+      const double p5 = pd * i2r;
+      e = p5 * i3r;
+      cd = 5.0 * (t * p5);
+    }
+    if (SRC) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        if (KIND & K_SL) acc[i] = fx_fma(d[i], c, fx_fma(in.q[i], i1r, acc[i]));
+        if (KIND & K_DL) {
+          acc[3 + i] = fx_fma(d[i], a, acc[3 + i]);
+          acc[6 + i] = fx_fma(d[i], b, acc[6 + i]);
+        }
+        acc[9 + i] = fx_fma(d[i], cd, fx_fma(-in.q[i], e, acc[9 + i]));
+      }
+      if (KIND & K_SL) sum[0] += c;
+      if (KIND & K_DL) {
+        sum[1] += a;
+        sum[2] += b;
+      }
+    } else {
+      const SrcRec64 &R = irec[ic];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc[i] = fx_fma(-d[i], cd, acc[i]);
+        if (KIND & K_SL) acc[i] = fx_fma(in.q[i], c, acc[i]);
+        if (KIND & K_DL) acc[i] = fx_fma(R.n[i], b, fx_fma(R.p[i], a, acc[i]));
+      }
+      sum[0] += e;
+    }
+  }
+  const SrcRec64 &Ro = orec[oc];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (SRC) {
+      if (KIND & K_SL) acc[9 + i] = fx_fma(-Ro.q[i], sum[0], acc[9 + i]);
+      if (KIND & K_DL)
+        acc[9 + i] = fx_fma(-Ro.n[i], sum[2], fx_fma(-Ro.p[i], sum[1], acc[9 + i]));
+    } else {
+      acc[i] = fx_fma(Ro.q[i], sum[0], acc[i]);
+    }
+  }
+  double *out = A.partial + ((size_t)blockIdx.y * (size_t)A.nout + (size_t)oc) * NA;
+#pragma unroll
+  for (int i = 0; i < NA; ++i) out[i] = acc[i];
+}
+
 // Sums the input splits in order and writes the caller's gradients.
 __global__ void k_adj_finish_src(int64_t ns, int32_t nsplit, const double *__restrict__ part,
                                  const double *__restrict__ w, double csl, double cdl,
@@ -509,6 +658,21 @@ __global__ void k_adj_finish_trg(int64_t nt, int32_t nsplit, const double *__res
   }
 }
 
+void launch_adj_nexp(int64_t ns, const double *nrm, int32_t *nexp, cudaStream_t st) {
+  int64_t g = (ns + 255) / 256;
+  if (g > 4096) g = 4096;
+  k_adj_nexp<<<(int)(g < 1 ? 1 : g), 256, 0, st>>>(ns, nrm, nexp);
+  count_launches(1);
+}
+
+template <bool SRC>
+static void launch_adj_fx(const AdjParams &A, dim3 grid, cudaStream_t st) {
+  if (!A.has_dl) k_adj_fx<SRC, K_SL><<<grid, kAdjThreads, 0, st>>>(A);
+  else if (!A.has_sl) k_adj_fx<SRC, K_DL><<<grid, kAdjThreads, 0, st>>>(A);
+  else k_adj_fx<SRC, K_SLDL><<<grid, kAdjThreads, 0, st>>>(A);
+  k_adj_fp64<SRC><<<grid, kAdjThreads, 0, st>>>(A);  // the device picks one of them
+}
+
 template <bool SRC>
 static void launch_adj_mixed(const AdjParams &A, dim3 grid, cudaStream_t st) {
   if (!A.has_dl) k_adj_mixed<SRC, K_SL><<<grid, kAdjPack, 0, st>>>(A);
@@ -517,9 +681,9 @@ static void launch_adj_mixed(const AdjParams &A, dim3 grid, cudaStream_t st) {
 }
 
 cudaError_t launch_adjoint(bool mixed, bool src_major, const AdjParams &A, cudaStream_t st) {
-  dim3 grid((unsigned)((A.nout + kAdjThreads - 1) / kAdjThreads), (unsigned)A.nsplit);
+  const dim3 grid((unsigned)((A.nout + kAdjThreads - 1) / kAdjThreads),
+                  (unsigned)(A.nsplit * A.nsub));
   if (mixed) {
-    grid.y *= (unsigned)A.nsub;
     cudaMemsetAsync(A.near_cnt, 0, sizeof(int32_t) * (size_t)A.nout, st);
     int64_t gn = (A.nout + kAdjThreads - 1) / kAdjThreads;
     if (gn > 65535) gn = 65535;
@@ -532,10 +696,9 @@ cudaError_t launch_adjoint(bool mixed, bool src_major, const AdjParams &A, cudaS
     }
     count_launches(1);
   } else {
-    if (src_major)
-      k_adj_fp64<true><<<grid, kAdjThreads, 0, st>>>(A);
-    else
-      k_adj_fp64<false><<<grid, kAdjThreads, 0, st>>>(A);
+    if (src_major) launch_adj_fx<true>(A, grid, st);
+    else launch_adj_fx<false>(A, grid, st);
+    count_launches(1);
   }
   count_launches(1);
   return cudaGetLastError();

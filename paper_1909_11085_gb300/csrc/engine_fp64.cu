@@ -350,13 +350,26 @@ void launch_pack_fp64(int64_t ns, const double *src, const double *f, const doub
   count_launches(1);
 }
 
+void launch_fx_range(int64_t ns, const double *src, int64_t nt, const double *trg, FxState *fx,
+                     cudaStream_t st) {
+  k_fx_range<<<pack_grid(3 * ns + 3 * nt), 256, 0, st>>>(ns, src, nt, trg, fx);
+  count_launches(1);
+}
+
+void launch_fx_records(int64_t n, const double *pts, const double *f, const double *nrm,
+                       const double *phi, const double *w, double csl, double cdl, FxState *fx,
+                       SrcFx *rec, cudaStream_t st) {
+  k_pack_fx<<<pack_grid(n), 256, 0, st>>>(n, pts, f, nrm, phi, w, csl, cdl, fx, rec);
+  count_launches(1);
+}
+
 void launch_pack_fx(int64_t ns, const double *src, int64_t nt, const double *trg, const double *f,
                     const double *nrm, const double *phi, const double *w, double csl, double cdl,
                     FxState *fx, SrcFx *recfx, SrcRec64 *rec, cudaStream_t st) {
-  k_fx_range<<<pack_grid(3 * ns + 3 * nt), 256, 0, st>>>(ns, src, nt, trg, fx);
-  k_pack_fx<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, fx, recfx);
+  launch_fx_range(ns, src, nt, trg, fx, st);
+  launch_fx_records(ns, src, f, nrm, phi, w, csl, cdl, fx, recfx, st);
   k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, fx, rec);
-  count_launches(3);
+  count_launches(1);
 }
 
 cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,

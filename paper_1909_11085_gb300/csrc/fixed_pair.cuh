@@ -297,6 +297,40 @@ FX_HD uint64_t fx_rsqrt(int64_t W, int &b) {
   return ((uint64_t)m << 38) + (uint64_t)(mc >> 22);
 }
 
+// V 2^-62 in [1/2, 1] as FP64 with exponent field f for [1/2, 1).
+FX_HD double fx_round(uint64_t V, int f) {
+  const uint64_t M = (V + 256) >> 9;
+  return fx_bits((uint32_t)(M >> 32) - 0x100000u + ((uint32_t)f << 20), (uint32_t)M);
+}
+// a b 2^-62 for a, b in [2^61, 2^62], doubled when below 2^61 (z: whether it was).
+FX_HD uint64_t fx_mul62(uint64_t a, uint64_t b, int &z) {
+  const uint64_t p = fx_mulhi(a << 1, b << 1);
+  z = (uint32_t)(p >> 32) < (1u << 29) ? 1 : 0;
+  return p << z;
+}
+
+// Difference of two positions, left-justified: d = J 2^(a - 63), |d| 2^-a in
+// [1/2, 2) and the limbs of J; false when it is below the points' threshold.
+FX_HD bool fx_diff(const int64_t (&x)[3], const int64_t (&y)[3], uint32_t xthr, uint32_t ythr,
+                   int E, int64_t (&J)[3], int32_t (&dh)[3], int32_t (&dl)[3], int &a) {
+  int64_t d[3];
+  uint32_t any = 0u;
+  for (int k = 0; k < 3; ++k) {
+    d[k] = x[k] - y[k];
+    const int32_t hi = (int32_t)(d[k] >> 32);
+    any |= (uint32_t)(hi ^ (hi >> 31));
+  }
+  if (any < xthr || any < ythr) return false;
+  const int s = fx_clz(any) - 1;  // left-justified: |J| in [2^62, 2^63)
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t hi = (uint32_t)((uint64_t)d[k] >> 32), lo = (uint32_t)d[k];
+    J[k] = (int64_t)(((uint64_t)fx_shl(lo, hi, s) << 32) | (lo << s));
+    fx_limbs(J[k], dh[k], dl[k]);
+  }
+  a = E + 1 - s;  // d = J 2^-s quanta of 2^(E - 62)
+  return true;
+}
+
 // ----------------------------------------------------------------------- pair
 // Returns false when the pair has to take the FP64 form, else adds it to acc.
 //   SL: q/r + d (d.q)/r^3,  DL: d (d.psi)(d.n)/r^5,  K_EQ: SL + s d/r^3 (an
@@ -307,36 +341,16 @@ constexpr int K_EQ = 4 | K_SL;
 template <int KIND>
 FX_HD bool fx_pair(const int64_t (&x)[3], uint32_t xthr, int E, const SrcFx &S, double (&acc)[3],
                    double s0 = 0.0) {
-  int64_t d[3];
-  uint32_t any = 0u;
-  for (int k = 0; k < 3; ++k) {
-    d[k] = x[k] - S.y[k];
-    const int32_t hi = (int32_t)(d[k] >> 32);
-    any |= (uint32_t)(hi ^ (hi >> 31));
-  }
-  if (any < xthr || any < S.thr) return false;
-  const int s = fx_clz(any) - 1;  // left-justified: |D| in [2^62, 2^63)
+  int64_t J[3];
   int32_t dh[3], dl[3];
+  int a, b, z;
+  if (!fx_diff(x, S.y, xthr, S.thr, E, J, dh, dl, a)) return false;
   double D[3];
-  for (int k = 0; k < 3; ++k) {
-    const uint32_t hi = (uint32_t)((uint64_t)d[k] >> 32), lo = (uint32_t)d[k];
-    const int64_t J = (int64_t)(((uint64_t)fx_shl(lo, hi, s) << 32) | (lo << s));
-    fx_limbs(J, dh[k], dl[k]);
-    D[k] = fx_to_double(J, 1023);  // J 2^-63
-  }
-  const int a = E + 1 - s;  // d = D 2^a: J = D 2^63, d = J 2^-s quanta of 2^(E - 62)
-  int b;
-  const uint64_t Y = fx_rsqrt(fx_norm2(dh, dl), b);  // 1/R = Y 2^(b - 62)
-  // Y rounded to 53 bits; y 2^b = 1/R
-  const uint64_t M = (Y + 256) >> 9;
-  const uint32_t mh = (uint32_t)(M >> 32) - 0x100000u, ml = (uint32_t)M;
-  const double ria = fx_bits(mh + ((uint32_t)(1022 + b - a) << 20), ml);  // 2^-a / R
-  // 1/R^2 = Y^2 2^(2b - 124)
-  const uint64_t Z = fx_mulhi(Y << 1, Y << 1);  // y^2 2^62, in [2^60, 2^62]
-  const int z = (uint32_t)(Z >> 32) < (1u << 29) ? 1 : 0;
-  const uint64_t M2 = ((Z << z) + 256) >> 9;
-  const double ri2 = fx_bits((uint32_t)(M2 >> 32) - 0x100000u + ((uint32_t)(1022 + 2 * b - z) << 20),
-                             (uint32_t)M2);
+  for (int k = 0; k < 3; ++k) D[k] = fx_to_double(J[k], 1023);  // J 2^-63
+  const uint64_t Y = fx_rsqrt(fx_norm2(dh, dl), b);             // 1/R = Y 2^(b - 62)
+  const double ria = fx_round(Y, 1022 + b - a);                 // 2^-a / R
+  const uint64_t Z = fx_mul62(Y, Y, z);                         // 1/R^2 = Z 2^(2b - z - 62)
+  const double ri2 = fx_round(Z, 1022 + 2 * b - z);
   double c;
   if (KIND & K_DL) {
     // dots in units of 2^(e - 60): field 1086 + e - 60
@@ -360,6 +374,14 @@ FX_HD bool fx_pair(const int64_t (&x)[3], uint32_t xthr, int E, const SrcFx &S, 
     for (int k = 0; k < 3; ++k) acc[k] = fx_fma(D[k], c, acc[k]);
   }
   return true;
+}
+
+// The adjoint's pairs (adjoint.cu) use the same parts for n points of both sets;
+// the coordinates' exponent is within kFxAdjExp so that 1/r^3 stays in range.
+constexpr int kFxAdjExp = 100;
+FX_HD bool fx_adj_use(const FxState &s, int64_t n) {
+  const int E = fx_exp(s);
+  return fx_use(s, n) && E <= kFxAdjExp && E >= -kFxAdjExp;
 }
 
 }  // namespace stk

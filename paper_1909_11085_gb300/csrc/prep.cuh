@@ -22,6 +22,13 @@ void launch_pack_fp64(int64_t ns, const double *src, const double *f, const doub
 void launch_pack_fx(int64_t ns, const double *src, int64_t nt, const double *trg, const double *f,
                     const double *nrm, const double *phi, const double *w, double csl, double cdl,
                     FxState *fx, SrcFx *recfx, SrcRec64 *rec, cudaStream_t st);
+// The parts of it: the largest coordinate of both point sets into *fx, and the
+// fixed point records of one.
+void launch_fx_range(int64_t ns, const double *src, int64_t nt, const double *trg, FxState *fx,
+                     cudaStream_t st);
+void launch_fx_records(int64_t n, const double *pts, const double *f, const double *nrm,
+                       const double *phi, const double *w, double csl, double cdl, FxState *fx,
+                       SrcFx *rec, cudaStream_t st);
 int bbox_partial_blocks(int64_t n);
 void launch_bbox(int64_t n, const double *pts, double *partial, double *box, cudaStream_t st);
 void launch_morton(int64_t n, const double *pts, const double *box, const int64_t *group_ptr,
@@ -71,7 +78,7 @@ struct AdjParams {
   const int32_t *iperm;    // sorted -> caller index of the input points
   int64_t nout, nin;
   int32_t nsplit;
-  int32_t nsub;            // mixed form: parts of a split, at tile boundaries
+  int32_t nsub;            // parts of a split, in the mixed form at tile boundaries
   int32_t has_sl, has_dl;
   const double *out64;     // caller FP64 positions of the output points
   const double *in64;      // caller FP64 positions of the input points
@@ -82,7 +89,13 @@ struct AdjParams {
   int32_t *near_idx;       // [nout][near_cap] input caller indices
   int32_t near_cap;
   float *oframe;           // [nout][9]: local coordinates and the CTA frame origin (hi, lo)
+  // FP64 form: fixed point records of both point sets, and the sources' normals'
+  // exponents
+  const FxState *fx;
+  const SrcFx *out_fx, *in_fx;
+  const int32_t *nexp;
 };
+void launch_adj_nexp(int64_t ns, const double *nrm, int32_t *nexp, cudaStream_t st);
 cudaError_t launch_adjoint(bool mixed, bool src_major, const AdjParams &A, cudaStream_t st);
 constexpr int32_t kAdjNearCap = 32;  // near pairs listed per output point
 void launch_adj_finish(bool src_major, int64_t n, int32_t nsplit, const double *part,

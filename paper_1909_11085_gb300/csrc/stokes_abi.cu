@@ -523,7 +523,8 @@ struct GradPlan {
   int32_t nsplit_src, nsplit_trg;
   int32_t nsub_src = 1, nsub_trg = 1;
   size_t srec, trec, ska, skb, sva, svb, tka, tkb, tva, tvb, hist, hist_scan, bbox_part, bbox,
-      part_src, part_trg, counters, near_cnt = 0, near_idx = 0, oframe = 0, total;
+      part_src, part_trg, counters, near_cnt = 0, near_idx = 0, oframe = 0, fx = 0, sfx = 0,
+      tfx = 0, nexp = 0, total;
 };
 
 int32_t adj_splits(int64_t nout, int64_t nin, const DevInfo &di) {
@@ -549,6 +550,17 @@ int32_t adj_parts(int64_t nout, int64_t nin, int32_t nsplit, const DevInfo &di) 
   return (int32_t)(s < 1 ? 1 : s);
 }
 
+// Parts a split of the FP64 form is cut into: CTAs for eight rounds of four per SM, of
+// at least 32 inputs each; all parts of an output point together at most 256.
+int32_t adj_parts_fp64(int64_t nout, int64_t nin, int32_t nsplit, const DevInfo &di) {
+  const int64_t ctas = ((nout + 127) / 128) * nsplit;
+  if (ctas <= 0) return 1;
+  int64_t s = ((int64_t)di.sms * 32 + ctas - 1) / ctas;
+  if (s > nin / nsplit / 32) s = nin / nsplit / 32;
+  if (s > 256 / nsplit) s = 256 / nsplit;
+  return (int32_t)(s < 1 ? 1 : s);
+}
+
 stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
   DevInfo di;
   CU(dev_info(di));
@@ -560,6 +572,9 @@ stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
   if (p.mixed) {
     p.nsub_src = adj_parts(ns, nt, p.nsplit_src, di);
     p.nsub_trg = adj_parts(nt, ns, p.nsplit_trg, di);
+  } else {
+    p.nsub_src = adj_parts_fp64(ns, nt, p.nsplit_src, di);
+    p.nsub_trg = adj_parts_fp64(nt, ns, p.nsplit_trg, di);
   }
   Alloc a;
   p.counters = a.take(sizeof(int32_t) * 4);
@@ -586,6 +601,11 @@ stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
     p.near_cnt = a.take(sizeof(int32_t) * nmax);
     p.near_idx = a.take(sizeof(int32_t) * nmax * (size_t)kAdjNearCap);
     p.oframe = a.take(sizeof(float) * 9 * nmax);
+  } else {
+    p.fx = a.take(sizeof(FxState));
+    p.sfx = a.take(sizeof(SrcFx) * (size_t)ns);
+    p.tfx = a.take(sizeof(SrcFx) * (size_t)nt);
+    p.nexp = a.take(sizeof(int32_t) * (size_t)ns);
   }
   p.total = a.off + 256;
   return STK_OK;
@@ -883,6 +903,13 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
     launch_pack_fp64(ns, src, f, nrm, phi, w, csl, cdl, at<SrcRec64>(ws, p.srec), st);
     launch_pack_fp64(nt, trg, g, nullptr, nullptr, nullptr, 1.0, 0.0, at<SrcRec64>(ws, p.trec),
                      st);
+    FxState *fx = at<FxState>(ws, p.fx);
+    CU(cudaMemsetAsync(fx, 0, sizeof(FxState), st));
+    launch_fx_range(ns, src, nt, trg, fx, st);
+    launch_fx_records(ns, src, f, nrm, phi, w, csl, cdl, fx, at<SrcFx>(ws, p.sfx), st);
+    launch_fx_records(nt, trg, g, nullptr, nullptr, nullptr, 1.0, 0.0, fx, at<SrcFx>(ws, p.tfx),
+                      st);
+    if (phi) launch_adj_nexp(ns, nrm, at<int32_t>(ws, p.nexp), st);
   }
   CU(cudaGetLastError());
   const int32_t *sperm = morton_perm(ns, src, ws, p.ska, p.skb, p.sva, p.svb, p.hist, p.hist_scan,
@@ -895,11 +922,15 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
   A.near_idx = p.mixed ? at<int32_t>(ws, p.near_idx) : nullptr;
   A.near_cap = kAdjNearCap;
   A.oframe = p.mixed ? at<float>(ws, p.oframe) : nullptr;
+  A.fx = at<FxState>(ws, p.fx);
+  A.nexp = at<int32_t>(ws, p.nexp);
   A.has_sl = f ? 1 : 0;
   A.has_dl = phi ? 1 : 0;
   if (want_src) {
     A.out_rec = at<void>(ws, p.srec);
     A.in_rec = at<void>(ws, p.trec);
+    A.out_fx = at<SrcFx>(ws, p.sfx);
+    A.in_fx = at<SrcFx>(ws, p.tfx);
     A.operm = sperm;
     A.iperm = tperm;
     A.nout = ns;
@@ -917,6 +948,8 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
   if (grad_x) {
     A.out_rec = at<void>(ws, p.trec);
     A.in_rec = at<void>(ws, p.srec);
+    A.out_fx = at<SrcFx>(ws, p.tfx);
+    A.in_fx = at<SrcFx>(ws, p.sfx);
     A.operm = tperm;
     A.iperm = sperm;
     A.nout = nt;
