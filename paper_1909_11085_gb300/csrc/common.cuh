@@ -10,6 +10,9 @@ namespace stk {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarp = 32;
 constexpr int kChunk = 64;      // sources staged per chunk (one bulk copy)
+// The mixed engine sums kSumChunks chunks in plain FP32, then two-sums them: parts of a
+// source range cut at whole groups sum the same groups.
+constexpr int kSumChunks = 8, kSumGroup = kSumChunks * kChunk;
 constexpr int kItemMax = 128;   // most targets per work item (32 lanes x 4)
 
 // Work-item shapes the autotuner chooses from: the most targets per item and

@@ -43,14 +43,24 @@
 
 namespace stk {
 
+constexpr int kTMax = 5;     // most targets per lane
+
 // Resident CTAs per SM the engine is compiled for (registers per thread =
-// 65536 / (128 * this)).
-#ifndef STK_ENGINE_MIN_BLOCKS
-#define STK_ENGINE_MIN_BLOCKS 3
-#endif
+// 65536 / (128 * this)), and the targets of a lane it evaluates together, stage by
+// stage: a packed FMA with three different register operands holds the FMA pipe for
+// 2.8 cycles, one that shares an operand with the instruction before it for 2.2, and
+// targets side by side share the source's vectors.  The double layer alone fits four
+// CTAs that way (139,264 x 204,800: 18.23 -> 17.79 ms, 619,520 x 193,600 points:
+// 75.6 -> 73.3); one target at a time it is best at three CTAs (four: 19.1 ms), as
+// are the single layer (140,000 points: 11.49 ms, grouped with four CTAs 11.98) and
+// both layers (16.15, 16.52), which need more registers.
+template <int KMODE>
+struct EngineShape {
+  static constexpr int kResident = KMODE == K_DL ? 4 : 3;
+  static constexpr int kGroup = KMODE == K_DL ? 3 : kTMax;
+};
 
 constexpr int kSegWin = 64;  // segments read into shared memory at a time
-constexpr int kTMax = 5;     // most targets per lane
 
 constexpr int kPairs = kChunk / 2;  // staged source pairs per chunk
 constexpr int kFields = 7;          // float4 fields per source pair
@@ -138,6 +148,18 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
+// Dot products of the first m differences with one vector of the source pair.
+template <int G>
+__device__ __forceinline__ void dots(int m, const float2 (&d)[G][3], const float2 (&v)[3],
+                                     float2 (&o)[G]) {
+#pragma unroll
+  for (int i = 0; i < m; ++i) o[i] = mul2(d[i][2], v[2]);
+#pragma unroll
+  for (int i = 0; i < m; ++i) o[i] = fma2(d[i][1], v[1], o[i]);
+#pragma unroll
+  for (int i = 0; i < m; ++i) o[i] = fma2(d[i][0], v[0], o[i]);
+}
+
 // Adds the far-field contribution of one staged source pair to T targets
 // (x2: each coordinate duplicated into both halves; ps: per-half sums).
 // SL:   q/r + d (d.q)/r^3             (q pre-scaled by w / (8 pi mu))
@@ -145,45 +167,50 @@ __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); 
 // SLDL: q/r + d [(d.q)/r^3 + (d.psi)(d.n)/r^5]
 // Per half the operations, operands and rounding are those of a scalar
 // evaluation: d = x - y, |r|^2 = dx dx + (dy dy + dz dz) (pair_r2).
-template <int T, int KIND, bool MASKED>
+template <int T, int GROUP, int KIND, bool MASKED>
 __device__ __forceinline__ void pair_block(const float2 (&x2)[T][3], float2 (&ps)[T][3],
                                            const float4 (&s)[kFields]) {
-  const float2 ny_x = lo2(s[0]), ny_y = hi2(s[0]), ny_z = lo2(s[1]), hh = hi2(s[1]);
-  const float2 qx = lo2(s[2]), qy = hi2(s[2]), qz = lo2(s[3]);
-  const float2 nx = hi2(s[3]), ny = lo2(s[4]), nz = hi2(s[4]);
-  const float2 px = lo2(s[5]), py = hi2(s[5]), pz = lo2(s[6]);
+  const float2 hh = hi2(s[1]);
+  const float2 ny[3] = {lo2(s[0]), hi2(s[0]), lo2(s[1])}, q[3] = {lo2(s[2]), hi2(s[2]), lo2(s[3])};
+  const float2 n[3] = {hi2(s[3]), lo2(s[4]), hi2(s[4])}, p[3] = {lo2(s[5]), hi2(s[5]), lo2(s[6])};
+  constexpr int NG = (T + GROUP - 1) / GROUP, G = (T + NG - 1) / NG;  // groups, targets of one
 #pragma unroll
-  for (int t = 0; t < T; ++t) {
-    const float2 dx = add2(x2[t][0], ny_x), dy = add2(x2[t][1], ny_y), dz = add2(x2[t][2], ny_z);
-    float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-    // near pair: rsqrt(+inf) = 0 removes it from this sum (k_near adds it)
-    if (MASKED) {
-      if (is_near(r2.x, hh.x)) r2.x = __int_as_float(0x7f800000);
-      if (is_near(r2.y, hh.y)) r2.y = __int_as_float(0x7f800000);
+  for (int g = 0; g < T; g += G) {
+    const int m = T - g < G ? T - g : G;
+    float2 d[G][3], r2[G], ri[G], dq[G], dp[G], dn[G];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int i = 0; i < m; ++i) d[i][k] = add2(x2[g + i][k], ny[k]);
+#pragma unroll
+    for (int i = 0; i < m; ++i) {
+      r2[i] = fma2(d[i][0], d[i][0], fma2(d[i][1], d[i][1], mul2(d[i][2], d[i][2])));
+      // near pair: rsqrt(+inf) = 0 removes it from this sum (k_near adds it)
+      if (MASKED) {
+        if (is_near(r2[i].x, hh.x)) r2[i].x = __int_as_float(0x7f800000);
+        if (is_near(r2[i].y, hh.y)) r2[i].y = __int_as_float(0x7f800000);
+      }
     }
-    const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-    const float2 ri2 = mul2(ri, ri);
-    if (KIND == K_SL) {
-      const float2 dq = fma2(dx, qx, fma2(dy, qy, mul2(dz, qz)));
-      const float2 c = mul2(dq, ri2);
-      ps[t][0] = fma2(fma2(dx, c, qx), ri, ps[t][0]);
-      ps[t][1] = fma2(fma2(dy, c, qy), ri, ps[t][1]);
-      ps[t][2] = fma2(fma2(dz, c, qz), ri, ps[t][2]);
-    } else if (KIND == K_DL) {
-      const float2 dp = fma2(dx, px, fma2(dy, py, mul2(dz, pz)));
-      const float2 dn = fma2(dx, nx, fma2(dy, ny, mul2(dz, nz)));
-      const float2 c = mul2(mul2(dp, dn), mul2(mul2(ri2, ri2), ri));
-      ps[t][0] = fma2(dx, c, ps[t][0]);
-      ps[t][1] = fma2(dy, c, ps[t][1]);
-      ps[t][2] = fma2(dz, c, ps[t][2]);
-    } else {
-      const float2 dq = fma2(dx, qx, fma2(dy, qy, mul2(dz, qz)));
-      const float2 dp = fma2(dx, px, fma2(dy, py, mul2(dz, pz)));
-      const float2 dn = fma2(dx, nx, fma2(dy, ny, mul2(dz, nz)));
-      const float2 c = mul2(fma2(mul2(dp, dn), ri2, dq), ri2);
-      ps[t][0] = fma2(fma2(dx, c, qx), ri, ps[t][0]);
-      ps[t][1] = fma2(fma2(dy, c, qy), ri, ps[t][1]);
-      ps[t][2] = fma2(fma2(dz, c, qz), ri, ps[t][2]);
+#pragma unroll
+    for (int i = 0; i < m; ++i) ri[i] = make_float2(rsqrt_ftz(r2[i].x), rsqrt_ftz(r2[i].y));
+    if (KIND & K_SL) dots<G>(m, d, q, dq);
+    if (KIND & K_DL) {
+      dots<G>(m, d, p, dp);
+      dots<G>(m, d, n, dn);
+    }
+#pragma unroll
+    for (int i = 0; i < m; ++i) {
+      float2(&u)[3] = ps[g + i];
+      const float2 ri2 = mul2(ri[i], ri[i]);
+      if (KIND == K_DL) {
+        const float2 c = mul2(mul2(dp[i], dn[i]), mul2(mul2(ri2, ri2), ri[i]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) u[k] = fma2(d[i][k], c, u[k]);
+      } else {
+        const float2 c = mul2(KIND == K_SL ? dq[i] : fma2(mul2(dp[i], dn[i]), ri2, dq[i]), ri2);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) u[k] = fma2(fma2(d[i][k], c, q[k]), ri[i], u[k]);
+      }
     }
   }
 }
@@ -207,7 +234,7 @@ __device__ __forceinline__ void load_pair(const WarpSmem &sm, int j, float4 (&s)
 
 // Pairs [0, nfar / 2) hold far sources only; pairs from nfar / 2 to the end
 // hold candidates (and possibly one far source with hh = 0, and a zero pad).
-template <int T, int KIND>
+template <int T, int GROUP, int KIND>
 __device__ __forceinline__ void chunk_compute(WarpSmem &sm, const EngineParams &P,
                                               const ItemCtx &ic, int n, int nfar,
                                               const float2 (&x2)[T][3], float2 (&ps)[T][3]) {
@@ -215,12 +242,12 @@ __device__ __forceinline__ void chunk_compute(WarpSmem &sm, const EngineParams &
   for (int j = ic.sg; j < jfar; j += ic.b) {
     float4 s[kFields];
     load_pair<KIND>(sm, j, s);
-    pair_block<T, KIND, false>(x2, ps, s);
+    pair_block<T, GROUP, KIND, false>(x2, ps, s);
   }
   for (int j = jfar + ic.sg; j < jend; j += ic.b) {
     float4 s[kFields];
     load_pair<KIND>(sm, j, s);
-    pair_block<T, KIND, true>(x2, ps, s);
+    pair_block<T, GROUP, KIND, true>(x2, ps, s);
   }
 }
 
@@ -387,12 +414,13 @@ template <int T, int KMODE>
 __device__ __forceinline__ void dispatch_compute(int kind, WarpSmem &sm, const EngineParams &P,
                                                  const ItemCtx &ic, int n, int nfar,
                                                  const float2 (&x2)[T][3], float2 (&ps)[T][3]) {
+  constexpr int G = EngineShape<KMODE>::kGroup;
   if (KMODE != 0) {
-    chunk_compute<T, KMODE>(sm, P, ic, n, nfar, x2, ps);
+    chunk_compute<T, G, KMODE>(sm, P, ic, n, nfar, x2, ps);
   } else if (kind == K_SL) {
-    chunk_compute<T, K_SL>(sm, P, ic, n, nfar, x2, ps);
+    chunk_compute<T, G, K_SL>(sm, P, ic, n, nfar, x2, ps);
   } else {
-    chunk_compute<T, K_DL>(sm, P, ic, n, nfar, x2, ps);
+    chunk_compute<T, G, K_DL>(sm, P, ic, n, nfar, x2, ps);
   }
 }
 
@@ -575,7 +603,7 @@ __device__ bool run_item(const EngineParams &P, const Item &it, int id, WarpSmem
     dispatch_compute<T, KMODE>(kind_cur, sm, P, ic, n_cur, nfar, x2, ps);
     // plain FP32 over eight chunks (<= 256 sources per half), then into the
     // (hi, lo) sums
-    if (++npend == 8 || !have_next) {
+    if (++npend == kSumChunks || !have_next) {
       npend = 0;
 #pragma unroll
       for (int t = 0; t < T; ++t)
@@ -635,7 +663,8 @@ __device__ bool run_item(const EngineParams &P, const Item &it, int id, WarpSmem
 }
 
 template <int KMODE>
-__global__ void __launch_bounds__(kWarpsPerCta *kWarp, STK_ENGINE_MIN_BLOCKS) k_engine_mixed(EngineParams P) {
+__global__ void __launch_bounds__(kWarpsPerCta *kWarp, EngineShape<KMODE>::kResident)
+    k_engine_mixed(EngineParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   WarpSmem &sm = reinterpret_cast<WarpSmem *>(smem_raw)[threadIdx.x / kWarp];
   const int lane = threadIdx.x & (kWarp - 1);
@@ -693,20 +722,21 @@ cudaError_t launch_engine_mixed(const EngineParams &P, int grid, cudaStream_t st
 }
 
 template <int KMODE>
-static cudaError_t set_smem_attr() {
-  return cudaFuncSetAttribute(k_engine_mixed<KMODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)engine_mixed_smem_bytes());
+static cudaError_t occupancy(int *blocks_per_sm) {
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_engine_mixed<KMODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)engine_mixed_smem_bytes());
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      blocks_per_sm, k_engine_mixed<KMODE>, kWarpsPerCta * kWarp, engine_mixed_smem_bytes());
 }
 
-cudaError_t engine_mixed_occupancy(int *blocks_per_sm) {
-  cudaError_t e;
-  if ((e = set_smem_attr<0>()) != cudaSuccess) return e;
-  if ((e = set_smem_attr<K_SL>()) != cudaSuccess) return e;
-  if ((e = set_smem_attr<K_DL>()) != cudaSuccess) return e;
-  if ((e = set_smem_attr<K_SLDL>()) != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_engine_mixed<K_SLDL>,
-                                                       kWarpsPerCta * kWarp,
-                                                       engine_mixed_smem_bytes());
+cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[4]) {
+  cudaError_t e = occupancy<0>(blocks_per_sm);
+  if (e == cudaSuccess) e = occupancy<K_SL>(blocks_per_sm + K_SL);
+  if (e == cudaSuccess) e = occupancy<K_DL>(blocks_per_sm + K_DL);
+  if (e == cudaSuccess) e = occupancy<K_SLDL>(blocks_per_sm + K_SLDL);
+  return e;
 }
 
 }  // namespace stk

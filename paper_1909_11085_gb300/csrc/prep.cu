@@ -395,14 +395,15 @@ __device__ __forceinline__ uint64_t cost_key(int64_t tn, int64_t nsrc) {
   return ((uint64_t)tn << 32) | s;
 }
 
-__global__ void k_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t item_max,
-                               Item *__restrict__ items, int64_t *__restrict__ range_ptr,
+__global__ void k_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t nsub,
+                               int32_t item_max, Item *__restrict__ items, int64_t *__restrict__ range_ptr,
                                int32_t *__restrict__ n_items) {
   const int32_t nchunk = (nt + item_max - 1) / item_max;
-  const int64_t tot = (int64_t)nchunk * nsplit;
+  const int32_t nseg = nsplit * nsub;
+  const int64_t tot = (int64_t)nchunk * nseg;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t c = (int32_t)(i / nsplit), s = (int32_t)(i % nsplit);
+    const int32_t c = (int32_t)(i / nseg), s = (int32_t)(i % nseg);
     Item it;
     it.t0 = c * item_max;
     const int32_t tn = min(item_max, nt - it.t0);
@@ -412,7 +413,15 @@ __global__ void k_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t i
     items[i] = it;
   }
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g <= nsplit) range_ptr[g] = (ns * g) / nsplit;
+  if (g <= nseg) {  // part k of split s, at whole groups of kSumGroup sources
+    const int64_t s = g / nsub, k = g % nsub, b = (ns * s) / nsplit;
+    if (k == 0) {
+      range_ptr[g] = b;
+    } else {
+      const int64_t ng = ((ns * (s + 1)) / nsplit - b + kSumGroup - 1) / kSumGroup;
+      range_ptr[g] = b + ng * k / nsub * kSumGroup;
+    }
+  }
   if (g == 0) *n_items = (int32_t)tot;
 }
 
@@ -611,11 +620,12 @@ void launch_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *total, cud
   count_launches(1);
 }
 
-void launch_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t item_max, Item *items,
-                         int64_t *range_ptr, int32_t *n_items, cudaStream_t st) {
-  const int64_t tot = (int64_t)((nt + item_max - 1) / item_max) * nsplit;
-  const int64_t need = tot > nsplit + 1 ? tot : nsplit + 1;
-  k_items_direct<<<grid_for(need, 256), 256, 0, st>>>(nt, ns, nsplit, item_max, items, range_ptr,
+void launch_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t nsub, int32_t item_max,
+                         Item *items, int64_t *range_ptr, int32_t *n_items, cudaStream_t st) {
+  const int64_t nseg = (int64_t)nsplit * nsub;
+  const int64_t tot = (int64_t)((nt + item_max - 1) / item_max) * nseg;
+  const int64_t need = tot > nseg + 1 ? tot : nseg + 1;
+  k_items_direct<<<grid_for(need, 256), 256, 0, st>>>(nt, ns, nsplit, nsub, item_max, items, range_ptr,
                                                       n_items);
   count_launches(1);
 }

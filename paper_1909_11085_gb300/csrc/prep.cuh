@@ -37,8 +37,9 @@ void launch_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *total, cud
 size_t radix_hist_entries(int64_t n);
 int radix_sort(uint64_t *ka, int32_t *va, uint64_t *kb, int32_t *vb, int64_t n, int bits,
                int32_t *hist, int32_t *hist_scan, cudaStream_t st);
-void launch_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t item_max, Item *items,
-                         int64_t *range_ptr, int32_t *n_items, cudaStream_t st);
+// nsplit equal ranges of the sources, each in nsub parts of whole groups of kSumGroup.
+void launch_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t nsub, int32_t item_max,
+                         Item *items, int64_t *range_ptr, int32_t *n_items, cudaStream_t st);
 void launch_p2p_items(int32_t nleaf, const int32_t *leaf_ptr, const int32_t *ulist_ptr,
                       const int32_t *ulist_idx, int32_t item_max, int32_t *cnt, int32_t *offs,
                       int32_t *n_items, Item *items, uint64_t *keys, int32_t *vals,
@@ -104,7 +105,8 @@ void launch_adj_finish(bool src_major, int64_t n, int32_t nsplit, const double *
 
 size_t engine_mixed_smem_bytes();
 cudaError_t launch_engine_mixed(const EngineParams &P, int grid, cudaStream_t stream);
-cudaError_t engine_mixed_occupancy(int *blocks_per_sm);
+// Resident CTAs per SM by kernel kind (0: kinds by segment).
+cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[4]);
 // Launches both FP64 engines (grids of resident CTAs); *F.state picks one.
 cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,
                                cudaStream_t stream);
