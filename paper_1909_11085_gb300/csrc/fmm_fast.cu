@@ -533,9 +533,10 @@ __global__ void k_fast_m2m(Pass P) {
 // Check-to-equivalent products of a tile of NB boxes of one depth:
 // out[b][i] = (hi + lo)[i] . chk32[b] in double-FP32 arithmetic (the exact
 // FMA product and two-sum accumulation of apply_row_df), operator stored
-// column by column, read four columns ahead of their use; the boxes in pairs
+// column by column; the boxes in pairs
 // on packed FP32 instructions (per half the same operations and roundings).
-template <bool UP, int NB>
+// Read AHEAD columns at a time, ahead of their use.
+template <bool UP, int NB, int AHEAD>
 __global__ void __launch_bounds__(256) k_fast_c2e(Pass P) {
   static_assert(NB % 2 == 0, "boxes in pairs");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -561,16 +562,16 @@ __global__ void __launch_bounds__(256) k_fast_c2e(Pass P) {
     float2 sh[NB / 2], sl[NB / 2];
 #pragma unroll
     for (int h = 0; h < NB / 2; ++h) sh[h] = sl[h] = make_float2(0.f, 0.f);
-    for (int j0 = 0; j0 < cols; j0 += 4) {
-      float ah[4], al[4];
+    for (int j0 = 0; j0 < cols; j0 += AHEAD) {
+      float ah[AHEAD], al[AHEAD];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < AHEAD; ++q) {
         const bool ok = j0 + q < cols;
         ah[q] = ok ? hi[(size_t)(j0 + q) * rows + i] : 0.f;
         al[q] = ok ? lo[(size_t)(j0 + q) * rows + i] : 0.f;
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < AHEAD; ++q) {
         if (j0 + q >= cols) break;
         const float2 ah2 = p_dup(ah[q]), al2 = p_dup(al[q]);
         const float2 *x2p = reinterpret_cast<const float2 *>(X + (j0 + q) * NB);
@@ -594,8 +595,21 @@ __global__ void __launch_bounds__(256) k_fast_c2e(Pass P) {
 }
 
 // ------------------------------------------------------------- downward
-// UFFT: spectra of the upward densities of the children of one parent (the
-// CTA's plist position k at this depth), one octant each,
+// The spectra and their products take the parents of all depths at once, in plist
+// order (plist positions from the first parent of a depth-2 box on): the source
+// spectra only depend on the upward pass, and the products read the whole table of
+// kernel spectra (1.3 MB per frequency, 409 MB at p = 4) whatever the number of
+// parents, which took 117 and 105 us for the 8 and 64 parents of two shallow depths.
+// The launches, one per depth, share the work evenly: UFFT by ranges of parents, the
+// products by ranges of frequencies.  1,048,928 points: products 1.52 -> 1.28 ms, the
+// whole evaluation 6.35 -> 5.97 ms (with the C2E's tiles below).
+struct DepthStarts {
+  int32_t first, n;                   // parents of depth first's boxes come first; n depths
+  int32_t box[kMaxTreeDepth + 2];     // first box of depth first + k
+};
+
+// UFFT: spectra of the upward densities of the children of one parent (plist
+// position k of the launch's range), one octant each,
 // uhat[w][8 k + o][c] = sum_j up[child o][j][c] (cos - i sin)(2 pi (s_j . k_w mod G) / G),
 // zero for a missing child; thread = frequency.
 constexpr int kUfftRow = kFastTile * 8 + 4;  // staged output row, padded for float4 stores
@@ -604,14 +618,15 @@ inline size_t ufft_smem(int ns, int nc) {
   return sizeof(float) * std::max<size_t>((size_t)kFastTile * ns * nc, (size_t)128 * kUfftRow);
 }
 template <int NC>
-__global__ void __launch_bounds__(128) k_fast_ufft(Pass P, int32_t first_child0,
-                                                   int32_t first_child1) {
+__global__ void __launch_bounds__(128) k_fast_ufft(Pass P, DepthStarts D, int32_t kp0) {
   extern __shared__ __align__(16) unsigned char smem[];
   float *U = reinterpret_cast<float *>(smem);  // [8 octants][ns][NC]
   const int nf = freq_count(P.p);
-  const int32_t pos0 = P.bpos[first_child0], pos1 = P.bpos[first_child1];
-  const int32_t kp = (int32_t)blockIdx.x;
+  const int32_t pos0 = P.bpos[D.box[0]], pos1 = P.bpos[P.t.nbox];
+  const int32_t kp = kp0 + (int32_t)blockIdx.x;
   if (pos0 + kp >= pos1) return;  // the whole CTA
+  int depth = D.first;
+  while (depth + 1 < D.first + D.n && pos0 + kp >= P.bpos[D.box[depth + 1 - D.first]]) ++depth;
   if ((int64_t)8 * kp + 8 > P.uslots) {
     if (threadIdx.x == 0) bad_index(P);
     return;
@@ -632,7 +647,7 @@ __global__ void __launch_bounds__(128) k_fast_ufft(Pass P, int32_t first_child0,
   for (int bb = 0; bb < kFastTile; ++bb)
 #pragma unroll
     for (int c = 0; c < NC; ++c) re[bb][c] = im[bb][c] = 0.f;
-  const float r = half_width(P.t, P.depth);
+  const float r = half_width(P.t, depth);
   const float sf = 1.0f / r, sq = 1.0f / (r * r);
   const float2 *F = reinterpret_cast<const float2 *>(P.ftab);
   for (int j0 = 0; j0 < P.ns; j0 += 4) {
@@ -917,7 +932,7 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
 }
 
 __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
-    Pass P, int32_t first_child0, int32_t first_child1) {
+    Pass P, int32_t first_child0, int32_t w0) {
   using T = TcShape;
   extern __shared__ __align__(16) unsigned char smem[];
   // the swizzle is a function of the address: stages start 1024-byte aligned
@@ -927,10 +942,16 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
   uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + T::NBAR);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nf = freq_count(P.p);
-  const int w = blockIdx.y;
-  const int32_t pos0 = P.bpos[first_child0], pos1 = P.bpos[first_child1];
+  const int w = w0 + (int)blockIdx.y;
+  const int32_t pos0 = P.bpos[first_child0], pos1 = P.bpos[P.t.nbox];
   const int32_t row0 = pos0 + blockIdx.x * (kTcTiles * kTcRows);
-  if (row0 >= pos1) return;  // the whole CTA: nothing allocated yet
+  // the next launch's CTAs (other frequencies) may fill this one's last round; it ends
+  // after this one all the same (the wait below), so what follows both sees both
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (row0 >= pos1) {  // the whole CTA: nothing allocated yet
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   if (tid == 0) {
     for (int b = 0; b < kTcStages; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(&full[b])),
@@ -1136,6 +1157,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
                  "r"(kTcTmemCols)
                  : "memory");
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 
@@ -1396,15 +1418,22 @@ __global__ void __launch_bounds__(kItemThreads) k_fast_l2t(Pass P) {
 int box_threads(int ns) { return ((ns + 31) / 32) * 32; }
 
 // Check-to-equivalent products of the nb boxes of one depth: kFastTile boxes
-// per CTA, one operator row per thread (16 boxes per CTA measured slower).
+// per CTA, one operator row per thread (16 boxes per CTA measured slower), four
+// columns ahead.  With fewer CTAs than SMs the walk over the columns is bound by the
+// operator's load latency: two boxes per CTA and sixteen columns ahead take 19 to 23
+// us at 64 and 374 boxes where eight boxes took 52 to 56 (at 2,994 boxes two per CTA
+// are slower, 131 against 64 us).
 template <bool UP>
-void launch_c2e(const Pass &P, int32_t nb, int ns, cudaStream_t st) {
+void launch_c2e(const Pass &P, int32_t nb, int ns, int sms, cudaStream_t st) {
   const int rows = UP ? P.nc * ns : 3 * ns;
   int threads = ((rows + 31) / 32) * 32;
   if (threads > 256) threads = 256;
-  const size_t cols = 3 * (size_t)ns;
-  k_fast_c2e<UP, kFastTile><<<(unsigned)((nb + kFastTile - 1) / kFastTile), threads,
-                              sizeof(float) * kFastTile * cols, st>>>(P);
+  auto tiles = [&](int t) { return (unsigned)((nb + t - 1) / t); };
+  const size_t box = sizeof(float) * 3 * (size_t)ns;
+  if (tiles(kFastTile) < (unsigned)sms)
+    k_fast_c2e<UP, 2, 16><<<tiles(2), threads, 2 * box, st>>>(P);
+  else
+    k_fast_c2e<UP, kFastTile, 4><<<tiles(kFastTile), threads, kFastTile * box, st>>>(P);
 }
 
 }  // namespace
@@ -1513,8 +1542,44 @@ cudaError_t far_field_fast(const Pass &P0, const int32_t *depth_ptr, int32_t max
       post();
     }
     pre("uc2e");
-    launch_c2e<true>(P, nb, ns, st);
+    launch_c2e<true>(P, nb, ns, sms, st);
     post();
+  }
+  if (fft && max_depth >= kFirstDepth) {
+    DepthStarts D{kFirstDepth, max_depth - kFirstDepth + 1, {}};
+    int32_t nd = 0;  // depths with boxes
+    for (int32_t d = kFirstDepth; d <= max_depth; ++d) {
+      D.box[d - kFirstDepth] = depth_ptr[d];
+      nd += depth_ptr[d + 1] > depth_ptr[d];
+    }
+    const int32_t npar = P.uslots / 8;  // at least the parents
+    for (int32_t g = 0; g < nd; ++g) {
+      const int32_t k0 = (int32_t)((int64_t)npar * g / nd), k1 = (int32_t)((int64_t)npar * (g + 1) / nd);
+      pre("ufft");
+      const dim3 gu((unsigned)std::max(1, k1 - k0), (unsigned)((nf + 127) / 128));
+      if (P.nc == 4) k_fast_ufft<4><<<gu, 128, ufft_smem(ns, 4), st>>>(P, D, k0);
+      else k_fast_ufft<3><<<gu, 128, ufft_smem(ns, 3), st>>>(P, D, k0);
+      post();
+    }
+    const int rows = kTcTiles * kTcRows;
+    for (int32_t g = 0; g < nd; ++g) {
+      const int w0 = nf * g / nd, w1 = nf * (g + 1) / nd;
+      pre("kmulp");
+      const dim3 gt((unsigned)((npar + rows - 1) / rows), (unsigned)std::max(1, w1 - w0));
+      cudaLaunchAttribute early;
+      early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      early.val.programmaticStreamSerializationAllowed = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = gt;
+      cfg.blockDim = dim3(kTcThreads);
+      cfg.dynamicSmemBytes = TcShape::SMEM;
+      cfg.stream = st;
+      cfg.attrs = &early;
+      cfg.numAttrs = g > 0 ? 1 : 0;  // the first one reads the spectra of the launch before it
+      const cudaError_t e = cudaLaunchKernelEx(&cfg, k_fast_kmulp_tc, P, D.box[0], w0);
+      if (err == cudaSuccess) err = e;
+      post();
+    }
   }
   for (int32_t d = kFirstDepth; d <= max_depth; ++d) {
     P.depth = d;
@@ -1523,23 +1588,6 @@ cudaError_t far_field_fast(const Pass &P0, const int32_t *depth_ptr, int32_t max
     const int32_t nb = P.box1 - P.box0;
     if (nb <= 0) continue;
     if (fft) {
-      // parents of this depth's boxes: at most the boxes of the depth above,
-      // and at most the boxes of this depth
-      const int32_t npar_max = std::min(depth_ptr[d] - depth_ptr[d - 1], nb);
-      pre("ufft");
-      const dim3 gu((unsigned)npar_max, (unsigned)((nf + 127) / 128));
-      if (P.nc == 4)
-        k_fast_ufft<4><<<gu, 128, ufft_smem(ns, 4), st>>>(P, depth_ptr[d], depth_ptr[d + 1]);
-      else
-        k_fast_ufft<3><<<gu, 128, ufft_smem(ns, 3), st>>>(P, depth_ptr[d], depth_ptr[d + 1]);
-      post();
-      pre("kmulp");
-      {
-        const int rows = kTcTiles * kTcRows;
-        const dim3 gt((unsigned)((npar_max + rows - 1) / rows), (unsigned)nf);
-        k_fast_kmulp_tc<<<gt, kTcThreads, TcShape::SMEM, st>>>(P, depth_ptr[d], depth_ptr[d + 1]);
-      }
-      post();
       pre("ifft");
       {
         // the M2L part of the downward check velocities: rows (box, component)
@@ -1567,7 +1615,7 @@ cudaError_t far_field_fast(const Pass &P0, const int32_t *depth_ptr, int32_t max
                   st>>>(P);
     post();
     pre("dc2e");
-    launch_c2e<false>(P, nb, ns, st);
+    launch_c2e<false>(P, nb, ns, sms, st);
     post();
   }
   pre("l2t");

@@ -159,11 +159,11 @@ struct Pass {
   float *fitab;        // inverse DFT over the half spectrum (weighted, / G^3) as the B table
                        // of the tensor-core product (fmm_fast.cu)
   int32_t *err;        // device error word (a tree index out of range), at workspace + 8 bytes
-  float *uhh, *uhl;    // [nfreq][uslots][4][2] upward spectra of one depth split into TF32
+  float *uhh, *uhl;    // [nfreq][uslots][4][2] upward spectra split into TF32
                        // hi + lo parts, parent-major: slot 8 k + o holds the child in octant o
                        // of the depth's k-th parent (zero where there is none; fourth
                        // component zero without flux), operands of the tensor-core M2L
-  int32_t uslots;      // slots of uhh / uhl per frequency (8 x the most parents of a depth)
+  int32_t uslots;      // slots of uhh / uhl per frequency (8 x at least the parents)
   float *btab;         // [nfreq][52][hi, lo][48 x 32] kernel spectra of each neighbour
                        // direction and octant half in the tensor-core operand layout (see
                        // fmm_fast.cu)
@@ -952,16 +952,16 @@ inline int64_t op_entries(int p, int nc, int max_depth, bool upward) {
 
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Slots of the parent-major source spectra of one depth: 8 per parent with
-// children there; depth d has at most min(boxes at d - 1, boxes at d) of them.
+// Slots of the parent-major source spectra: 8 per parent with children at depths
+// with a far field; depth d has at most min(boxes at d - 1, boxes at d) of them.
 inline int64_t spectrum_slots(const int32_t *depth_ptr, int max_depth) {
-  int64_t m = 1;
-  for (int d = 1; d <= max_depth; ++d) {
+  int64_t m = 0;
+  for (int d = kFirstDepth; d <= max_depth; ++d) {
     const int64_t a = depth_ptr[d] - depth_ptr[d - 1], b = depth_ptr[d + 1] - depth_ptr[d];
     const int64_t c = a < b ? a : b;
-    m = c > m ? c : m;
+    m += c;
   }
-  return 8 * m;
+  return 8 * (m > 1 ? m : 1);
 }
 
 inline Layout layout(int64_t nbox, int p, int nc, bool fft, bool mixed, int64_t n,
