@@ -669,8 +669,7 @@ __global__ void __launch_bounds__(128) k_fast_ufft(Pass P, DepthStarts D, int32_
         }
     }
   }
-  // the tensor-core products read the spectra as TF32 hi + lo parts, four
-  // components per child and frequency (the fourth zero without flux); at one
+  // four components per child and frequency (the fourth zero without flux); at one
   // frequency a parent's 8 children are 256 contiguous bytes, the unit its
   // neighbours gather.  The [w][8][8] block is staged in shared memory and
   // written out as one contiguous run per frequency
@@ -680,38 +679,33 @@ __global__ void __launch_bounds__(128) k_fast_ufft(Pass P, DepthStarts D, int32_
   const int w0 = blockIdx.y * blockDim.x;
   const int nw = min((int)blockDim.x, nf - w0);
   constexpr int per_w = kFastTile * 2;  // float4 per frequency
-  for (int half = 0; half < 2; ++half) {
-    __syncthreads();
-    if (active) {
+  __syncthreads();
+  if (active) {
 #pragma unroll
-      for (int bb = 0; bb < kFastTile; ++bb)
+    for (int bb = 0; bb < kFastTile; ++bb)
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          float v[4];
+      for (int q = 0; q < 2; ++q) {
+        float v[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            // component c = 2q + k/2, real part for even k; scaled to the depth:
-            // the kernel spectra are those of half-width 1, the Stokeslet
-            // homogeneous of degree -1, the source of degree -2
-            const int c = 2 * q + (k >> 1);
-            const float x = c < NC ? (c < 3 ? sf : sq) * ((k & 1) ? im[bb][c < NC ? c : 0]
-                                                                  : re[bb][c < NC ? c : 0])
-                                   : 0.f;
-            const float h = tf32_rna(x);
-            v[k] = half ? tf32_rna(x - h) : h;
-          }
-          *reinterpret_cast<float4 *>(&S[wl * kRow + bb * 8 + 4 * q]) =
-              make_float4(v[0], v[1], v[2], v[3]);
+        for (int k = 0; k < 4; ++k) {
+          // component c = 2q + k/2, real part for even k; scaled to the depth:
+          // the kernel spectra are those of half-width 1, the Stokeslet
+          // homogeneous of degree -1, the source of degree -2
+          const int c = 2 * q + (k >> 1);
+          v[k] = c < NC ? (c < 3 ? sf : sq) * ((k & 1) ? im[bb][c < NC ? c : 0]
+                                                       : re[bb][c < NC ? c : 0])
+                        : 0.f;
         }
-    }
-    __syncthreads();
-    float *dst = half ? P.uhl : P.uhh;
-    for (int e = threadIdx.x; e < nw * per_w; e += blockDim.x) {
-      const int ww = e / per_w, q = e % per_w;
-      const float4 v = *reinterpret_cast<const float4 *>(&S[ww * kRow + 4 * q]);
-      *reinterpret_cast<float4 *>(dst + ((size_t)(w0 + ww) * P.uslots + 8 * (size_t)kp) * 8 +
-                                  4 * q) = v;
-    }
+        *reinterpret_cast<float4 *>(&S[wl * kRow + bb * 8 + 4 * q]) =
+            make_float4(v[0], v[1], v[2], v[3]);
+      }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nw * per_w; e += blockDim.x) {
+    const int ww = e / per_w, q = e % per_w;
+    const float4 v = *reinterpret_cast<const float4 *>(&S[ww * kRow + 4 * q]);
+    *reinterpret_cast<float4 *>(P.uh + ((size_t)(w0 + ww) * P.uslots + 8 * (size_t)kp) * 8 +
+                                4 * q) = v;
   }
 }
 
@@ -746,22 +740,6 @@ __global__ void k_fast_vpar(Pass P) {
   }
 }
 
-__device__ __forceinline__ void cp_async_zfill(void *dst, const void *src, bool valid, int bytes) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  const int sz = valid ? bytes : 0;
-  if (bytes == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(sz)
-                 : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(sz)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // ----------------------------------------------------------------------
 // The spectral products on the tensor cores (tcgen05, kind::tf32).  For one
 // frequency w the products of a parent P are one dense complex contraction:
@@ -776,10 +754,10 @@ __device__ __forceinline__ void cp_async_wait() {
 // so that hi.hi + hi.lo + lo.hi carries FP32 accuracy (the lo.lo term is below
 // it).  The K dimension runs in 52 chunks of 32 (one neighbour direction,
 // four of its children's octants), 128 contiguous bytes per parent row in the
-// parent-major spectra; a chunk is staged in shared memory in the MMA's
+// parent-major spectra; a chunk's B is staged in shared memory in the MMA's
 // K-major layout with the 128-byte swizzle (a row's 128 bytes in one line,
-// its 16-byte pieces permuted by the row index within each 8-row group).
-constexpr int kTcThreads = 256;
+// its 16-byte pieces permuted by the row index within each 8-row group), its A
+// in tensor memory, a parent per lane.
 constexpr int kTcRows = 128;
 constexpr int kTcCols = 48;        // 8 targets x 3 components x (re, im)
 constexpr int kTcK = 32;           // K per chunk (128 bytes of TF32)
@@ -817,12 +795,13 @@ __device__ __forceinline__ uint64_t tc_sdesc_sw128(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) |
          ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-__device__ __forceinline__ void tc_mma(uint32_t dt, uint64_t a, uint64_t b, uint32_t idesc,
+// D (tensor memory) += A (tensor memory, K along the columns) B (shared memory)
+__device__ __forceinline__ void tc_mma(uint32_t dt, uint32_t a, uint64_t b, uint32_t idesc,
                                        uint32_t accum) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
-      "l"(a), "l"(b), "r"(idesc), "r"(accum)
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(dt),
+      "r"(a), "l"(b), "r"(idesc), "r"(accum)
       : "memory");
 }
 // Byte offset of element (row, k), k < 32, in a K-major tile with the 128-byte
@@ -833,37 +812,49 @@ __host__ __device__ __forceinline__ uint32_t sw128_off(int row, int k) {
                     ((k & 3) << 2));
 }
 
-// Per CTA: one frequency and kTcTiles tiles of 128 parents.  Warp roles:
-//   warps 0-3 (producers): for each chunk, copy the TF32 hi/lo spectra of the
-//     4 octants of their rows' neighbour by cp.async into the swizzled MMA
-//     layout (8 lanes per row: one 128-byte line per row; zero-filled where the
-//     neighbour has no children) and the chunk's B from the table k_fast_btab
-//     built for the call; once a chunk's copies have landed, fence them for the
-//     tensor core and arrive on the chunk's "full" barrier;
-//   thread 128 (MMA): wait "full", issue 4 K-steps x 2 MMAs per tile, commit
-//     to the chunk's "empty" barrier (producers refill a buffer only after it);
-//   warps 4-7 (epilogue): after the final commit, read the accumulators from
+// Per CTA: one frequency and a tile of 128 parents.  Roles:
+//   warps 0-3 and 4-7 (producers), a parent's row per thread, one group for the chunks
+//     of each octant half: copy the spectra of the 4 octants of the rows' neighbour by
+//     cp.async into the group's ring in shared memory (8 lanes per row: one 128-byte
+//     line; zero-filled where the neighbour has no children), read the own row back,
+//     split it into TF32 hi + lo, store both to the group's operand in tensor memory,
+//     from where the MMA reads A, and arrive on its "full" barrier;
+//   thread 288 (B): the chunk's B from the table k_fast_btab built for the call, by
+//     bulk copies completing on the chunk's barrier;
+//   thread 256 (MMA): wait for both, issue 4 K-steps x 2 MMAs, commit to the chunk's
+//     "empty" barriers (a buffer is refilled only after it);
+//   warps 8-11 (epilogue): after the final commit, read the accumulators from
 //     tensor memory (one lane quarter each) and write the check spectra.
-// A ring of kTcStages buffers lets the producers run ahead of the MMAs.
 // Every wait is bounded; on expiry the role records STK_ETIMEOUT in the error
 // word and stops, and the CTA still drains its copies and MMAs before it
 // frees tensor memory.
-constexpr int kTcTiles = 1;
-constexpr int kTcStages = 2;
-constexpr int kTcAhead = 1;  // chunks of copies a producer keeps in flight (< kTcStages)
-constexpr int kTcMinBlocks = 2;  // 2 x 90 KB: one CTA's set-up and epilogue overlap the other's loop
-// per tile 96 accumulator columns: [0, 48) hi.hi + lo.hi, [48, 96) hi.lo (summed at the end)
-constexpr uint32_t kTcTmemCols = kTcTiles == 1 ? 128 : 256;  // accumulators 128 columns apart
-constexpr int kTcProducers = 128;
+//
+// Bound: shared memory and the producers' instructions per chunk.  With A as TF32 hi
+// and lo parts in global and shared memory a chunk gathered 44 KB from L2 and moved
+// 94 KB through shared memory (32 + 12 written, 50 read); now 28 and 62 KB.
+// 1,048,928 points: 1.28 -> 1.00 ms; with one group of producers the split's
+// instructions were the bound (1.5 ms), and with hi and lo stored to shared memory by
+// eight warps it took the time it had.
+constexpr int kTcStages = 2;  // A operands in tensor memory, one per group
+constexpr int kTcRing = 2;    // chunks of spectra in shared memory per group
+constexpr int kTcBStages = 3;
+constexpr int kTcMinBlocks = 2;  // one CTA's set-up and epilogue overlap the other's loop
+// tensor memory: 96 accumulator columns, [0, 48) hi.hi + lo.hi, [48, 96) hi.lo (summed at
+// the end), and from kTcACol on kTcStages operands of kTcK columns hi and kTcK lo
+constexpr uint32_t kTcACol = 128, kTcTmemCols = 256;
+static_assert(kTcACol + kTcStages * 2 * kTcK <= kTcTmemCols, "tensor memory");
+constexpr int kTcProducers = 2 * kTcRows;  // a thread per row and octant half
+constexpr int kTcThreads = kTcProducers + 128;
 struct TcShape {
-  static constexpr int ATILE = kTcRows * kTcK * 4;      // bytes of one A tile (hi or lo)
-  static constexpr int ASTAGE = kTcTiles * 2 * ATILE;   // hi, lo of every tile
+  static constexpr int ACHUNK = kTcRows * kTcK * 4;     // bytes of one chunk of spectra
   static constexpr int BTILE = kTcCols * kTcK * 4;      // 6 swizzle groups of 8 rows
-  static constexpr int STAGE = ASTAGE + 2 * BTILE;      // a multiple of 1024
-  static constexpr int NBAR = 2 * kTcStages + 1;        // full, empty, done
-  static constexpr size_t SMEM = 1024 + (size_t)kTcStages * STAGE + 8 * NBAR + 16;
+  static constexpr int BSTAGE = 2 * BTILE;              // hi, lo
+  static constexpr int NBAR = 2 * kTcStages + 2 * kTcBStages + 1;  // full, empty of A, of B; done
+  static constexpr size_t SMEM =
+      1024 + (size_t)2 * kTcRing * ACHUNK + (size_t)kTcBStages * BSTAGE + 8 * NBAR + 16;
 };
-static_assert(TcShape::STAGE % 1024 == 0, "swizzle groups stay 1024-byte aligned");
+static_assert(TcShape::ACHUNK % 1024 == 0 && TcShape::BTILE % 1024 == 0,
+              "swizzle groups stay 1024-byte aligned");
 static_assert(kTcChunks % 2 == 0, "two octant halves per direction");
 
 // The B operand of every (frequency, chunk): for direction dd, octant half h
@@ -931,20 +922,44 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                : "memory");
 }
 
+// 16 columns of the thread's tensor memory lane
+__device__ __forceinline__ void tc_store16(uint32_t taddr, const uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+      "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void cp_async_zfill16(void *dst, const void *src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr(dst)), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
     Pass P, int32_t first_child0, int32_t w0) {
   using T = TcShape;
   extern __shared__ __align__(16) unsigned char smem[];
   // the swizzle is a function of the address: stages start 1024-byte aligned
-  unsigned char *stages = smem + ((1024u - (saddr(smem) & 1023u)) & 1023u);  // [kTcStages][STAGE]
-  uint64_t *bars = reinterpret_cast<uint64_t *>(stages + kTcStages * T::STAGE);
-  uint64_t *full = bars, *empty = bars + kTcStages, *done = bars + 2 * kTcStages;
+  unsigned char *As = smem + ((1024u - (saddr(smem) & 1023u)) & 1023u);  // [2][kTcRing][ACHUNK]
+  unsigned char *Bs = As + 2 * kTcRing * T::ACHUNK;                      // [kTcBStages][BSTAGE]
+  uint64_t *bars = reinterpret_cast<uint64_t *>(Bs + kTcBStages * T::BSTAGE);
+  uint64_t *full = bars, *empty = full + kTcStages, *fullb = empty + kTcStages,
+           *emptyb = fullb + kTcBStages, *done = emptyb + kTcBStages;
   uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + T::NBAR);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nf = freq_count(P.p);
   const int w = w0 + (int)blockIdx.y;
   const int32_t pos0 = P.bpos[first_child0], pos1 = P.bpos[P.t.nbox];
-  const int32_t row0 = pos0 + blockIdx.x * (kTcTiles * kTcRows);
+  const int32_t row0 = pos0 + blockIdx.x * kTcRows;
   // the next launch's CTAs (other frequencies) may fill this one's last round; it ends
   // after this one all the same (the wait below), so what follows both sees both
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -953,13 +968,19 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
     return;
   }
   if (tid == 0) {
-    for (int b = 0; b < kTcStages; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(&full[b])),
-                   "r"(kTcProducers)
+    auto init = [](uint64_t *bar, int count) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(bar)), "r"(count)
                    : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&empty[b])) : "memory");
+    };
+    for (int b = 0; b < kTcStages; ++b) {
+      init(&full[b], kTcRows);
+      init(&empty[b], 1);
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(done)) : "memory");
+    for (int b = 0; b < kTcBStages; ++b) {
+      init(&fullb[b], 1);
+      init(&emptyb[b], 1);
+    }
+    init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -976,83 +997,111 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
   const int32_t nbox = P.t.nbox;
   bool ok = true;
 
-  if (warp < 4) {
+  if (warp < kTcProducers / 32) {
     // ---------------------------------------------------------- producers
-    // warp pw copies rows 32 pw .. 32 pw + 31 of every tile; lane holds the
-    // neighbour's local plist position for row 32 pw + lane, and in a copy
-    // round 8 lanes take one row (lane / 8) and its 16-byte pieces (lane % 8)
-    const unsigned char *UHH = reinterpret_cast<const unsigned char *>(P.uhh);
-    const unsigned char *UHL = reinterpret_cast<const unsigned char *>(P.uhl);
+    // group pg = warp / 4 takes the chunks of octant half pg, one per direction, into
+    // its own ring and its own operand in tensor memory; warp pw of it copies rows 32 pw
+    // .. 32 pw + 31; lane holds the neighbour's local plist position for row 32 pw +
+    // lane, and in a round 8 lanes take one row (lane / 8) and its 16-byte pieces
+    constexpr int kDirs = kTcChunks / 2;
+    const int pg = warp >> 2, pw = warp & 3;
+    const unsigned char *UH = reinterpret_cast<const unsigned char *>(P.uh) + 128 * pg;
+    unsigned char *ring = As + (size_t)pg * kTcRing * T::ACHUNK;
     const int32_t npar = min(pos1 - pos0, P.uslots / 8);
     const size_t wrow = (size_t)w * P.uslots;  // first slot of this frequency
-    int32_t rowi[kTcTiles];
+    const int32_t rowi = row0 + 32 * pw + lane;
+    auto load_q = [&](int dd) {
+      int32_t v = dd < kDirs && rowi < pos1 ? P.vpar[(size_t)dd * nbox + rowi] : -1;
+      if (v >= 0) {
+        v -= pos0;
+        if (v < 0 || v >= npar) {
+          bad_index(P);
+          v = -1;
+        }
+      }
+      return v;
+    };
+    const int rsub = lane >> 3, piece = lane & 7;
+    auto copy = [&](int dd, int32_t q) {  // one commit group
+      unsigned char *dst = ring + (size_t)(dd % kTcRing) * T::ACHUNK;
+      if (dd < kDirs)
 #pragma unroll
-    for (int k = 0; k < kTcTiles; ++k) rowi[k] = row0 + k * kTcRows + 32 * warp + lane;
-    // neighbour positions of the next direction are loaded while the current
-    // one is copied
-    auto load_q = [&](int dd, int32_t *q) {
+        for (int i = 0; i < 8; ++i) {
+          const int32_t lq = __shfl_sync(kFull, q, 4 * i + rsub);
+          const size_t go = lq >= 0 ? (wrow + 8 * (size_t)lq) * 32 + 16 * piece : 0;
+          cp_async_zfill16(dst + sw128_off(32 * pw + 4 * i + rsub, 4 * piece), UH + go, lq >= 0);
+        }
+      cp_async_commit();
+    };
+    int32_t q = load_q(0);
+    for (int dd = 0; dd < kTcRing - 1; ++dd) {
+      const int32_t qn = load_q(dd + 1);
+      copy(dd, q);
+      q = qn;
+    }
+    const uint32_t arow =
+        tmem + ((uint32_t)(32 * pw) << 16) + kTcACol + (uint32_t)(pg * 2 * kTcK);
+    for (int dd = 0; dd < kDirs; ++dd) {
+      // the buffer of direction dd + kTcRing - 1 is the one this warp read last
+      const int32_t qn = load_q(dd + kTcRing);
+      copy(dd + kTcRing - 1, q);
+      q = qn;
+      cp_async_wait<kTcRing - 1>();
+      __syncwarp();
+      bool go = true;
+      if (dd > 0) go = tc_wait(&empty[pg], (uint32_t)((dd - 1) & 1));
+      if (!__all_sync(kFull, go)) {
+        if (lane == 0 && P.err) atomicCAS(P.err, 0, kErrTimeout);
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const unsigned char *src = ring + (size_t)(dd % kTcRing) * T::ACHUNK;
 #pragma unroll
-      for (int k = 0; k < kTcTiles; ++k) {
-        int32_t v = rowi[k] < pos1 ? P.vpar[(size_t)dd * nbox + rowi[k]] : -1;
-        if (v >= 0) {
-          v -= pos0;
-          if (v < 0 || v >= npar) {
-            bad_index(P);
-            v = -1;
+      for (int c = 0; c < kTcK; c += 16) {
+        uint32_t h[16], l[16];
+#pragma unroll
+        for (int e = 0; e < 16; e += 4) {
+          const float4 x = *reinterpret_cast<const float4 *>(src + sw128_off(32 * pw + lane, c + e));
+          const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float hi = tf32_rna(xs[k]);
+            h[e + k] = __float_as_uint(hi);
+            l[e + k] = __float_as_uint(tf32_rna(xs[k] - hi));
           }
         }
-        q[k] = v;
+        tc_store16(arow + (uint32_t)c, h);
+        tc_store16(arow + (uint32_t)(kTcK + c), l);
       }
-    };
-    int32_t qcur[kTcTiles], qnext[kTcTiles];
-    load_q(0, qcur);
-    const int rsub = lane >> 3, piece = lane & 7;
-    for (int g = 0; g < kTcChunks && ok; ++g) {
-      const int s = g % kTcStages, dd = g >> 1, half = g & 1;
-      if (half == 0 && dd + 1 < kTcChunks / 2) load_q(dd + 1, qnext);
-      if (g >= kTcStages && !tc_wait(&empty[s], (uint32_t)(((g / kTcStages) - 1) & 1))) {
-        ok = false;
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      tc_arrive(&full[pg]);
+      __syncwarp();  // every lane has read its row: the next copy may overwrite it
+    }
+    cp_async_wait<0>();
+  } else if (tid == kTcProducers + 32) {
+    // ------------------------------------------------------------------ B
+    int g = 0;
+    for (; g < kTcChunks; ++g) {
+      const int b = g % kTcBStages;
+      if (g >= kTcBStages && !tc_wait(&emptyb[b], (uint32_t)(((g / kTcBStages) - 1) & 1))) {
         if (P.err) atomicCAS(P.err, 0, kErrTimeout);
         break;
       }
-      unsigned char *st = stages + (size_t)s * T::STAGE;
-#pragma unroll
-      for (int k = 0; k < kTcTiles; ++k) {
-        unsigned char *ah = st + (size_t)k * 2 * T::ATILE, *al = ah + T::ATILE;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int rw = 4 * i + rsub;            // row within the warp's 32
-          const int32_t lq = __shfl_sync(kFull, qcur[k], rw);
-          const int r = 32 * warp + rw;            // row within the tile
-          const bool okc = lq >= 0;
-          const size_t go = okc ? ((wrow + 8 * (size_t)lq + 4 * half) * 32 + 16 * piece) : 0;
-          const uint32_t o = sw128_off(r, 4 * piece);
-          cp_async_zfill(ah + o, UHH + go, okc, 16);
-          cp_async_zfill(al + o, UHL + go, okc, 16);
-        }
-      }
-      {  // B: the chunk's kernel spectra, hi then lo, as laid out in the table
-        unsigned char *bdst = st + T::ASTAGE;
-        const unsigned char *bsrc = reinterpret_cast<const unsigned char *>(
-            P.btab + ((size_t)w * kTcChunks + g) * 2 * kTcCols * kTcK);
-        for (int e = tid; e < 2 * T::BTILE / 16; e += kTcProducers)
-          cp_async_zfill(bdst + 16 * e, bsrc + 16 * e, true, 16);
-      }
-      cp_async_commit();
-      if (g >= kTcAhead) {  // chunk g - kTcAhead: its copies have landed
-        cp_async_wait<kTcAhead>();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_arrive(&full[(g - kTcAhead) % kTcStages]);
-      }
-      if (half == 1)
-#pragma unroll
-        for (int k = 0; k < kTcTiles; ++k) qcur[k] = qnext[k];
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(&fullb[b])),
+                   "r"(T::BSTAGE)
+                   : "memory");
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+              "r"(saddr(Bs + (size_t)b * T::BSTAGE)),
+          "l"(P.btab + ((size_t)w * kTcChunks + g) * 2 * kTcCols * kTcK), "r"(T::BSTAGE),
+          "r"(saddr(&fullb[b]))
+          : "memory");
     }
-    cp_async_wait<0>();
-    if (ok) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      for (int c = kTcChunks - kTcAhead; c < kTcChunks; ++c) tc_arrive(&full[c % kTcStages]);
-    }
+    // every copy has landed before the CTA can end, whatever the other roles did
+    for (int c = max(0, g - kTcBStages); c < g; ++c)
+      if (!tc_wait(&fullb[c % kTcBStages], (uint32_t)((c / kTcBStages) & 1)))
+        if (P.err) atomicCAS(P.err, 0, kErrTimeout);
   } else if (tid == kTcProducers) {
     // ---------------------------------------------------------------- MMA
     // D F32, A and B TF32, K-major; N = 96 (B hi then B lo, adjacent in the
@@ -1065,28 +1114,25 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
     int last = -1;
     for (int g = 0; g < kTcChunks; ++g) {
       const int s = g % kTcStages;
-      if (!tc_wait(&full[s], (uint32_t)((g / kTcStages) & 1))) {
+      const int b = g % kTcBStages;
+      if (!tc_wait(&full[s], (uint32_t)((g / kTcStages) & 1)) ||
+          !tc_wait(&fullb[b], (uint32_t)((g / kTcBStages) & 1))) {
         ok = false;
         if (P.err) atomicCAS(P.err, 0, kErrTimeout);
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned char *st = stages + (size_t)s * T::STAGE;
-      const uint32_t bh = saddr(st + T::ASTAGE);
+      const uint32_t bh = saddr(Bs + (size_t)b * T::BSTAGE);
+      const uint32_t ah = tmem + kTcACol + (uint32_t)(s * 2 * kTcK);
 #pragma unroll
-      for (int tt = 0; tt < kTcTiles; ++tt) {
-        const uint32_t ah = saddr(st + (size_t)tt * 2 * T::ATILE), al = ah + T::ATILE;
-        const uint32_t d = tmem + (uint32_t)(tt * 128);
-#pragma unroll
-        for (int ks = 0; ks < kTcK / 8; ++ks) {
-          const uint32_t kb = 32u * ks;  // 8 TF32 per K-step
-          // [hi.hi | hi.lo] in one product of N = 96, then lo.hi into the first half
-          tc_mma(d, tc_sdesc_sw128(ah + kb), tc_sdesc_sw128(bh + kb), idesc96,
-                 (g > 0 || ks > 0) ? 1u : 0u);
-          tc_mma(d, tc_sdesc_sw128(al + kb), tc_sdesc_sw128(bh + kb), idesc48, 1u);
-        }
+      for (int ks = 0; ks < kTcK / 8; ++ks) {
+        const uint64_t bd = tc_sdesc_sw128(bh + 32u * ks);  // 8 TF32 per K-step
+        // [hi.hi | hi.lo] in one product of N = 96, then lo.hi into the first half
+        tc_mma(tmem, ah + 8u * ks, bd, idesc96, (g > 0 || ks > 0) ? 1u : 0u);
+        tc_mma(tmem, ah + kTcK + 8u * ks, bd, idesc48, 1u);
       }
       tc_commit(&empty[s]);
+      tc_commit(&emptyb[b]);
       last = g;
     }
     if (ok) {
@@ -1096,7 +1142,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
       if (P.err) atomicCAS(P.err, 0, kErrTimeout);
     }
   }
-  if (warp >= 4) {
+  if (warp >= kTcProducers / 32) {
     // ----------------------------------------------------------- epilogue
     __syncwarp();
     const bool fin = tc_wait(done, 0);
@@ -1104,15 +1150,14 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (__all_sync(kFull, fin)) {
       const int quarter = warp & 3;
-#pragma unroll 1
-      for (int tt = 0; tt < kTcTiles; ++tt) {
-        const int32_t i = row0 + tt * kTcRows + quarter * 32 + lane;
+      {
+        const int32_t i = row0 + quarter * 32 + lane;
         float d[kTcCols];
 #pragma unroll
         for (int part = 0; part < 2 * kTcCols / 16; ++part) {
           uint32_t v[16];
           const uint32_t taddr =
-              tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(tt * 128 + part * 16);
+              tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 16);
           asm volatile(
               "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
               "%10, %11, %12, %13, %14, %15}, [%16];"
@@ -1561,7 +1606,7 @@ cudaError_t far_field_fast(const Pass &P0, const int32_t *depth_ptr, int32_t max
       else k_fast_ufft<3><<<gu, 128, ufft_smem(ns, 3), st>>>(P, D, k0);
       post();
     }
-    const int rows = kTcTiles * kTcRows;
+    const int rows = kTcRows;
     for (int32_t g = 0; g < nd; ++g) {
       const int w0 = nf * g / nd, w1 = nf * (g + 1) / nd;
       pre("kmulp");

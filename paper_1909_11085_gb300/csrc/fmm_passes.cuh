@@ -159,11 +159,10 @@ struct Pass {
   float *fitab;        // inverse DFT over the half spectrum (weighted, / G^3) as the B table
                        // of the tensor-core product (fmm_fast.cu)
   int32_t *err;        // device error word (a tree index out of range), at workspace + 8 bytes
-  float *uhh, *uhl;    // [nfreq][uslots][4][2] upward spectra split into TF32
-                       // hi + lo parts, parent-major: slot 8 k + o holds the child in octant o
-                       // of the depth's k-th parent (zero where there is none; fourth
-                       // component zero without flux), operands of the tensor-core M2L
-  int32_t uslots;      // slots of uhh / uhl per frequency (8 x at least the parents)
+  float *uh;           // [nfreq][uslots][4][2] upward spectra, parent-major: slot 8 k + o
+                       // holds the child in octant o of the k-th parent (zero where
+                       // there is none; fourth component zero without flux), operands of the tensor-core M2L
+  int32_t uslots;      // slots of uh per frequency (8 x at least the parents)
   float *btab;         // [nfreq][52][hi, lo][48 x 32] kernel spectra of each neighbour
                        // direction and octant half in the tensor-core operand layout (see
                        // fmm_fast.cu)
@@ -937,7 +936,7 @@ struct Layout {
   size_t surf, chk, up, dn, sidx, tw, uhat, chat, m2l;
   size_t ploc, qf, pf, nf, surf32, up32, dn32, tw32, spec32, uhat32, chat32, m2l32;
   size_t chk32, ops_hi, ops_lo;
-  size_t child8, bflag, bpos, plist, ftab, fitab, vpar, uhh, uhl, btab;
+  size_t child8, bflag, bpos, plist, ftab, fitab, vpar, uh, btab;
   int64_t uslots;
   size_t icnt, ipb, ioff, items;
   size_t ktab, kexp, edens, eexp;
@@ -982,7 +981,7 @@ inline Layout layout(int64_t nbox, int p, int nc, bool fft, bool mixed, int64_t 
   L.chk = L.up = L.dn = L.tw = L.uhat = L.chat = L.m2l = none;
   L.ploc = L.qf = L.pf = L.nf = L.surf32 = L.up32 = L.dn32 = L.tw32 = L.spec32 = L.uhat32 =
       L.chat32 = L.m2l32 = L.chk32 = L.ops_hi = L.ops_lo = none;
-  L.child8 = L.bflag = L.bpos = L.plist = L.ftab = L.fitab = L.vpar = L.uhh = L.uhl = L.btab =
+  L.child8 = L.bflag = L.bpos = L.plist = L.ftab = L.fitab = L.vpar = L.uh = L.btab =
       none;
   L.uslots = spectrum_slots(depth_ptr, max_depth);
   L.icnt = L.ipb = L.ioff = L.items = none;
@@ -1026,8 +1025,7 @@ inline Layout layout(int64_t nbox, int p, int nc, bool fft, bool mixed, int64_t 
       L.fitab = take(sizeof(float) * 2 * 64 * 32 * (size_t)((ns + 63) / 64) *
                      ((2 * nf + 31) / 32));  // the inverse-DFT product's B table
       L.vpar = take(sizeof(int32_t) * 26 * B);
-      L.uhh = take(sizeof(float) * 8 * nf * (size_t)L.uslots);
-      L.uhl = take(sizeof(float) * 8 * nf * (size_t)L.uslots);
+      L.uh = take(sizeof(float) * 8 * nf * (size_t)L.uslots);
       L.btab = take(sizeof(float) * nf * 52 * 2 * 48 * 32);
     }
     L.child8 = take(sizeof(int32_t) * 8 * B);
@@ -1088,8 +1086,7 @@ inline void bind(Pass &P, char *ws, const Layout &L, bool fft, bool mixed) {
   P.fitab = (fft && mixed) ? f(L.fitab) : nullptr;
   P.vpar = (fft && mixed) ? i32(L.vpar) : nullptr;
   P.uslots = (int32_t)L.uslots;
-  P.uhh = (fft && mixed) ? f(L.uhh) : nullptr;
-  P.uhl = (fft && mixed) ? f(L.uhl) : nullptr;
+  P.uh = (fft && mixed) ? f(L.uh) : nullptr;
   P.btab = (fft && mixed) ? f(L.btab) : nullptr;
   P.icnt = mixed ? i32(L.icnt) : nullptr;
   P.ipb = mixed ? i32(L.ipb) : nullptr;
