@@ -198,12 +198,12 @@ __device__ __forceinline__ void eval_src_pairs_any(const Pass &P, const float4 *
 // entry a (first, second) pair; the positions already scaled by the radius
 // and in the target box's frame.
 constexpr int kEqFields = 4;
-// Adds the field of the staged pairs j0, j0 + js, ... < np at T targets:
+// Adds the field of the staged pairs j0, j0 + js, ... < np at the first T of two targets:
 // Stokeslet (e + d (d.e)/r^2)/r into uf, point source d e.w/r^3 into uq.
 template <bool FLUX, int T = 2>
 __device__ __forceinline__ void eval_eq_pairs(const float4 *E, int cap, int j0, int np, int js,
-                                              const float2 (&x)[T][3], float2 (&uf)[T][3],
-                                              float2 (&uq)[T][3]) {
+                                              const float2 (&x)[2][3], float2 (&uf)[2][3],
+                                              float2 (&uq)[2][3]) {
   for (int j = j0; j < np; j += js) {
     const float4 a = E[j], b = E[cap + j], c = E[2 * cap + j];
     const float2 nyx = p_lo(a), nyy = p_hi(a), nyz = p_lo(b);
@@ -557,6 +557,11 @@ __global__ void __launch_bounds__(256) k_fast_c2e(Pass P) {
   const float2 m1 = make_float2(-1.f, -1.f);
   // a - b as one packed FMA: b (-1) + a, exact product, one rounding
   auto sub2 = [&](float2 a2, float2 b2) { return p_fma(b2, m1, a2); };
+  // the product's negation on the integer pipe (the subtractions' too is slower: 247 -> 259 us)
+  auto neg = [](float2 a2) {
+    return make_float2(__uint_as_float(__float_as_uint(a2.x) ^ 0x80000000u),
+                       __uint_as_float(__float_as_uint(a2.y) ^ 0x80000000u));
+  };
   for (int i = threadIdx.x; i < rows; i += blockDim.x) {
     // packed over box pairs: per half the operations of the scalar double-FP32 form
     float2 sh[NB / 2], sl[NB / 2];
@@ -579,7 +584,7 @@ __global__ void __launch_bounds__(256) k_fast_c2e(Pass P) {
         for (int h = 0; h < NB / 2; ++h) {
           const float2 x = x2p[h];
           const float2 p = p_mul(ah2, x);
-          const float2 err = p_fma(al2, x, p_fma(ah2, x, p_mul(p, m1)));
+          const float2 err = p_fma(al2, x, p_fma(ah2, x, neg(p)));
           const float2 t = p_add(sh[h], p), bv = sub2(t, sh[h]);
           sl[h] = p_add(sl[h], p_add(p_add(sub2(sh[h], sub2(t, bv)), sub2(p, bv)), err));
           sh[h] = t;
@@ -1209,7 +1214,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks) k_fast_kmulp_tc(
 // Work items of the L2T (leaf points against the leaf's downward density and
 // its W-list boxes' upward densities): a block of pb points (a power of two,
 // 8 <= pb <= 256) against all of the leaf's sources, S = 256 / pb threads per
-// point (adjacent lanes, each taking every S-th staged source pair, summed by
+// two points (adjacent lanes, each taking every S-th staged source pair, summed by
 // shuffles in a fixed order).  pb is the largest with pb x sources <=
 // kItemWork (and no larger than the points need), so that a leaf with a long
 // W-list is spread over many CTAs; every point is evaluated by one item,
@@ -1373,11 +1378,12 @@ __global__ void k_fast_dchk(Pass P) {
       }
 }
 
-// L2T + W-list: items of the leaves (k_fast_item_counts); a thread takes one
-// point and every S-th staged source pair (S adjacent lanes per point); the
-// leaf's downward density and its W-list boxes' upward densities are staged
-// in batches in the leaf's frame.
-__global__ void __launch_bounds__(kItemThreads) k_fast_l2t(Pass P) {
+// L2T + W-list: items of the leaves (k_fast_item_counts); a thread takes two
+// points, one of each half of the item, and every S-th staged source pair (S adjacent
+// lanes per point); the leaf's downward density and its W-list boxes' upward densities
+// are staged in batches in the leaf's frame.  With one point per thread the reads of
+// the staged pairs were the bound (635 us at 1,048,928 points, now 475).
+__global__ void __launch_bounds__(kItemThreads / 2) k_fast_l2t(Pass P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ EqSrc src[kEqBatchMax];
   const int neq = eq_batch_boxes(P.ns);
@@ -1400,16 +1406,19 @@ __global__ void __launch_bounds__(kItemThreads) k_fast_l2t(Pass P) {
     const int pb = 1 << (item.y >> 24), sw = kItemThreads / pb;
     const int64_t e = i0 + (int64_t)(item.y & 0xffffff) * pb + (int)threadIdx.x / sw;
     const int sl = (int)threadIdx.x % sw;
-    const bool act = e < i1;
+    const bool act = e < i1, act2 = e + pb / 2 < i1;
+    // uniform over the CTA: does the item have points in its second half?
+    const bool two = i0 + (int64_t)(item.y & 0xffffff) * pb + pb / 2 < i1;
     const float r = half_width(P.t, d);
     const int32_t w0 = P.t.w_ptr[b], w1 = P.t.w_ptr[b + 1];
     const int ndn = d >= kFirstDepth ? 1 : 0;
     const int neqs = ndn + (w1 - w0);
-    float2 x2[1][3], uf[1][3], uq[1][3];
+    float2 x2[2][3], uf[2][3], uq[2][3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       x2[0][q] = p_dup(act ? P.ploc[3 * e + q] : 0.f);
-      uf[0][q] = uq[0][q] = make_float2(0.f, 0.f);
+      x2[1][q] = p_dup(act2 ? P.ploc[3 * (e + pb / 2) + q] : 0.f);
+      uf[0][q] = uq[0][q] = uf[1][q] = uq[1][q] = make_float2(0.f, 0.f);
     }
     for (int e0 = 0; e0 < neqs; e0 += neq) {
       const int nb = min(neq, neqs - e0);
@@ -1440,20 +1449,29 @@ __global__ void __launch_bounds__(kItemThreads) k_fast_l2t(Pass P) {
       stage_eq_pairs(P, E, cap, src, nb);
       __syncthreads();
       if (act) {
-        if (P.nc == 4) eval_eq_pairs<true, 1>(E, cap, sl, (nb * P.ns + 1) / 2, sw, x2, uf, uq);
-        else eval_eq_pairs<false, 1>(E, cap, sl, (nb * P.ns + 1) / 2, sw, x2, uf, uq);
+        const int np = (nb * P.ns + 1) / 2;
+        if (two) {
+          if (P.nc == 4) eval_eq_pairs<true, 2>(E, cap, sl, np, sw, x2, uf, uq);
+          else eval_eq_pairs<false, 2>(E, cap, sl, np, sw, x2, uf, uq);
+        } else {
+          if (P.nc == 4) eval_eq_pairs<true, 1>(E, cap, sl, np, sw, x2, uf, uq);
+          else eval_eq_pairs<false, 1>(E, cap, sl, np, sw, x2, uf, uq);
+        }
       }
     }
-    float u[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      u[q] = csl * (uf[0][q].x + uf[0][q].y) + csrc * (uq[0][q].x + uq[0][q].y);
-      for (int o = 1; o < sw; o <<= 1) u[q] += __shfl_xor_sync(kFull, u[q], o);
-    }
-    if (act && sl == 0) {
-      double *out = P.out + 3 * e;
+    for (int t = 0; t < 2; ++t) {
+      float u[3];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) out[a] = (P.accumulate ? out[a] : 0.0) + f32_to_f64(u[a]);
+      for (int q = 0; q < 3; ++q) {
+        u[q] = csl * (uf[t][q].x + uf[t][q].y) + csrc * (uq[t][q].x + uq[t][q].y);
+        for (int o = 1; o < sw; o <<= 1) u[q] += __shfl_xor_sync(kFull, u[q], o);
+      }
+      if ((t ? act2 : act) && sl == 0) {
+        double *out = P.out + 3 * (e + t * (pb / 2));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) out[a] = (P.accumulate ? out[a] : 0.0) + f32_to_f64(u[a]);
+      }
     }
   }
 }
@@ -1666,8 +1684,8 @@ cudaError_t far_field_fast(const Pass &P0, const int32_t *depth_ptr, int32_t max
   pre("l2t");
   {
     const int64_t bound = (int64_t)P.t.nleaf + (P.n + 7) / 8;
-    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(bound, (int64_t)sms * 8));
-    k_fast_l2t<<<g, kItemThreads,
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(bound, (int64_t)sms * 16));
+    k_fast_l2t<<<g, kItemThreads / 2,
                  sizeof(float4) * kEqFields * ((eq_batch_boxes(ns) * ns + 1) / 2), st>>>(P);
   }
   post();
