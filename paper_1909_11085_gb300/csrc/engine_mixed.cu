@@ -45,23 +45,23 @@ namespace stk {
 
 constexpr int kTMax = 5;     // most targets per lane
 
-// Resident CTAs per SM the engine is compiled for (registers per thread =
-// 65536 / (128 * this)), and the targets of a lane it evaluates together, stage by
-// stage: a packed FMA with three different register operands holds the FMA pipe for
-// 2.8 cycles, one that shares an operand with the instruction before it for 2.2, and
-// targets side by side share the source's vectors.  The double layer alone fits four
-// CTAs that way (139,264 x 204,800: 18.23 -> 17.79 ms, 619,520 x 193,600 points:
-// 75.6 -> 73.3); one target at a time it is best at three CTAs (four: 19.1 ms), as
-// are the single layer (140,000 points: 11.49 ms, grouped with four CTAs 11.98) and
-// both layers (16.15, 16.52), which need more registers.
-template <int KMODE>
+// The double layer of direct sums, whose items are long, has a form of its own (LONG):
+// four CTAs per SM where the others have three (registers per thread = 65536 / (128 x
+// CTAs)), and the targets of a lane in groups of three, evaluated stage by stage.  A
+// packed FMA with three different register operands holds the FMA pipe for 2.8 cycles,
+// one that shares an operand with the instruction before it for 2.2, and targets side by
+// side share the source's vectors: 139,264 x 204,800 points 18.23 -> 17.78 ms, 619,520 x
+// 193,600 75.6 -> 73.3 (four CTAs without the groups: 19.1).  A warp is slower in it, which
+// the near field's few and uneven items show (double layer of 100,000 points in leaves of
+// 256: 700 us, 840 in this form), and the other kinds need more registers (single layer of
+// 140,000 points 11.49 ms, 11.98 in this form; both layers 16.15, 16.52).
+template <bool LONG>
 struct EngineShape {
-  static constexpr int kResident = KMODE == K_DL ? 4 : 3;
-  static constexpr int kGroup = KMODE == K_DL ? 3 : kTMax;
+  static constexpr int kResident = LONG ? 4 : 3;
 };
+constexpr int kGroup = 3;  // targets evaluated together in the long form
 
 constexpr int kSegWin = 64;  // segments read into shared memory at a time
-
 constexpr int kPairs = kChunk / 2;  // staged source pairs per chunk
 constexpr int kFields = 7;          // float4 fields per source pair
 
@@ -148,6 +148,56 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
+// Adds the far-field contribution of one staged source pair to T targets
+// (x2: each coordinate duplicated into both halves; ps: per-half sums).
+// SL:   q/r + d (d.q)/r^3             (q pre-scaled by w / (8 pi mu))
+// DL:   d (d.psi)(d.n)/r^5            (psi pre-scaled by 6 w / (8 pi))
+// SLDL: q/r + d [(d.q)/r^3 + (d.psi)(d.n)/r^5]
+// Per half the operations, operands and rounding are those of a scalar
+// evaluation: d = x - y, |r|^2 = dx dx + (dy dy + dz dz) (pair_r2).
+template <int T, int KIND, bool MASKED>
+__device__ __forceinline__ void pair_block(const float2 (&x2)[T][3], float2 (&ps)[T][3],
+                                           const float4 (&s)[kFields]) {
+  const float2 ny_x = lo2(s[0]), ny_y = hi2(s[0]), ny_z = lo2(s[1]), hh = hi2(s[1]);
+  const float2 qx = lo2(s[2]), qy = hi2(s[2]), qz = lo2(s[3]);
+  const float2 nx = hi2(s[3]), ny = lo2(s[4]), nz = hi2(s[4]);
+  const float2 px = lo2(s[5]), py = hi2(s[5]), pz = lo2(s[6]);
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const float2 dx = add2(x2[t][0], ny_x), dy = add2(x2[t][1], ny_y), dz = add2(x2[t][2], ny_z);
+    float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    // near pair: rsqrt(+inf) = 0 removes it from this sum (k_near adds it)
+    if (MASKED) {
+      if (is_near(r2.x, hh.x)) r2.x = __int_as_float(0x7f800000);
+      if (is_near(r2.y, hh.y)) r2.y = __int_as_float(0x7f800000);
+    }
+    const float2 ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+    const float2 ri2 = mul2(ri, ri);
+    if (KIND == K_SL) {
+      const float2 dq = fma2(dx, qx, fma2(dy, qy, mul2(dz, qz)));
+      const float2 c = mul2(dq, ri2);
+      ps[t][0] = fma2(fma2(dx, c, qx), ri, ps[t][0]);
+      ps[t][1] = fma2(fma2(dy, c, qy), ri, ps[t][1]);
+      ps[t][2] = fma2(fma2(dz, c, qz), ri, ps[t][2]);
+    } else if (KIND == K_DL) {
+      const float2 dp = fma2(dx, px, fma2(dy, py, mul2(dz, pz)));
+      const float2 dn = fma2(dx, nx, fma2(dy, ny, mul2(dz, nz)));
+      const float2 c = mul2(mul2(dp, dn), mul2(mul2(ri2, ri2), ri));
+      ps[t][0] = fma2(dx, c, ps[t][0]);
+      ps[t][1] = fma2(dy, c, ps[t][1]);
+      ps[t][2] = fma2(dz, c, ps[t][2]);
+    } else {
+      const float2 dq = fma2(dx, qx, fma2(dy, qy, mul2(dz, qz)));
+      const float2 dp = fma2(dx, px, fma2(dy, py, mul2(dz, pz)));
+      const float2 dn = fma2(dx, nx, fma2(dy, ny, mul2(dz, nz)));
+      const float2 c = mul2(fma2(mul2(dp, dn), ri2, dq), ri2);
+      ps[t][0] = fma2(fma2(dx, c, qx), ri, ps[t][0]);
+      ps[t][1] = fma2(fma2(dy, c, qy), ri, ps[t][1]);
+      ps[t][2] = fma2(fma2(dz, c, qz), ri, ps[t][2]);
+    }
+  }
+}
+
 // Dot products of the first m differences with one vector of the source pair.
 template <int G>
 __device__ __forceinline__ void dots(int m, const float2 (&d)[G][3], const float2 (&v)[3],
@@ -160,24 +210,18 @@ __device__ __forceinline__ void dots(int m, const float2 (&d)[G][3], const float
   for (int i = 0; i < m; ++i) o[i] = fma2(d[i][0], v[0], o[i]);
 }
 
-// Adds the far-field contribution of one staged source pair to T targets
-// (x2: each coordinate duplicated into both halves; ps: per-half sums).
-// SL:   q/r + d (d.q)/r^3             (q pre-scaled by w / (8 pi mu))
-// DL:   d (d.psi)(d.n)/r^5            (psi pre-scaled by 6 w / (8 pi))
-// SLDL: q/r + d [(d.q)/r^3 + (d.psi)(d.n)/r^5]
-// Per half the operations, operands and rounding are those of a scalar
-// evaluation: d = x - y, |r|^2 = dx dx + (dy dy + dz dz) (pair_r2).
-template <int T, int GROUP, int KIND, bool MASKED>
-__device__ __forceinline__ void pair_block(const float2 (&x2)[T][3], float2 (&ps)[T][3],
-                                           const float4 (&s)[kFields]) {
+// The double layer of the same, kGroup targets at a time: the same operations per half.
+template <int T, bool MASKED>
+__device__ __forceinline__ void pair_block_long(const float2 (&x2)[T][3], float2 (&ps)[T][3],
+                                                const float4 (&s)[kFields]) {
   const float2 hh = hi2(s[1]);
-  const float2 ny[3] = {lo2(s[0]), hi2(s[0]), lo2(s[1])}, q[3] = {lo2(s[2]), hi2(s[2]), lo2(s[3])};
+  const float2 ny[3] = {lo2(s[0]), hi2(s[0]), lo2(s[1])};
   const float2 n[3] = {hi2(s[3]), lo2(s[4]), hi2(s[4])}, p[3] = {lo2(s[5]), hi2(s[5]), lo2(s[6])};
-  constexpr int NG = (T + GROUP - 1) / GROUP, G = (T + NG - 1) / NG;  // groups, targets of one
+  constexpr int NG = (T + kGroup - 1) / kGroup, G = (T + NG - 1) / NG;  // groups, targets of one
 #pragma unroll
   for (int g = 0; g < T; g += G) {
     const int m = T - g < G ? T - g : G;
-    float2 d[G][3], r2[G], ri[G], dq[G], dp[G], dn[G];
+    float2 d[G][3], r2[G], ri[G], dp[G], dn[G];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
@@ -185,7 +229,6 @@ __device__ __forceinline__ void pair_block(const float2 (&x2)[T][3], float2 (&ps
 #pragma unroll
     for (int i = 0; i < m; ++i) {
       r2[i] = fma2(d[i][0], d[i][0], fma2(d[i][1], d[i][1], mul2(d[i][2], d[i][2])));
-      // near pair: rsqrt(+inf) = 0 removes it from this sum (k_near adds it)
       if (MASKED) {
         if (is_near(r2[i].x, hh.x)) r2[i].x = __int_as_float(0x7f800000);
         if (is_near(r2[i].y, hh.y)) r2[i].y = __int_as_float(0x7f800000);
@@ -193,24 +236,14 @@ __device__ __forceinline__ void pair_block(const float2 (&x2)[T][3], float2 (&ps
     }
 #pragma unroll
     for (int i = 0; i < m; ++i) ri[i] = make_float2(rsqrt_ftz(r2[i].x), rsqrt_ftz(r2[i].y));
-    if (KIND & K_SL) dots<G>(m, d, q, dq);
-    if (KIND & K_DL) {
-      dots<G>(m, d, p, dp);
-      dots<G>(m, d, n, dn);
-    }
+    dots<G>(m, d, p, dp);
+    dots<G>(m, d, n, dn);
 #pragma unroll
     for (int i = 0; i < m; ++i) {
-      float2(&u)[3] = ps[g + i];
       const float2 ri2 = mul2(ri[i], ri[i]);
-      if (KIND == K_DL) {
-        const float2 c = mul2(mul2(dp[i], dn[i]), mul2(mul2(ri2, ri2), ri[i]));
+      const float2 c = mul2(mul2(dp[i], dn[i]), mul2(mul2(ri2, ri2), ri[i]));
 #pragma unroll
-        for (int k = 0; k < 3; ++k) u[k] = fma2(d[i][k], c, u[k]);
-      } else {
-        const float2 c = mul2(KIND == K_SL ? dq[i] : fma2(mul2(dp[i], dn[i]), ri2, dq[i]), ri2);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) u[k] = fma2(fma2(d[i][k], c, q[k]), ri[i], u[k]);
-      }
+      for (int k = 0; k < 3; ++k) ps[g + i][k] = fma2(d[i][k], c, ps[g + i][k]);
     }
   }
 }
@@ -234,7 +267,7 @@ __device__ __forceinline__ void load_pair(const WarpSmem &sm, int j, float4 (&s)
 
 // Pairs [0, nfar / 2) hold far sources only; pairs from nfar / 2 to the end
 // hold candidates (and possibly one far source with hh = 0, and a zero pad).
-template <int T, int GROUP, int KIND>
+template <int T, bool LONG, int KIND>
 __device__ __forceinline__ void chunk_compute(WarpSmem &sm, const EngineParams &P,
                                               const ItemCtx &ic, int n, int nfar,
                                               const float2 (&x2)[T][3], float2 (&ps)[T][3]) {
@@ -242,12 +275,14 @@ __device__ __forceinline__ void chunk_compute(WarpSmem &sm, const EngineParams &
   for (int j = ic.sg; j < jfar; j += ic.b) {
     float4 s[kFields];
     load_pair<KIND>(sm, j, s);
-    pair_block<T, GROUP, KIND, false>(x2, ps, s);
+    if (LONG) pair_block_long<T, false>(x2, ps, s);
+    else pair_block<T, KIND, false>(x2, ps, s);
   }
   for (int j = jfar + ic.sg; j < jend; j += ic.b) {
     float4 s[kFields];
     load_pair<KIND>(sm, j, s);
-    pair_block<T, GROUP, KIND, true>(x2, ps, s);
+    if (LONG) pair_block_long<T, true>(x2, ps, s);
+    else pair_block<T, KIND, true>(x2, ps, s);
   }
 }
 
@@ -410,22 +445,21 @@ __device__ __forceinline__ bool cursor_next(const EngineParams &P, const Item &i
   return true;
 }
 
-template <int T, int KMODE>
+template <int T, int KMODE, bool LONG>
 __device__ __forceinline__ void dispatch_compute(int kind, WarpSmem &sm, const EngineParams &P,
                                                  const ItemCtx &ic, int n, int nfar,
                                                  const float2 (&x2)[T][3], float2 (&ps)[T][3]) {
-  constexpr int G = EngineShape<KMODE>::kGroup;
   if (KMODE != 0) {
-    chunk_compute<T, G, KMODE>(sm, P, ic, n, nfar, x2, ps);
+    chunk_compute<T, LONG, KMODE>(sm, P, ic, n, nfar, x2, ps);
   } else if (kind == K_SL) {
-    chunk_compute<T, G, K_SL>(sm, P, ic, n, nfar, x2, ps);
+    chunk_compute<T, false, K_SL>(sm, P, ic, n, nfar, x2, ps);
   } else {
-    chunk_compute<T, G, K_DL>(sm, P, ic, n, nfar, x2, ps);
+    chunk_compute<T, false, K_DL>(sm, P, ic, n, nfar, x2, ps);
   }
 }
 
 // One work item with T targets per lane and b source slices per warp.
-template <int T, int KMODE>
+template <int T, int KMODE, bool LONG>
 __device__ bool run_item(const EngineParams &P, const Item &it, int id, WarpSmem &sm, int b,
                          uint32_t &phase, int lane) {
   ItemCtx ic;
@@ -600,7 +634,7 @@ __device__ bool run_item(const EngineParams &P, const Item &it, int id, WarpSmem
       issue_chunk(sm, P.rec, cur.s, n_next, lane);
       cur.s += n_next;
     }
-    dispatch_compute<T, KMODE>(kind_cur, sm, P, ic, n_cur, nfar, x2, ps);
+    dispatch_compute<T, KMODE, LONG>(kind_cur, sm, P, ic, n_cur, nfar, x2, ps);
     // plain FP32 over eight chunks (<= 256 sources per half), then into the
     // (hi, lo) sums
     if (++npend == kSumChunks || !have_next) {
@@ -662,8 +696,8 @@ __device__ bool run_item(const EngineParams &P, const Item &it, int id, WarpSmem
   return true;
 }
 
-template <int KMODE>
-__global__ void __launch_bounds__(kWarpsPerCta *kWarp, EngineShape<KMODE>::kResident)
+template <int KMODE, bool LONG>
+__global__ void __launch_bounds__(kWarpsPerCta *kWarp, EngineShape<LONG>::kResident)
     k_engine_mixed(EngineParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   WarpSmem &sm = reinterpret_cast<WarpSmem *>(smem_raw)[threadIdx.x / kWarp];
@@ -691,20 +725,20 @@ __global__ void __launch_bounds__(kWarpsPerCta *kWarp, EngineShape<KMODE>::kResi
     const int b = (P.policy != 1 && tn <= 40) ? 4 : (tn <= 80 ? 2 : 1);
     const int slots_per_t = kWarp / b;
     if (tn <= 3 * slots_per_t)
-      ok = run_item<3, KMODE>(P, it, id, sm, b, phase, lane);
+      ok = run_item<3, KMODE, LONG>(P, it, id, sm, b, phase, lane);
     else if (tn <= 4 * slots_per_t)
-      ok = run_item<4, KMODE>(P, it, id, sm, b, phase, lane);
+      ok = run_item<4, KMODE, LONG>(P, it, id, sm, b, phase, lane);
     else
-      ok = run_item<5, KMODE>(P, it, id, sm, b, phase, lane);
+      ok = run_item<5, KMODE, LONG>(P, it, id, sm, b, phase, lane);
     if (!ok) break;
   }
 }
 
 size_t engine_mixed_smem_bytes() { return sizeof(WarpSmem) * kWarpsPerCta; }
 
-template <int KMODE>
+template <int KMODE, bool LONG = false>
 static cudaError_t launch_kmode(const EngineParams &P, int grid, cudaStream_t stream) {
-  k_engine_mixed<KMODE><<<grid, kWarpsPerCta * kWarp, engine_mixed_smem_bytes(), stream>>>(P);
+  k_engine_mixed<KMODE, LONG><<<grid, kWarpsPerCta * kWarp, engine_mixed_smem_bytes(), stream>>>(P);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -716,26 +750,29 @@ cudaError_t launch_engine_mixed(const EngineParams &P, int grid, cudaStream_t st
   if (P.kind_alternating) return launch_kmode<0>(P, grid, stream);
   switch (P.kind) {
     case K_SL: return launch_kmode<K_SL>(P, grid, stream);
-    case K_DL: return launch_kmode<K_DL>(P, grid, stream);
+    case K_DL:
+      return engine_mixed_form(P) == kEngineLong ? launch_kmode<K_DL, true>(P, grid, stream)
+                                                 : launch_kmode<K_DL>(P, grid, stream);
     default: return launch_kmode<K_SLDL>(P, grid, stream);
   }
 }
 
-template <int KMODE>
+template <int KMODE, bool LONG = false>
 static cudaError_t occupancy(int *blocks_per_sm) {
   const cudaError_t e =
-      cudaFuncSetAttribute(k_engine_mixed<KMODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(k_engine_mixed<KMODE, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)engine_mixed_smem_bytes());
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, k_engine_mixed<KMODE>, kWarpsPerCta * kWarp, engine_mixed_smem_bytes());
+      blocks_per_sm, k_engine_mixed<KMODE, LONG>, kWarpsPerCta * kWarp, engine_mixed_smem_bytes());
 }
 
-cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[4]) {
+cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[kEngineForms]) {
   cudaError_t e = occupancy<0>(blocks_per_sm);
   if (e == cudaSuccess) e = occupancy<K_SL>(blocks_per_sm + K_SL);
   if (e == cudaSuccess) e = occupancy<K_DL>(blocks_per_sm + K_DL);
   if (e == cudaSuccess) e = occupancy<K_SLDL>(blocks_per_sm + K_SLDL);
+  if (e == cudaSuccess) e = occupancy<K_DL, true>(blocks_per_sm + kEngineLong);
   return e;
 }
 

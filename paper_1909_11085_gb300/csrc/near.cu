@@ -211,6 +211,7 @@ __device__ __forceinline__ void finish_unit(NearSmem<TARGETS> &sm, const EngineP
 }
 
 __global__ void __launch_bounds__(kNearWarps *kWarp, kNearMinBlocks) k_near(EngineParams P) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_near_over, as room comes free
   __shared__ NearSmem<kItemMax> smem[kNearWarps];
   NearSmem<kItemMax> &sm = smem[threadIdx.x / kWarp];
   const int lane = threadIdx.x & (kWarp - 1);
@@ -279,8 +280,12 @@ struct OverSmem {
 static_assert(sizeof(OverSmem) <= 48 * 1024, "no opt-in shared memory");
 
 __global__ void __launch_bounds__(kOverThreads, 2) k_near_over(EngineParams P) {
+  // (the engine's results only: complete before k_near began); it ends after k_near
   const int n_over = *P.over_cnt;
-  if (n_over == 0 || *P.err_flag) return;
+  if (n_over == 0 || *P.err_flag) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   extern __shared__ __align__(16) unsigned char over_smem[];
   OverSmem &sm = *reinterpret_cast<OverSmem *>(over_smem);
   const int tid = threadIdx.x, lane = tid & (kWarp - 1), wid = tid / kWarp;
@@ -395,6 +400,7 @@ __global__ void __launch_bounds__(kOverThreads, 2) k_near_over(EngineParams P) {
     if (nc) take(nc);
     if (tn > 0) finish_unit(ws, P, t0, tn, it.tn_part >> 8, qn, lane);
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace
@@ -407,7 +413,19 @@ void launch_near(const EngineParams &P, int sms, int64_t max_items, cudaStream_t
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
   k_near<<<(int)grid, kNearWarps * kWarp, 0, st>>>(P);
-  k_near_over<<<2 * sms, kOverThreads, sizeof(OverSmem), st>>>(P);
+  // k_near_over reads and adds to nothing of k_near's: it starts as that one's CTAs end
+  // (2 to 6 us of a call when no list has overflowed)
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * sms));
+  cfg.blockDim = dim3(kOverThreads);
+  cfg.dynamicSmemBytes = sizeof(OverSmem);
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_near_over, P);
   count_launches(2);
 }
 

@@ -430,11 +430,13 @@ __global__ void k_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t n
   if (g == 0) *n_items = (int32_t)tot;
 }
 
+// Items per leaf, and the leaves' ends as the engine's 64-bit segment ends.
 __global__ void k_p2p_count(int32_t nleaf, const int32_t *__restrict__ leaf_ptr, int32_t item_max,
-                            int32_t *__restrict__ cnt) {
-  for (int32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nleaf; b += gridDim.x * blockDim.x) {
-    const int32_t nb = leaf_ptr[b + 1] - leaf_ptr[b];
-    cnt[b] = (nb + item_max - 1) / item_max;
+                            int32_t *__restrict__ cnt, int64_t *__restrict__ range) {
+  for (int32_t b = blockIdx.x * blockDim.x + threadIdx.x; b <= nleaf; b += gridDim.x * blockDim.x) {
+    const int32_t i = leaf_ptr[b];
+    range[b] = i;
+    if (b < nleaf) cnt[b] = (leaf_ptr[b + 1] - i + item_max - 1) / item_max;
   }
 }
 
@@ -637,9 +639,9 @@ void launch_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t nsub, i
 
 void launch_p2p_items(int32_t nleaf, const int32_t *leaf_ptr, const int32_t *ulist_ptr,
                       const int32_t *ulist_idx, int32_t item_max, int32_t *cnt, int32_t *offs,
-                      int32_t *n_items, Item *items, uint64_t *keys, int32_t *vals,
+                      int32_t *n_items, int64_t *range, Item *items, uint64_t *keys, int32_t *vals,
                       cudaStream_t st) {
-  k_p2p_count<<<grid_for(nleaf, 256), 256, 0, st>>>(nleaf, leaf_ptr, item_max, cnt);
+  k_p2p_count<<<grid_for((int64_t)nleaf + 1, 256), 256, 0, st>>>(nleaf, leaf_ptr, item_max, cnt, range);
   count_launches(1);
   k_scan_excl<<<1, kScanThreads, 0, st>>>(cnt, nleaf, offs, n_items);
   count_launches(1);
@@ -684,13 +686,4 @@ void launch_zero_ints(int32_t *p, int n, cudaStream_t st) {
 }  // namespace stk
 
 namespace stk {
-__global__ void k_widen(int64_t n, const int32_t *__restrict__ in, int64_t *__restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = in[i];
-}
-void launch_widen(int64_t n, const int32_t *in, int64_t *out, cudaStream_t st) {
-  k_widen<<<grid_for(n, 256), 256, 0, st>>>(n, in, out);
-  count_launches(1);
-}
 }  // namespace stk

@@ -42,7 +42,7 @@ void launch_items_direct(int32_t nt, int64_t ns, int32_t nsplit, int32_t nsub, i
                          Item *items, int64_t *range_ptr, int32_t *n_items, cudaStream_t st);
 void launch_p2p_items(int32_t nleaf, const int32_t *leaf_ptr, const int32_t *ulist_ptr,
                       const int32_t *ulist_idx, int32_t item_max, int32_t *cnt, int32_t *offs,
-                      int32_t *n_items, Item *items, uint64_t *keys, int32_t *vals,
+                      int32_t *n_items, int64_t *range, Item *items, uint64_t *keys, int32_t *vals,
                       cudaStream_t st);
 void launch_batched_items(int32_t nsusp, const int64_t *susp_ptr, const int64_t *n_cell,
                           int32_t item_max, int32_t *cnt, int32_t *offs, int32_t *n_items,
@@ -69,7 +69,6 @@ cudaError_t launch_direct_small(int kinds, const double *src, const double *f, c
 void launch_finish(int64_t nt, int32_t nparts, const double *part_out, const int32_t *tperm,
                    int32_t accumulate, double *out, cudaStream_t st);
 void launch_zero_ints(int32_t *p, int n, cudaStream_t st);
-void launch_widen(int64_t n, const int32_t *in, int64_t *out, cudaStream_t st);
 
 // Adjoint passes (adjoint.cu).
 struct AdjParams {
@@ -105,8 +104,15 @@ void launch_adj_finish(bool src_major, int64_t n, int32_t nsplit, const double *
 
 size_t engine_mixed_smem_bytes();
 cudaError_t launch_engine_mixed(const EngineParams &P, int grid, cudaStream_t stream);
-// Resident CTAs per SM by kernel kind (0: kinds by segment).
-cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[4]);
+// Forms of the engine: by kernel kind (0: kinds by segment), and the double layer of
+// direct sums.
+constexpr int kEngineLong = 4, kEngineForms = 5;
+inline int engine_mixed_form(const EngineParams &P) {
+  if (P.kind_alternating) return 0;
+  return P.kind == K_DL && !P.seg_list ? kEngineLong : P.kind;
+}
+// Resident CTAs per SM by form.
+cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[kEngineForms]);
 // Launches both FP64 engines (grids of resident CTAs); *F.state picks one.
 cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,
                                cudaStream_t stream);

@@ -66,7 +66,7 @@ constexpr int64_t kSpinLimit = 4000000000LL;  // SM cycles, about 2 s at 2 GHz
 struct DevInfo {
   int dev = -1;
   int sms = 0;
-  int occ_mixed[4] = {0, 0, 0, 0};  // by kernel kind, 0: alternating
+  int occ_mixed[kEngineForms] = {};  // by form
   int occ_fp64 = 0;
   int occ_fx = 0;
 };
@@ -394,7 +394,7 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
   P.policy = p.tile.policy;
   P.part_out = direct_out ? direct_out : at<double>(ws, p.part);
   P.nt = (int32_t)p.nt;
-  const int occ = p.mixed ? di.occ_mixed[P.kind_alternating ? 0 : P.kind] : di.occ_fp64;
+  const int occ = p.mixed ? di.occ_mixed[engine_mixed_form(P)] : di.occ_fp64;
   int64_t grid = (int64_t)di.sms * occ;
   const int64_t need = (p.max_items + kWarpsPerCta - 1) / kWarpsPerCta;
   if (grid > need) grid = need;
@@ -776,11 +776,10 @@ stk_status stokes_p2p_leaflists(const double *pts, const double *f, const double
   if (s != STK_OK) return s;
   if (sd) CU(cudaEventRecord(sd->join, sd->s));
   int64_t *range = at<int64_t>(ws, p.range);
-  launch_widen((int64_t)nleaf + 1, leaf_ptr, range, st);
   int32_t *counters = at<int32_t>(ws, p.counters);
   const int32_t *order = build_sorted_items(p, ws, st, [&](uint64_t *keys, int32_t *vals) {
     launch_p2p_items(nleaf, leaf_ptr, ulist_ptr, ulist_idx, p.tile.item_max, at<int32_t>(ws, p.cnt),
-                     at<int32_t>(ws, p.offs), counters, at<Item>(ws, p.items), keys, vals, st);
+                     at<int32_t>(ws, p.offs), counters, range, at<Item>(ws, p.items), keys, vals, st);
   });
   CU(cudaGetLastError());
   if (sd) CU(cudaStreamWaitEvent(st, sd->join, 0));
