@@ -54,7 +54,8 @@ typedef enum {
 } stk_status;
 
 typedef enum {
-  /* FP64 throughout: pair differences, 1/r and products in double. */
+  /* FP64 accuracy: pair differences, dot products and 1/r in double or, where the
+   * inputs' range allows it, in 64-bit fixed point of no larger error. */
   STK_FP64 = 0,
   /* FP32 pair arithmetic in per-work-item local frames with compensated
    * (two-sum) accumulation; pairs closer than near_ratio * h_j get their
@@ -300,7 +301,8 @@ stk_status stokes_upsample_patches(const double *coarse, int32_t npatch, int32_t
  * trg [nt][3]; outputs: patch [nt] (-1: none within d_eps), uv [nt][2],
  * y [nt][3], n [nt][3], dist [nt] (-1 for none).  Patch boxes are grown by
  * d_eps and 5% of their diagonal, so a target whose closest point lies
- * further outside its patch's node box than that is not found.  FP64.
+ * further outside its patch's node box than that is not found.  FP64 results; candidates
+ * are ranked in FP32 and the closest points finished in FP64.
  * 2 <= q <= 12. */
 stk_status stokes_near_patch_search(const double *nodes, int32_t npatch, int32_t q,
                                     const double *trg, int64_t nt, double d_eps, int32_t *patch,
