@@ -38,7 +38,8 @@
 // the patch's centre), which take two multiply-adds per degree for a basis
 // value and its derivative where the barycentric form takes two divisions.  A
 // pair that FP32 cannot settle (a target on a node, a step that does not
-// decrease the distance, no convergence, a Hessian near singular) takes the
+// decrease the distance, no convergence, a Hessian near singular) and one whose
+// closest point lies beside a node's parameter (kNzNodeGap) takes the
 // plain FP64 iteration (nz_closest), the search's definition.
 // 2^20 targets against 320 patches (63.9 k hits): see k_nz_search.
 // Results are FP64; the normal is (dP/du x dP/dv) / |dP/du x dP/dv|.
@@ -344,6 +345,71 @@ __device__ void nz_eval(int n1, const double *__restrict__ X, const double *xk, 
   }
 }
 
+// The same by a warp.  Every sum is one lane's, over the terms of the forms above in their
+// order (and sig is rounded before the difference, as there), so the results are theirs bit
+// for bit.  Lanes 0 .. n1 - 1 hold the u basis, 16 .. 16 + n1 - 1 the v basis; then a lane
+// takes up to three of the 6 n1 row sums, and lanes 0 .. 8 the sums over the rows.
+__device__ __forceinline__ void nz_basis_warp(int n1, const double *xk, const double *wk, double u,
+                                              double v, int lane, double &L, double &D) {
+  const int half = lane & 16, k = (lane & 15) < n1 ? lane & 15 : 0;
+  const double t = half ? v : u;
+  const unsigned on = __ballot_sync(kFull, (lane & 15) < n1 && fabs(t - xk[k]) < 1e-14);
+  const unsigned mine = (on >> half) & 0xffffu;
+  const int hit = mine ? 31 - __clz(mine) : -1;
+  const double r = hit >= 0 ? (k == hit ? 0.0 : (wk[k] / wk[hit]) / (xk[hit] - xk[k]))
+                            : 1.0 / (t - xk[k]);
+  const double a = wk[k] * r;
+  double S = 0.0, S2 = 0.0;  // with a node hit: the sum of the row's other entries
+  for (int m = 0; m < n1; ++m) {
+    const double am = __shfl_sync(kFull, a, half + m), rm = __shfl_sync(kFull, r, half + m);
+    if (hit < 0) {
+      S += am;
+      S2 += am * rm;
+    } else if (m != hit) {
+      S -= rm;
+    }
+  }
+  if (hit >= 0) {
+    L = k == hit ? 1.0 : 0.0;
+    D = k == hit ? S : r;
+  } else {
+    const double iS = 1.0 / S, sig = __dmul_rn(S2, iS);
+    L = a * iS;
+    D = L * (sig - r);
+  }
+}
+__device__ __noinline__ void nz_eval_warp(int n1, const double *__restrict__ X, const double *xk,
+                                          const double *wk, double u, double v, int lane,
+                                          double *P, double *Pu, double *Pv) {
+  static_assert(kNzMaxN1 <= 16 && 6 * kNzMaxN1 <= 3 * kWarp, "a basis per half warp, three sums per lane");
+  double L, D;
+  nz_basis_warp(n1, xk, wk, u, v, lane, L, D);
+  double T[3] = {0.0, 0.0, 0.0};  // sum s = 6 i + c (values, c < 3) or 6 i + 3 + c (v derivatives)
+  for (int j = 0; j < n1; ++j) {
+    const double lj = __shfl_sync(kFull, L, 16 + j), dj = __shfl_sync(kFull, D, 16 + j);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const int s = lane + kWarp * m, i = s / 6, c = s % 3;
+      if (i < n1) T[m] = fma(s % 6 < 3 ? lj : dj, X[3 * (i * n1 + j) + c], T[m]);
+    }
+  }
+  const int out = lane < 9 ? lane / 3 : 0, c = lane % 3;  // P, P_u, P_v
+  double acc = 0.0;
+  for (int i = 0; i < n1; ++i) {
+    const double li = __shfl_sync(kFull, L, i), di = __shfl_sync(kFull, D, i);
+    const int s = 6 * i + c + (out == 2 ? 3 : 0);
+    const double t0 = __shfl_sync(kFull, T[0], s & 31), t1 = __shfl_sync(kFull, T[1], s & 31),
+                 t2 = __shfl_sync(kFull, T[2], s & 31);
+    acc = fma(out == 1 ? di : li, s < 32 ? t0 : s < 64 ? t1 : t2, acc);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    P[q] = __shfl_sync(kFull, acc, q);
+    Pu[q] = __shfl_sync(kFull, acc, 3 + q);
+    Pv[q] = __shfl_sync(kFull, acc, 6 + q);
+  }
+}
+
 // The node of a patch nearest to x: squared distance and its (u, v).
 __device__ double nz_nearest_node(int n1, const double *__restrict__ X, const double *xk,
                                   const double x[3], double &u, double &v) {
@@ -361,12 +427,50 @@ __device__ double nz_nearest_node(int n1, const double *__restrict__ X, const do
   return best;
 }
 
-// Closest point of a patch to x, from the start (u, v).
+__device__ double nz_nearest_node_warp(int n1, const double *__restrict__ X, const double *xk,
+                                       const double x[3], int lane, double &u, double &v) {
+  double best = DBL_MAX;
+  int at = n1 * n1;  // the first of the nearest ones
+  for (int e = lane; e < n1 * n1; e += kWarp) {
+    const double *xp = X + 3 * e;
+    const double d = (xp[0] - x[0]) * (xp[0] - x[0]) + (xp[1] - x[1]) * (xp[1] - x[1]) +
+                     (xp[2] - x[2]) * (xp[2] - x[2]);
+    if (d < best) {
+      best = d;
+      at = e;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double d = __shfl_xor_sync(kFull, best, o);
+    const int e = __shfl_xor_sync(kFull, at, o);
+    if (d < best || (d == best && e < at)) {
+      best = d;
+      at = e;
+    }
+  }
+  if (at < n1 * n1) {
+    u = xk[at / n1];
+    v = xk[at % n1];
+  }
+  return best;
+}
+
+// Closest point of a patch to x, from the start (u, v): by each thread, or (WARP) by a
+// warp for one x, with the same results.
+template <bool WARP>
+__device__ __forceinline__ void nz_eval_by(int n1, const double *__restrict__ X, const double *xk,
+                                           const double *wk, double u, double v, int lane,
+                                           double P[3], double Pu[3], double Pv[3]) {
+  if (WARP) nz_eval_warp(n1, X, xk, wk, u, v, lane, P, Pu, Pv);
+  else nz_eval(n1, X, xk, wk, u, v, P, Pu, Pv);
+}
+template <bool WARP>
 __device__ double nz_closest(int n1, const double *__restrict__ X, const double *xk,
-                             const double *wk, const double x[3], double &u, double &v,
+                             const double *wk, const double x[3], int lane, double &u, double &v,
                              double y[3], double nn[3]) {
   double P[3], Pu[3], Pv[3];
-  nz_eval(n1, X, xk, wk, u, v, P, Pu, Pv);
+  nz_eval_by<WARP>(n1, X, xk, wk, u, v, lane, P, Pu, Pv);
   double f = 0.0;
 #pragma unroll
   for (int c = 0; c < 3; ++c) f += (P[c] - x[c]) * (P[c] - x[c]);
@@ -407,7 +511,7 @@ __device__ double nz_closest(int n1, const double *__restrict__ X, const double 
     for (int ls = 0; ls < 40; ++ls) {
       un = fmin(1.0, fmax(-1.0, u + a * su));
       vn = fmin(1.0, fmax(-1.0, v + a * sv));
-      nz_eval(n1, X, xk, wk, un, vn, Pn, Pun, Pvn);
+      nz_eval_by<WARP>(n1, X, xk, wk, un, vn, lane, Pn, Pun, Pvn);
       fn = 0.0;
 #pragma unroll
       for (int c = 0; c < 3; ++c) fn += (Pn[c] - x[c]) * (Pn[c] - x[c]);
@@ -734,15 +838,18 @@ __device__ __forceinline__ bool nz_pair32(int n1, const float4 *__restrict__ C, 
   return ok && d < 3e18f;  // false for NaN too
 }
 
-// The plain FP64 iteration from the nearest node (out of line: rare).
+// The plain FP64 iteration from the nearest node (out of line: rare).  res: u, v, y, n.
+template <bool WARP>
 __device__ __noinline__ double nz_pair_plain(int n1, const double *__restrict__ X, const double *xk,
                                              const double *wk, const double *x, double d_eps,
-                                             double rp, double *res) {
+                                             double rp, int lane, double *res) {
   const double xx[3] = {x[0], x[1], x[2]};
   double u, v, y[3], nn[3];
   // every point of the patch lies within rp of a node
-  if (sqrt(nz_nearest_node(n1, X, xk, xx, u, v)) - rp > d_eps) return DBL_MAX;
-  const double d = nz_closest(n1, X, xk, wk, xx, u, v, y, nn);
+  const double d2 = WARP ? nz_nearest_node_warp(n1, X, xk, xx, lane, u, v)
+                         : nz_nearest_node(n1, X, xk, xx, u, v);
+  if (sqrt(d2) - rp > d_eps) return DBL_MAX;
+  const double d = nz_closest<WARP>(n1, X, xk, wk, xx, lane, u, v, y, nn);
   res[0] = u;
   res[1] = v;
 #pragma unroll
@@ -892,11 +999,63 @@ __device__ __forceinline__ void nz_stage32(NzWarpSmem &sm, const NzPatches &Q, i
   __syncwarp();
 }
 
+// The barycentric basis of the plain iteration loses eps / |t - x_k| of its derivatives
+// when a parameter t comes near a node x_k: the normals are good to about 2e-15 / |t - x_k|
+// (11 nodes; arcs and spheres, coordinates up to 100), those of the Chebyshev form to
+// 1e-14 everywhere.  The plain iteration is the search's definition, so where the two
+// could differ by more than 1e-9 of a normal's size it takes the pair; closer to a node
+// than kNzNodeNone, where its derivatives hold fewer than six digits, the Chebyshev form's
+// stand.  Random targets: 22 kNzNodeGap of the pairs, some 14 of the 63.9 k hits of k_nz_search's
+// figures, which take the call from 1.02 to 1.27 ms (the Armijo test fails in the noise, so
+// such a pair takes all 40 iterations).
+constexpr double kNzNodeGap = 1e-5, kNzNodeNone = 1e-9;
+__device__ __forceinline__ bool nz_beside_node(int n1, const double *xkd, const float *xk,
+                                               double t) {
+  bool beside = false;
+  const float tf = (float)t;
+  for (int k = 0; k < n1; ++k)
+    if (fabsf(tf - xk[k]) < 2.f * (float)kNzNodeGap) {  // few: FP64 only for these
+      const double gap = fabs(t - xkd[k]);
+      beside = beside || (gap < kNzNodeGap && gap >= kNzNodeNone);
+    }
+  return beside;
+}
+
+// The plain iteration of the lanes' (p, slot) pairs where `plain`: a warp per pair, or a
+// thread per pair where there are many (a thread alone takes 1.8 ms for its 40 iterations,
+// a warp 0.25).
+constexpr int kNzPlainLanes = 8;
+__device__ __forceinline__ void nz_plain(NzWarpSmem &sm, const NzPatches &Q, int n1,
+                                         const double *xkd, const double *wkd, double d_eps,
+                                         bool plain, int p, int slot, int lane, double &d,
+                                         double (&res)[8]) {
+  unsigned todo = __ballot_sync(kFull, plain);
+  const size_t pn = (size_t)n1 * n1 * 3;
+  if (__popc(todo) > kNzPlainLanes) {
+    if (plain)
+      d = nz_pair_plain<false>(n1, Q.nodes + p * pn, xkd, wkd, sm.x[slot], d_eps, Q.rp[p], lane,
+                               res);
+    return;
+  }
+  for (; todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const int lp = __shfl_sync(kFull, p, l), ls = __shfl_sync(kFull, slot, l);
+    double r[8];
+    const double ld = nz_pair_plain<true>(n1, Q.nodes + lp * pn, xkd, wkd, sm.x[ls], d_eps,
+                                          Q.rp[lp], lane, r);
+    if (lane == l) {
+      d = ld;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) res[q] = r[q];
+    }
+  }
+}
+
 // FP64 stage of the waiting pairs.
 template <int N1>
 __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, int n1,
-                                           const double *xkd, const double *wkd, double d_eps,
-                                           int &nref, int lane) {
+                                           const float *xk, const double *xkd, const double *wkd,
+                                           double d_eps, int &nref, int lane) {
   int n = 0;  // drop the pairs that another patch has beaten since
   for (int e0 = 0; e0 < nref; e0 += kWarp) {
     const int e = e0 + lane;
@@ -928,18 +1087,20 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
     const bool act = e < n;
     double d = DBL_MAX, res[8];
     int p = 0, slot = -1 - lane;
+    bool plain = false;
     if (act) {
       p = sm.rp[e];
       slot = sm.rs[e] & 31;
       const double x[3] = {sm.x[slot][0], sm.x[slot][1], sm.x[slot][2]};
-      d = -1.0;
-      if (!(sm.rs[e] & 32))
+      plain = sm.rs[e] & 32;
+      if (!plain) {
         d = nz_pair64<N1>(n1, Q.c32 + (size_t)p * n1 * n1, Q.c64 + 2 * (size_t)p * n1 * n1,
                           Q.meta[p], x, sm.ru[e], sm.rv[e], res);
-      if (!(d >= 0.0))
-        d = nz_pair_plain(n1, Q.nodes + (size_t)p * n1 * n1 * 3, xkd, wkd, sm.x[slot], d_eps,
-                          Q.rp[p], res);
+        plain = !(d >= 0.0) || nz_beside_node(n1, xkd, xk, res[0]) ||
+                nz_beside_node(n1, xkd, xk, res[1]);
+      }
     }
+    nz_plain(sm, Q, n1, xkd, wkd, d_eps, plain, p, slot, lane, d, res);
     // the nearest patch of a target, ties to the lower index; pairs of one
     // target take turns
     const unsigned grp = __match_any_sync(kFull, slot);
@@ -1044,11 +1205,11 @@ __global__ void __launch_bounds__(kNzWarps *kWarp, 3) k_nz_search(
         }
         nq = rest;
         __syncwarp();
-        if (nref > kNzRefine - kWarp) nz_stage64<N1>(sm, Q, n1, xkd, wkd, d_eps, nref, lane);
+        if (nref > kNzRefine - kWarp) nz_stage64<N1>(sm, Q, n1, xk, xkd, wkd, d_eps, nref, lane);
       }
       if (!any && nq == 0) break;
     }
-    if (nref) nz_stage64<N1>(sm, Q, n1, xkd, wkd, d_eps, nref, lane);
+    if (nref) nz_stage64<N1>(sm, Q, n1, xk, xkd, wkd, d_eps, nref, lane);
     __syncwarp();
     if (has) {
       const bool near = sm.bp[lane] >= 0 && sm.bd[lane] <= d_eps;
