@@ -928,6 +928,7 @@ struct NzWarpSmem {
   double res[kWarp][8];     // best so far: u, v, y, n
   double bd[kWarp];         //   distance
   int32_t bp[kWarp];        //   patch
+  int32_t bplain[kWarp];    //   whether the plain iteration gave it
   float best[kWarp];        // no nearer patch can be further than this (FP32 bound)
   int32_t qp[kNzQueue];     // queued pairs: patch
   int32_t qs[kNzQueue];     //   target slot
@@ -1009,6 +1010,9 @@ __device__ __forceinline__ void nz_stage32(NzWarpSmem &sm, const NzPatches &Q, i
 // figures, which take the call from 1.02 to 1.27 ms (the Armijo test fails in the noise, so
 // such a pair takes all 40 iterations).
 constexpr double kNzNodeGap = 1e-5, kNzNodeNone = 1e-9;
+// Distances closer than this share of the coordinates' size could be equal: some thirty
+// times the rounding of the interpolants' sums.
+constexpr double kNzTie = 1e-13;
 __device__ __forceinline__ bool nz_beside_node(int n1, const double *xkd, const float *xk,
                                                double t) {
   bool beside = false;
@@ -1102,13 +1106,37 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
     }
     nz_plain(sm, Q, n1, xkd, wkd, d_eps, plain, p, slot, lane, d, res);
     // the nearest patch of a target, ties to the lower index; pairs of one
-    // target take turns
+    // target take turns.  Two patches that meet in an edge hold its nodes as the same
+    // numbers, and the plain iteration finds the same distance to it from both; the
+    // Chebyshev sums, relative to each patch's own centre, only to rounding.  So distances
+    // that could be equal are those of the plain iteration.
     const unsigned grp = __match_any_sync(kFull, slot);
     const int turn = __popc(grp & ((1u << lane) - 1u));
     for (int k = 0; __any_sync(kFull, act && k <= turn); ++k) {
-      if (act && k == turn && (d < sm.bd[slot] || (d == sm.bd[slot] && p < sm.bp[slot]))) {
+      const bool now = act && k == turn;
+      bool tie = false;
+      if (now && sm.bp[slot] >= 0) {
+        const double *x = sm.x[slot];
+        const double size = fabs(x[0]) + fabs(x[1]) + fabs(x[2]) + (double)Q.meta[p].scale;
+        tie = fabs(d - sm.bd[slot]) <= kNzTie * size && !(plain && sm.bplain[slot]);
+      }
+      if (__any_sync(kFull, tie)) {
+        nz_plain(sm, Q, n1, xkd, wkd, d_eps, tie && !plain, p, slot, lane, d, res);
+        plain = plain || tie;
+        const bool other = tie && !sm.bplain[slot];
+        double bd = 0.0, bres[8];
+        nz_plain(sm, Q, n1, xkd, wkd, d_eps, other, other ? sm.bp[slot] : 0, slot, lane, bd, bres);
+        if (other) {
+          sm.bd[slot] = bd;
+          sm.bplain[slot] = 1;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) sm.res[slot][q] = bres[q];
+        }
+      }
+      if (now && (d < sm.bd[slot] || (d == sm.bd[slot] && p < sm.bp[slot]))) {
         sm.bd[slot] = d;
         sm.bp[slot] = p;
+        sm.bplain[slot] = plain;
 #pragma unroll
         for (int q = 0; q < 8; ++q) sm.res[slot][q] = res[q];
       }

@@ -53,3 +53,63 @@ def test_beside_a_node(lib, along):
     assert (ref[0] >= 0).all()
     for g, r in zip(got, ref):
         np.testing.assert_array_equal(g, r)
+
+
+def _strips(n, fold):
+    """n square patches in a row along x, folded down by `fold` more at each shared edge (of
+    constant u, with the same nodes on both sides), the last index first in space when odd."""
+    out, at, ang = [], np.zeros(2), 0.0
+    V = np.tile(CC, (Q + 1, 1))
+    for _ in range(n):
+        step = np.array([np.cos(ang), -np.sin(ang)])
+        s = 1.0 - CC  # u = 1 at the start of the patch
+        line = at + s[:, None] * step
+        line[0] = at
+        at = line[-1].copy()
+        ang += fold
+        out.append(np.stack([np.repeat(line[:, 0], Q + 1), V.ravel(),
+                             np.repeat(line[:, 1], Q + 1)], 1))
+    return np.stack(out)
+
+
+@pytest.mark.parametrize("flip", [False, True])
+def test_ties_on_an_edge(lib, flip):
+    """Targets beyond a convex edge have their closest point on it: both patches hold it, and
+    the lower index wins."""
+    nodes = _strips(2, 0.9) + np.array([0.3, 0.7, -0.2])
+    edge = nodes[0, -1]
+    np.testing.assert_array_equal(nodes[0, -(Q + 1):], nodes[1, :Q + 1])
+    nodes = (nodes[::-1] if flip else nodes).reshape(-1, 3)
+    rng = np.random.default_rng(32)
+    m = 600
+    ang = rng.uniform(0.1, 0.8, m)  # between the two patches' normals
+    out = np.stack([np.sin(ang), 0 * ang, np.cos(ang)], 1)
+    x = np.stack([np.full(m, edge[0]), 0.7 + rng.uniform(-0.95, 0.95, m), np.full(m, edge[2])], 1)
+    x = x + rng.uniform(0.01, 0.3, m)[:, None] * out
+    p, uv, y, n, d = _search(lib, nodes, 2, x, 0.4)
+    assert (p == 0).all()
+    ref = _search(lib, nodes, 2, x, 0.4, scale=2.0 ** -100)
+    for g, r in zip((p, uv, y, n, d), ref):
+        np.testing.assert_array_equal(g, r)
+
+
+def test_cube_edges_and_corners(lib):
+    """A cube's faces, whose edges run in different directions in the parameters: the patch
+    is the definition's, ties or not."""
+    u, v = [a.ravel() for a in np.meshgrid(CC, CC, indexing="ij")]
+    faces = []
+    for ax in range(3):
+        for sg in (1.0, -1.0):
+            c = np.zeros((u.size, 3))
+            c[:, ax], c[:, (ax + 1) % 3], c[:, (ax + 2) % 3] = sg, sg * u, v
+            faces.append(5.0 * c)
+    nodes = np.concatenate(faces)
+    rng = np.random.default_rng(33)
+    x = rng.uniform(-6.0, 6.0, (4000, 3))
+    got, ref = (_search(lib, nodes, 6, x, 1.0, scale=s) for s in (1.0, 2.0 ** -100))
+    np.testing.assert_array_equal(got[0], ref[0])
+    beyond = (np.abs(x) > 5.0).sum(1) > 1  # closest to an edge or a corner
+    assert (ref[0][beyond] >= 0).sum() > 200
+    hit = ref[0] >= 0
+    np.testing.assert_allclose(got[2][hit], ref[2][hit], rtol=0, atol=1e-9)
+    np.testing.assert_allclose(got[4][hit], ref[4][hit], rtol=0, atol=1e-12)
