@@ -1010,9 +1010,12 @@ __device__ __forceinline__ void nz_stage32(NzWarpSmem &sm, const NzPatches &Q, i
 // figures, which take the call from 1.02 to 1.27 ms (the Armijo test fails in the noise, so
 // such a pair takes all 40 iterations).
 constexpr double kNzNodeGap = 1e-5, kNzNodeNone = 1e-9;
-// Distances closer than this share of the coordinates' size could be equal: some thirty
-// times the rounding of the interpolants' sums.
+// Distances closer than this share of the coordinates' size could be equal, to each other
+// or to d_eps: some thirty times the rounding of the interpolants' sums.
 constexpr double kNzTie = 1e-13;
+__device__ __forceinline__ double nz_size(const NzMeta &m, const double *x) {
+  return fabs(x[0]) + fabs(x[1]) + fabs(x[2]) + (double)m.scale;
+}
 __device__ __forceinline__ bool nz_beside_node(int n1, const double *xkd, const float *xk,
                                                double t) {
   bool beside = false;
@@ -1100,8 +1103,8 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
       if (!plain) {
         d = nz_pair64<N1>(n1, Q.c32 + (size_t)p * n1 * n1, Q.c64 + 2 * (size_t)p * n1 * n1,
                           Q.meta[p], x, sm.ru[e], sm.rv[e], res);
-        plain = !(d >= 0.0) || nz_beside_node(n1, xkd, xk, res[0]) ||
-                nz_beside_node(n1, xkd, xk, res[1]);
+        plain = !(d >= 0.0) || fabs(d - d_eps) <= kNzTie * nz_size(Q.meta[p], x) ||
+                nz_beside_node(n1, xkd, xk, res[0]) || nz_beside_node(n1, xkd, xk, res[1]);
       }
     }
     nz_plain(sm, Q, n1, xkd, wkd, d_eps, plain, p, slot, lane, d, res);
@@ -1116,9 +1119,8 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
       const bool now = act && k == turn;
       bool tie = false;
       if (now && sm.bp[slot] >= 0) {
-        const double *x = sm.x[slot];
-        const double size = fabs(x[0]) + fabs(x[1]) + fabs(x[2]) + (double)Q.meta[p].scale;
-        tie = fabs(d - sm.bd[slot]) <= kNzTie * size && !(plain && sm.bplain[slot]);
+        tie = fabs(d - sm.bd[slot]) <= kNzTie * nz_size(Q.meta[p], sm.x[slot]) &&
+              !(plain && sm.bplain[slot]);
       }
       if (__any_sync(kFull, tie)) {
         nz_plain(sm, Q, n1, xkd, wkd, d_eps, tie && !plain, p, slot, lane, d, res);

@@ -113,3 +113,16 @@ def test_cube_edges_and_corners(lib):
     hit = ref[0] >= 0
     np.testing.assert_allclose(got[2][hit], ref[2][hit], rtol=0, atol=1e-9)
     np.testing.assert_allclose(got[4][hit], ref[4][hit], rtol=0, atol=1e-12)
+
+
+def test_distance_of_exactly_d_eps(lib):
+    """d_eps set to a target's own distance, as the definition has it: found."""
+    R, L, nth, nz = 6.0, 8.0, 6, 2
+    nodes = G.cylinder_wall_patches(R, L, nth, nz, Q)[0]
+    rng = np.random.default_rng(34)
+    x = _wall_targets(rng, rng.uniform(0, 2 * np.pi, 40), rng.uniform(0.5, 7.5, 40), R)
+    d = _search(lib, nodes, nth * nz, x, 1.0, scale=2.0 ** -100)[4]
+    for i in range(40):
+        p, _, _, _, di = _search(lib, nodes, nth * nz, x[i:i + 1], d[i])
+        assert p[0] >= 0 and di[0] == d[i]
+        assert _search(lib, nodes, nth * nz, x[i:i + 1], np.nextafter(d[i], 0.0))[0][0] == -1
