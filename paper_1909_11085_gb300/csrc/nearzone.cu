@@ -967,7 +967,8 @@ __device__ __forceinline__ void nz_stage32(NzWarpSmem &sm, const NzPatches &Q, i
       }
     }
     const float lb = sqrtf(best) - m.rp - tol;
-    keep = !(lb > d_eps || lb > sm.best[slot]);  // NaN: kept
+    plain = !(best < INFINITY);                            // squares beyond FP32's range
+    keep = plain || !(lb > d_eps || lb > sm.best[slot]);  // NaN: kept
     if (keep) {
       // a target on a node is at distance exactly 0, which only the plain
       // iteration's interpolant gives

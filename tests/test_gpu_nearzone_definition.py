@@ -126,3 +126,18 @@ def test_distance_of_exactly_d_eps(lib):
         p, _, _, _, di = _search(lib, nodes, nth * nz, x[i:i + 1], d[i])
         assert p[0] >= 0 and di[0] == d[i]
         assert _search(lib, nodes, nth * nz, x[i:i + 1], np.nextafter(d[i], 0.0))[0][0] == -1
+
+
+@pytest.mark.parametrize("power", [-140, 30, 70, 140])
+def test_lengths_out_of_fp32s_range(lib, power):
+    """Lengths whose squares, or which themselves, leave FP32's range."""
+    R, L, nth, nz = 6.0, 8.0, 6, 2
+    nodes = G.cylinder_wall_patches(R, L, nth, nz, Q)[0]
+    rng = np.random.default_rng(35)
+    x = np.concatenate([_wall_targets(rng, rng.uniform(0, 2 * np.pi, 100),
+                                      rng.uniform(0.5, 7.5, 100), R), rng.uniform(-9, 9, (100, 3))])
+    got, ref = (_search(lib, nodes, nth * nz, x, 0.7, scale=2.0 ** s) for s in (power, -100))
+    assert (ref[0] >= 0).sum() > 90
+    np.testing.assert_array_equal(got[0], ref[0])
+    np.testing.assert_allclose(got[2], ref[2], rtol=0, atol=1e-9)
+    np.testing.assert_allclose(got[4], ref[4], rtol=0, atol=1e-12)
