@@ -546,7 +546,28 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_fx(AdjParams A) {
     int64_t J[3];
     int32_t dh[3], dl[3];
     int ea, eb, z, z3;
-    if (!fx_diff(T.y, S.y, T.thr, S.thr, E, J, dh, dl, ea)) {
+    // dots in units of 2^(e - 60): field 1086 + e - 60
+    double dg = 0.0, dp = 0.0, dn = 0.0;
+    bool fits = fx_diff(T.y, S.y, T.thr, S.thr, E, J, dh, dl, ea);
+    if (fits) {
+      const int64_t vg = fx_dot(dh, dl, T.qh, T.ql);
+      const int bg = 1026 + T.eq + ea;
+      if (!(KIND & K_DL) || !fx_faint(vg)) dg = fx_to_double(vg, bg);
+      else fits = fx_faint_dot(vg, J, dh, T.qh, T.ql, fx_is_exact(T.thr, S.thr & ~kFxRoundQ, kFxRoundQ),
+                               bg, dg);
+      if (KIND & K_DL) {
+        const int en = SRC ? own_en : A.nexp[ic];
+        const int64_t vp = fx_dot(dh, dl, S.ph, S.pl), vn = fx_dot(dh, dl, S.nh, S.nl);
+        const int bp = 1026 + S.epn - en + ea, bn = 1026 + en + ea;
+        if (!fx_faint(vp)) dp = fx_to_double(vp, bp);
+        else fits = fits && fx_faint_dot(vp, J, dh, S.ph, S.pl, fx_is_exact(T.thr, S.thr, kFxRoundP),
+                                         bp, dp);
+        if (!fx_faint(vn)) dn = fx_to_double(vn, bn);
+        else fits = fits && fx_faint_dot(vn, J, dh, S.nh, S.nl, fx_is_exact(T.thr, S.thr, kFxRoundN),
+                                         bn, dn);
+      }
+    }
+    if (!fits) {
       double s[NA];
       for (int i = 0; i < NA; ++i) s[i] = acc[i];
       adj_fx_slow<SRC>(SRC ? irec + ic : orec + oc, SRC ? orec + oc : irec + ic, KIND & K_SL,
@@ -561,14 +582,9 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_fx(AdjParams A) {
     const uint64_t Z = fx_mul62(Y, Y, z), W = fx_mul62(Z, Y, z3);
     const double i1r = fx_round(Y, 1022 + eb - ea), i2r = fx_round(Z, 1022 + 2 * (eb - ea) - z);
     const double i3r = fx_round(W, 1022 + 3 * (eb - ea) - z - z3);
-    // dots in units of 2^(e - 60): field 1086 + e - 60
-    const double dg = fx_to_double(fx_dot(dh, dl, T.qh, T.ql), 1026 + T.eq + ea);
     const double c = dg * i3r, t = c * i2r;
     double e, cd, a = 0.0, b = 0.0, pd = 0.0;  // cd: the bracket above
     if (KIND & K_DL) {
-      const int en = SRC ? own_en : A.nexp[ic];
-      const double dp = fx_to_double(fx_dot(dh, dl, S.ph, S.pl), 1026 + S.epn - en + ea);
-      const double dn = fx_to_double(fx_dot(dh, dl, S.nh, S.nl), 1026 + en + ea);
       a = t * dn;
       b = t * dp;
       pd = dp * dn;

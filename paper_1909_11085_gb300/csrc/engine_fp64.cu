@@ -103,7 +103,7 @@ __device__ void run_item64(const EngineParams &P, const Item &it, int b, int lan
 }
 
 __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 4) k_engine_fp64(EngineParams P, FxParams F) {
-  if (fx_use(*F.state, F.ns)) return;  // k_engine_fx does the call
+  if (fx_use(*F.state, F.ns, F.nt)) return;  // k_engine_fx does the call
   const int lane = threadIdx.x & (kWarp - 1);
   const int n_items = *P.n_items;
   while (true) {
@@ -143,28 +143,26 @@ __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 4) k_engine_fp64(EnginePa
 }
 
 // ------------------------------------------------------------ fixed point
-// The FP64 form of a pair that fixed point cannot hold; n and psi from their
-// fixed point parts (61 bits on the vector's own exponent).
+// The FP64 form of a pair that fixed point cannot hold, from the caller's values (j: the
+// source).
 template <int KIND>
-__device__ __noinline__ void fx_slow(const double *xp, const double *yp, const SrcFx *S,
-                                     double *acc) {
+__device__ __noinline__ void fx_slow(const FxParams &F, const double *xp, const double *yp,
+                                     int64_t j, const double *q, double *acc) {
   const double dx = xp[0] - yp[0], dy = xp[1] - yp[1], dz = xp[2] - yp[2];
   const double r2 = dx * dx + dy * dy + dz * dz;
   if (!(r2 > 0.0)) return;  // zero-distance pair contributes nothing
   const double ri = rsqrt(r2), ri2 = ri * ri;
   double c = 0.0;
   if (KIND & K_DL) {
-    double n[3], p[3];
-    for (int k = 0; k < 3; ++k) {
-      n[k] = ldexp((double)(((int64_t)S->nh[k] << 30) + S->nl[k]), -60);
-      p[k] = ldexp((double)(((int64_t)S->ph[k] << 30) + S->pl[k]), S->epn - 60);
-    }
-    c = (dx * p[0] + dy * p[1] + dz * p[2]) * (dx * n[0] + dy * n[1] + dz * n[2]);
+    const double wc = (F.w ? F.w[j] : 1.0) * F.cdl;
+    const double *n = F.nrm + 3 * j, *p = F.phi + 3 * j;
+    c = (dx * (wc * p[0]) + dy * (wc * p[1]) + dz * (wc * p[2])) *
+        (dx * n[0] + dy * n[1] + dz * n[2]);
   }
   const double d[3] = {dx, dy, dz};
   if (KIND & K_SL) {
-    c = (dx * S->q[0] + dy * S->q[1] + dz * S->q[2] + c * ri2) * ri2;
-    for (int k = 0; k < 3; ++k) acc[k] += (S->q[k] + d[k] * c) * ri;
+    c = (dx * q[0] + dy * q[1] + dz * q[2] + c * ri2) * ri2;
+    for (int k = 0; k < 3; ++k) acc[k] += (q[k] + d[k] * c) * ri;
   } else {
     c *= ri2 * ri2 * ri;
     for (int k = 0; k < 3; ++k) acc[k] += d[k] * c;
@@ -172,14 +170,15 @@ __device__ __noinline__ void fx_slow(const double *xp, const double *yp, const S
 }
 
 template <int KIND>
-__device__ __forceinline__ void seg_fx(const EngineParams &P, const SrcFx *__restrict__ rec, int64_t s, int64_t e, int b, int E,
-                                       const int64_t (&X)[3], uint32_t xthr, const double *xp,
-                                       double (&acc)[3]) {
+__device__ __forceinline__ void seg_fx(const EngineParams &P, const FxParams &F,
+                                       const SrcFx *__restrict__ rec, int64_t s, int64_t e, int b,
+                                       int E, const int64_t (&X)[3], uint32_t xthr,
+                                       const double *xp, double (&acc)[3]) {
   for (int64_t k = s; k < e; k += b) {
     const SrcFx &S = rec[k];
     if (!fx_pair<KIND>(X, xthr, E, S, acc)) {
       double a[3] = {acc[0], acc[1], acc[2]};
-      fx_slow<KIND>(xp, P.src64 + 3 * (size_t)k, &S, a);
+      fx_slow<KIND>(F, xp, P.src64 + 3 * (size_t)k, k, S.q, a);
       acc[0] = a[0];
       acc[1] = a[1];
       acc[2] = a[2];
@@ -200,11 +199,13 @@ constexpr int kFxCols = 256, kFxSlices = 16;
 // 34,816 points on themselves: 71.5 -> 19.9 ms (k_engine_fp64 -> this), near
 // field of 262,096 points: 44.3 -> 7.5 ms (24.2 ms with items of 128 targets,
 // whose last round left the GPU idle).
+// Double layer of a flat wall of 4,096 points at z = 10 at targets 0.1 and less above it
+// (faint dots, summed exactly): 0.41 ms, 0.32 in general position, 1.0 in k_engine_fp64.
 template <int KMODE>
 __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 6) k_engine_fx(EngineParams P, FxParams F) {
   __shared__ double sums[kWarpsPerCta][3][kFxCols];
   const FxState fs = *F.state;
-  if (!fx_use(fs, F.ns)) return;  // k_engine_fp64 does the call
+  if (!fx_use(fs, F.ns, F.nt)) return;  // k_engine_fp64 does the call
   const int E = fx_exp(fs);
   double(*R)[kFxCols] = sums[threadIdx.x / kWarp];
   const int lane = threadIdx.x & (kWarp - 1);
@@ -250,11 +251,11 @@ __global__ void __launch_bounds__(kWarpsPerCta *kWarp, 6) k_engine_fx(EnginePara
             ++e;
           }
         if (KMODE ? KMODE == K_SL : !(sid & 1))
-          seg_fx<K_SL>(P, F.rec, s, en, b, E, X, xthr, xp, acc);
+          seg_fx<K_SL>(P, F, F.rec, s, en, b, E, X, xthr, xp, acc);
         else if (KMODE ? KMODE == K_DL : true)
-          seg_fx<K_DL>(P, F.rec, s, en, b, E, X, xthr, xp, acc);
+          seg_fx<K_DL>(P, F, F.rec, s, en, b, E, X, xthr, xp, acc);
         else
-          seg_fx<K_SLDL>(P, F.rec, s, en, b, E, X, xthr, xp, acc);
+          seg_fx<K_SLDL>(P, F, F.rec, s, en, b, E, X, xthr, xp, acc);
       }
       if (c0 + lane < ncol)
 #pragma unroll
@@ -284,7 +285,9 @@ __global__ void k_fx_range(int64_t ns, const double *__restrict__ src, int64_t n
   if ((threadIdx.x & 31) == 0) atomicMax(&st->field, f);
 }
 
-__global__ void k_pack_fx(int64_t ns, const double *__restrict__ src, const double *__restrict__ f,
+// Records of the sources; trg: the targets whose inexact coordinates are counted too.
+__global__ void k_pack_fx(int64_t ns, const double *__restrict__ src, int64_t nt,
+                          const double *__restrict__ trg, const double *__restrict__ f,
                           const double *__restrict__ nrm, const double *__restrict__ phi,
                           const double *__restrict__ w, double csl, double cdl,
                           FxState *__restrict__ st, SrcFx *__restrict__ rec) {
@@ -303,27 +306,37 @@ __global__ void k_pack_fx(int64_t ns, const double *__restrict__ src, const doub
       n[k] = phi ? nrm[3 * j + k] : 0.0;
       p[k] = phi ? wj * cdl * phi[3 * j + k] : 0.0;
     }
-    const int eq = fx_block(R.q, R.qh, R.ql), en = fx_block(n, R.nh, R.nl),
-              ep = fx_block(p, R.ph, R.pl);
+    const int eq = fx_block(R.q, R.qh, R.ql, R.thr, kFxRoundQ),
+              en = fx_block(n, R.nh, R.nl, R.thr, kFxRoundN),
+              ep = fx_block(p, R.ph, R.pl, R.thr, kFxRoundP);
     const bool ok = eq <= kFxMaxExp && eq >= -kFxMaxExp && en <= kFxMaxExp && en >= -kFxMaxExp &&
                     ep <= kFxMaxExp && ep >= -kFxMaxExp;
     R.eq = (int16_t)eq;
     R.epn = (int16_t)(en + ep);
     bad |= !ok;
-    inexact += R.thr != kFxExact;
+    inexact += R.thr >= kFxInexact;
     rec[j] = R;
   }
   if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) st->bad = 1;
   inexact = __reduce_add_sync(kFull, inexact);
   if (inexact && (threadIdx.x & 31) == 0) atomicAdd(&st->inexact, inexact);
+  int trg_inexact = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nt;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    uint32_t thr = kFxExact;
+    for (int k = 0; k < 3; ++k) fx_coord(trg[3 * i + k], E, thr);
+    trg_inexact += thr != kFxExact;
+  }
+  trg_inexact = __reduce_add_sync(kFull, trg_inexact);
+  if (trg_inexact && (threadIdx.x & 31) == 0) atomicAdd(&st->trg_inexact, trg_inexact);
 }
 
 __global__ void k_pack_fp64(int64_t ns, const double *__restrict__ src,
                             const double *__restrict__ f, const double *__restrict__ nrm,
                             const double *__restrict__ phi, const double *__restrict__ w,
                             double csl, double cdl, const FxState *__restrict__ fx,
-                            SrcRec64 *__restrict__ rec) {
-  if (fx && fx_use(*fx, ns)) return;
+                            int64_t nt, SrcRec64 *__restrict__ rec) {
+  if (fx && fx_use(*fx, ns, nt)) return;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
        j += (int64_t)gridDim.x * blockDim.x) {
     SrcRec64 R;
@@ -346,7 +359,7 @@ static int pack_grid(int64_t n) {
 void launch_pack_fp64(int64_t ns, const double *src, const double *f, const double *nrm,
                       const double *phi, const double *w, double csl, double cdl, SrcRec64 *rec,
                       cudaStream_t st) {
-  k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, nullptr, rec);
+  k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, nullptr, 0, rec);
   count_launches(1);
 }
 
@@ -359,7 +372,7 @@ void launch_fx_range(int64_t ns, const double *src, int64_t nt, const double *tr
 void launch_fx_records(int64_t n, const double *pts, const double *f, const double *nrm,
                        const double *phi, const double *w, double csl, double cdl, FxState *fx,
                        SrcFx *rec, cudaStream_t st) {
-  k_pack_fx<<<pack_grid(n), 256, 0, st>>>(n, pts, f, nrm, phi, w, csl, cdl, fx, rec);
+  k_pack_fx<<<pack_grid(n), 256, 0, st>>>(n, pts, 0, nullptr, f, nrm, phi, w, csl, cdl, fx, rec);
   count_launches(1);
 }
 
@@ -367,9 +380,10 @@ void launch_pack_fx(int64_t ns, const double *src, int64_t nt, const double *trg
                     const double *nrm, const double *phi, const double *w, double csl, double cdl,
                     FxState *fx, SrcFx *recfx, SrcRec64 *rec, cudaStream_t st) {
   launch_fx_range(ns, src, nt, trg, fx, st);
-  launch_fx_records(ns, src, f, nrm, phi, w, csl, cdl, fx, recfx, st);
-  k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, fx, rec);
-  count_launches(1);
+  k_pack_fx<<<pack_grid(ns > nt ? ns : nt), 256, 0, st>>>(ns, src, nt, trg, f, nrm, phi, w, csl, cdl,
+                                                          fx, recfx);
+  k_pack_fp64<<<pack_grid(ns), 256, 0, st>>>(ns, src, f, nrm, phi, w, csl, cdl, fx, nt, rec);
+  count_launches(2);
 }
 
 cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,

@@ -20,8 +20,11 @@
 //
 // What fixed point cannot hold takes the FP64 pair (fx_slow): a coordinate
 // below 2^(E - 10) in magnitude may have bits under the quantum ("inexact"),
-// which matters only for a pair closer than 2^(E - 8); pairs closer than
-// 2^(E - 30) (coincident ones among them) always take it.
+// which matters for a pair closer than 2^(E - 8) and for one whose difference is
+// nearly perpendicular to n or psi component by component (fx_faint_dot: a flat
+// wall seen from just beside it; with exact coordinates its dot products are summed
+// exactly instead); pairs closer than 2^(E - 26) (coincident ones among them)
+// always take it.
 #pragma once
 
 #include <cmath>
@@ -114,7 +117,8 @@ constexpr uint32_t kFxLow = 0x3fffffffu;  // the low part: 30 bits
 
 // A pair whose largest |d_k| has a high word below both points' thresholds
 // takes the FP64 form.
-constexpr uint32_t kFxExact = 1u;          // exact coordinates: |d| < 2^32 quanta
+constexpr uint32_t kFxExact = 1u;          // exact coordinates: |d| < 2^32 quanta (2^36 with)
+constexpr uint32_t kFxRoundQ = 2u, kFxRoundN = 4u, kFxRoundP = 8u;  // these: q, n, psi lost bits
 constexpr uint32_t kFxInexact = 1u << 22;  // an inexact coordinate: |d| < 2^54 quanta
 constexpr uint32_t kFxNever = ~0u;         // nothing of the point fits
 
@@ -136,21 +140,24 @@ constexpr int kFxMaxExp = 300;
 // exponent field of a coordinate, whether something does not fit, and the
 // sources with an inexact coordinate.
 struct FxState {
-  int32_t field, bad, inexact;
+  int32_t field, bad, inexact, trg_inexact;
 };
 // What the FP64 engines need besides EngineParams.
 struct FxParams {
   const SrcFx *rec;
   const FxState *state;
-  int64_t ns;  // sources
+  int64_t ns, nt;                // sources, targets
+  const double *nrm, *phi, *w;   // the caller's (may be NULL where the kind has no use for it)
+  double cdl;                    // double-layer factor
 };
 FX_HD int fx_exp(const FxState &s) { return s.field - 1022; }
 // Points with bits below the grid (coordinates small against the largest one)
-// send their close pairs to the FP64 form; with more than one source in 16
-// like that the plain FP64 engine takes the call.
-FX_HD bool fx_use(const FxState &s, int64_t ns) {
+// send their close and faint pairs to the FP64 form; with more than one source or
+// target in 16 like that the plain FP64 engine takes the call.
+FX_HD bool fx_use(const FxState &s, int64_t ns, int64_t nt = 0) {
   const int E = fx_exp(s);
-  return !s.bad && E <= kFxMaxExp && E >= -kFxMaxExp && (int64_t)s.inexact * 16 <= ns;
+  return !s.bad && E <= kFxMaxExp && E >= -kFxMaxExp && (int64_t)s.inexact * 16 <= ns &&
+         (int64_t)s.trg_inexact * 16 <= nt;
 }
 
 // A coordinate on the grid of exponent E (|v| < 2^E, kFxMaxExp >= |E|),
@@ -188,8 +195,9 @@ FX_HD int64_t fx_coord(double v, int E, uint32_t &thr) {
 FX_HD int fx_field(double v) { return (int)((fx_to_bits(v) >> 52) & 0x7ff); }
 
 // Block fixed point of a vector; returns its exponent e (|v_k| < 2^e; 0 for a
-// zero vector).
-FX_HD int fx_block(const double (&v)[3], int32_t (&h)[3], int32_t (&l)[3]) {
+// zero vector).  `flag` is added to thr where a component loses bits.
+FX_HD int fx_block(const double (&v)[3], int32_t (&h)[3], int32_t (&l)[3], uint32_t &thr,
+                   uint32_t flag) {
   int ef = 0;
   for (int k = 0; k < 3; ++k) ef = ef > fx_field(v[k]) ? ef : fx_field(v[k]);
   const int e = ef ? ef - 1022 : 0;
@@ -200,14 +208,20 @@ FX_HD int fx_block(const double (&v)[3], int32_t (&h)[3], int32_t (&l)[3]) {
     if (f) {  // (a subnormal or zero component is dropped)
       const uint64_t m = (u & 0xfffffffffffffull) | (1ull << 52);  // m 2^(f - 1075)
       const int s = f - 1015 - e;                                  // to quanta of 2^(e - 60): <= 7
+      if (s < 0 && (s <= -54 || (m & ((1ull << -s) - 1)))) thr |= flag;
       if (s >= 0) V = (int64_t)(m << s);
       else if (s > -54) V = (int64_t)((m + (1ull << (-s - 1))) >> -s);
       if (u >> 63) V = -V;
     }
+    if (!f && (u << 1)) thr |= flag;
     h[k] = (int32_t)(V >> 30);
     l[k] = (int32_t)((uint32_t)V & kFxLow);
   }
   return e;
+}
+FX_HD int fx_block(const double (&v)[3], int32_t (&h)[3], int32_t (&l)[3]) {
+  uint32_t thr = 0u;
+  return fx_block(v, h, l, thr, 0u);
 }
 
 // ---------------------------------------------------------------- conversions
@@ -262,6 +276,44 @@ FX_HD int64_t fx_norm2(const int32_t (&h)[3], const int32_t (&l)[3]) {
   hh = fx_mad(h[2], h[2], hh);
   cr = fx_mad(h[2], l[2], cr);
   return hh + (cr >> 29);
+}
+
+// A dot product's error is absolute, some 2^-59 of the vectors' largest components, where
+// FP64's is relative to its products.  So a dot product V far below full scale (2^58 to
+// 2^60) is looked at again: where larger products cancel FP64 loses as much and V stands;
+// where each of them is small (a plane seen from just beside it) the products are summed
+// exactly, if the coordinates and the vector b are exact, and the pair takes the FP64 form
+// otherwise (false).  eb: V's exponent as for fx_to_double; exact: see above.
+constexpr uint32_t kFxFaint = 1u << 18;  // 2^50 in the units of a dot product
+FX_HD bool fx_faint(int64_t V) {
+  const int32_t hi = (int32_t)(V >> 32);
+  return (uint32_t)(hi ^ (hi >> 31)) < kFxFaint;
+}
+FX_HD bool fx_faint_dot(int64_t V, const int64_t (&J)[3], const int32_t (&dh)[3],
+                        const int32_t (&bh)[3], const int32_t (&bl)[3], bool exact, int eb,
+                        double &dot) {
+  uint64_t size = 0;
+  for (int k = 0; k < 3; ++k)
+    size += (uint64_t)(uint32_t)(dh[k] < 0 ? -dh[k] : dh[k]) *
+            (uint32_t)(bh[k] < 0 ? -bh[k] : bh[k]);
+  if ((uint32_t)(size >> 32) >= kFxFaint) {
+    dot = fx_to_double(V, eb);
+    return true;
+  }
+  if (!exact) return false;
+  __int128 sum = 0;  // units of 2^-63 of V's
+  for (int k = 0; k < 3; ++k) sum += (__int128)J[k] * (((int64_t)bh[k] << 30) + bl[k]);
+  const uint64_t sign = (uint64_t)(sum >> 127), hi = (uint64_t)(sum >> 64) ^ sign,
+                 lo = (uint64_t)sum ^ sign;
+  const int s = hi >> 32 ? 66 - fx_clz((uint32_t)(hi >> 32))  // sum 2^-s has at most 62 bits
+                : hi     ? 34 - fx_clz((uint32_t)hi)
+                         : (lo >> 62 ? 2 : 0);
+  dot = fx_to_double((int64_t)(sum >> s), eb - 63 + s);
+  return true;
+}
+// Whether the coordinates of both points and the vectors flagged are exact.
+FX_HD bool fx_is_exact(uint32_t xthr, uint32_t ythr, uint32_t flag) {
+  return (xthr | ythr) < kFxInexact && !((xthr | ythr) & flag);
 }
 
 // 1/sqrt of W 2^-60, W in [2^58, 2^62): Y 2^(b - 62) with Y in [2^61, 2^62].
@@ -345,6 +397,18 @@ FX_HD bool fx_pair(const int64_t (&x)[3], uint32_t xthr, int E, const SrcFx &S, 
   int32_t dh[3], dl[3];
   int a, b, z;
   if (!fx_diff(x, S.y, xthr, S.thr, E, J, dh, dl, a)) return false;
+  double dp = 0.0, dn = 0.0;
+  if (KIND & K_DL) {
+    // dots in units of 2^(e - 60): field 1086 + e - 60
+    const int64_t vp = fx_dot(dh, dl, S.ph, S.pl), vn = fx_dot(dh, dl, S.nh, S.nl);
+    if (!fx_faint(vp)) dp = fx_to_double(vp, 1026 + S.epn - a);
+    else if (!fx_faint_dot(vp, J, dh, S.ph, S.pl, fx_is_exact(xthr, S.thr, kFxRoundP),
+                           1026 + S.epn - a, dp))
+      return false;
+    if (!fx_faint(vn)) dn = fx_to_double(vn, 1026);
+    else if (!fx_faint_dot(vn, J, dh, S.nh, S.nl, fx_is_exact(xthr, S.thr, kFxRoundN), 1026, dn))
+      return false;
+  }
   double D[3];
   for (int k = 0; k < 3; ++k) D[k] = fx_to_double(J[k], 1023);  // J 2^-63
   const uint64_t Y = fx_rsqrt(fx_norm2(dh, dl), b);             // 1/R = Y 2^(b - 62)
@@ -353,9 +417,6 @@ FX_HD bool fx_pair(const int64_t (&x)[3], uint32_t xthr, int E, const SrcFx &S, 
   const double ri2 = fx_round(Z, 1022 + 2 * b - z);
   double c;
   if (KIND & K_DL) {
-    // dots in units of 2^(e - 60): field 1086 + e - 60
-    const double dp = fx_to_double(fx_dot(dh, dl, S.ph, S.pl), 1026 + S.epn - a);
-    const double dn = fx_to_double(fx_dot(dh, dl, S.nh, S.nl), 1026);
     if (KIND & K_SL) {
       const double dq = fx_to_double(fx_dot(dh, dl, S.qh, S.ql), 1026 + S.eq);
       c = fx_fma(dp * dn, ri2, dq) * ri2;

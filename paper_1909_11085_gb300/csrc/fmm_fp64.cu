@@ -153,8 +153,8 @@ __device__ __forceinline__ void add_points(const Pass &P, EvalSmem &sm, const do
         nn[k] = P.phi ? P.nrm[3 * i + k] : 0.0;
         pp[k] = P.phi ? wd * P.phi[3 * i + k] : 0.0;
       }
-      const int eq = fx_block(S.q, S.qh, S.ql), en = fx_block(nn, S.nh, S.nl),
-                ep = fx_block(pp, S.ph, S.pl);
+      const int eq = fx_block(S.q, S.qh, S.ql), en = fx_block(nn, S.nh, S.nl, thr, kFxRoundN),
+                ep = fx_block(pp, S.ph, S.pl, thr, kFxRoundP);
       if (!(in_range(eq) && in_range(en) && in_range(ep))) thr = kFxNever;
       S.eq = (int16_t)eq;
       S.epn = (int16_t)(en + ep);

@@ -60,6 +60,7 @@ stk_status fail(stk_status s, const char *msg) {
   } while (0)
 
 constexpr double kPi = 3.14159265358979323846;
+constexpr double kCdl = 6.0 / (8.0 * kPi);  // double-layer factor
 constexpr int64_t kMaxN = 0x7fffffffLL;
 constexpr int64_t kSpinLimit = 4000000000LL;  // SM cycles, about 2 s at 2 GHz
 
@@ -379,7 +380,9 @@ SideStream *fork_side(cudaStream_t st) {
 // Engine launch common to all forms.
 // direct_out (optional): with one part and targets in caller order, the
 // engines write the caller's output instead of the partial buffer (no finish).
-stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
+// nrm, phi, w: the caller's source arrays (for the FP64 form).
+stk_status run_engine(const Plan &p, void *ws, EngineParams &P, const double *nrm,
+                      const double *phi, const double *w, cudaStream_t st,
                       double *direct_out = nullptr) {
   DevInfo di;
   CU(dev_info(di));
@@ -414,7 +417,7 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
   } else {
     P.rec64 = at<SrcRec64>(ws, p.rec);
     const FxParams F{at<SrcFx>(ws, p.recfx), reinterpret_cast<const FxState *>(counters + kFxCounter),
-                     p.ns};
+                     p.ns, P.trg64 == P.src64 ? 0 : p.nt, nrm, phi, w, kCdl};
     int64_t grid_fx = (int64_t)di.sms * di.occ_fx;
     if (grid_fx > need) grid_fx = need;
     CU(launch_engine_fp64(P, F, (int)grid, (int)(grid_fx < 1 ? 1 : grid_fx), st));
@@ -430,7 +433,7 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, cudaStream_t st,
 stk_status pack(const Plan &p, void *ws, const double *src, const double *f, const double *nrm,
                 const double *phi, const double *w, const double *h, const double *trg, double mu,
                 double alpha, cudaStream_t st) {
-  const double csl = 1.0 / (8.0 * kPi * mu), cdl = 6.0 / (8.0 * kPi);
+  const double csl = 1.0 / (8.0 * kPi * mu), cdl = kCdl;
   if (p.mixed)
     launch_pack_mixed(p.ns, src, f, nrm, phi, w, h, alpha, csl, cdl, src, at<SrcRec>(ws, p.rec),
                       st);
@@ -532,7 +535,7 @@ stk_status direct_common(int32_t kinds, const double *src, const double *f, cons
   P.range_ptr = at<int64_t>(ws, p.range);
   P.kind = kinds;
   P.kind_alternating = 0;
-  s = run_engine(p, ws, P, st);
+  s = run_engine(p, ws, P, nrm, phi, w, st);
   if (s != STK_OK) return s;
   launch_finish(nt, p.nseg_ranges, at<double>(ws, p.part), P.tperm, o->accumulate, out, st);
   CU(cudaGetLastError());
@@ -798,7 +801,7 @@ stk_status stokes_p2p_leaflists(const double *pts, const double *f, const double
   // points are targets in caller order and there is one part: without
   // accumulation the engines write out directly
   const bool direct = !opts->accumulate;
-  s = run_engine(p, ws, P, st, direct ? out : nullptr);
+  s = run_engine(p, ws, P, nrm, phi, w, st, direct ? out : nullptr);
   if (s != STK_OK) return s;
   if (!direct) launch_finish(n, 1, at<double>(ws, p.part), nullptr, opts->accumulate, out, st);
   CU(cudaGetLastError());
@@ -861,7 +864,7 @@ stk_status stokes_batched_eval(const double *pts, const double *f, const double 
   P.range_ptr = at<int64_t>(ws, p.range);
   P.kind = K_SLDL;
   P.kind_alternating = 1;
-  s = run_engine(p, ws, P, st);
+  s = run_engine(p, ws, P, nrm, phi, w, st);
   if (s != STK_OK) return s;
   launch_finish(n, 1, at<double>(ws, p.part), P.tperm, opts->accumulate, out, st);
   CU(cudaGetLastError());
