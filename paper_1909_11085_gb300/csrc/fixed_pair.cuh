@@ -195,12 +195,16 @@ FX_HD int64_t fx_coord(double v, int E, uint32_t &thr) {
 FX_HD int fx_field(double v) { return (int)((fx_to_bits(v) >> 52) & 0x7ff); }
 
 // Block fixed point of a vector; returns its exponent e (|v_k| < 2^e; 0 for a
-// zero vector).  `flag` is added to thr where a component loses bits.
+// zero vector, -1022, which fits no form, for one of subnormals).  `flag` is added to thr where a component loses bits.
 FX_HD int fx_block(const double (&v)[3], int32_t (&h)[3], int32_t (&l)[3], uint32_t &thr,
                    uint32_t flag) {
   int ef = 0;
-  for (int k = 0; k < 3; ++k) ef = ef > fx_field(v[k]) ? ef : fx_field(v[k]);
-  const int e = ef ? ef - 1022 : 0;
+  uint64_t any = 0;
+  for (int k = 0; k < 3; ++k) {
+    ef = ef > fx_field(v[k]) ? ef : fx_field(v[k]);
+    any |= fx_to_bits(v[k]) << 1;
+  }
+  const int e = ef || any ? ef - 1022 : 0;
   for (int k = 0; k < 3; ++k) {
     const uint64_t u = fx_to_bits(v[k]);
     const int f = (int)((u >> 52) & 0x7ff);

@@ -1,7 +1,8 @@
-"""FP64 double layers and gradients on a flat wall at targets from far to
+"""FP64 sums at the ends of the fixed point pair: double layers and gradients on a flat wall at targets from far to
 very close above it, where every pair's difference is nearly perpendicular to the
 normal: coordinates off the fixed point grid (a wall through the origin), on it
-(a wall at z = 10) and a mixture, against the oracle at the FP64 sums' bar."""
+(a wall at z = 10) and a mixture, and densities below FP64's normal range, against the
+oracle at the FP64 sums' bar."""
 import numpy as np
 import pytest
 
@@ -62,3 +63,14 @@ def test_gradients(lib, h, z0):
         ref = oracle.sldl_grad(src, None, nrm, phi, w, trg, g, 1.0)
         for k in ("phi", "y", "n", "x"):
             assert rel_l2(got[k].cpu().numpy(), ref["grad_" + k]) <= GRAD64
+
+
+def test_subnormal_densities(lib):
+    """Densities and velocities of some 1e-309, whose rounding of 5e-324 is far below the bar."""
+    rng = np.random.default_rng(43)
+    src, f = rng.uniform(-1, 1, (70, 3)), rng.uniform(-1, 1, (70, 3)) * 1e-309
+    w = np.ones(70)
+    S, F, Wt = cuda(src, f, w)
+    got, ref = lib.sl(S, F, Wt, None, 1.0, precision="fp64").cpu().numpy(), oracle.sl(src, f, w, src)
+    s = np.abs(ref).max()
+    assert s > 0 and rel_l2(got / s, ref / s) <= TOL64
