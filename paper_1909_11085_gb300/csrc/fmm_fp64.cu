@@ -19,8 +19,13 @@
 // add_vlist sums 12 products per surface point pair.  Both are block fixed
 // point of 54 bits in two parts of 27, so that a product is 3 integer
 // multiply-adds (16 cycles against the 68 of an FP64 one) and a sum over 64
-// points is exact; what is lost is the 2^-55 of the largest value each operand
-// is rounded by, less than the partial sums' roundings in FP64.
+// points is exact.  What is lost is relative to the largest kernel value of an
+// offset times the largest density of a box: 2^-55 of each operand's rounding and,
+// of either sign, up to 2^-54 for the product of the low parts, where a partial sum in
+// FP64 is rounded by 2^-53 of itself.  So that forces and sources, on one exponent, are
+// of one size, the viscosity goes with the forces: the table holds the Stokeslet of
+// viscosity 1 (errors below 1e-15 at viscosities of 1e-9 to 1e6, random operators; with
+// the viscosity in the table 1.6e-9 at 1e-9).
 //
 // 65,524 points, p = 4 (131,570 V-list pairs, 4,532 W-list): see k_f64_eval.
 #include "fixed_pair.cuh"
@@ -242,11 +247,12 @@ __device__ __forceinline__ void table_values(const Pass &P, int o, int m, double
     r2 = fma(d[k], d[k], r2);
   }
   const double ri = r2 > 0.0 ? 1.0 / sqrt(r2) : 0.0, ri3 = ri * ri * ri;
+  const double csl = 0.5 * P.csrc;  // of viscosity 1
   int c = 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = a; b < 3; ++b) v[c++] = P.csl * ((a == b ? ri : 0.0) + d[a] * d[b] * ri3);
+    for (int b = a; b < 3; ++b) v[c++] = csl * ((a == b ? ri : 0.0) + d[a] * d[b] * ri3);
 #pragma unroll
   for (int a = 0; a < 3; ++a) v[c++] = P.csrc * d[a] * ri3;
 }
@@ -282,26 +288,29 @@ __global__ void __launch_bounds__(kTableThreads) k_f64_setup(Pass P) {
 }
 
 // UC2E, a CTA per box: the upward density, and for the kernel table its fixed
-// point form scaled to half-width 1 (forces by 1 / r, sources by 1 / r^2).
+// point form scaled to half-width 1 and viscosity 1 (forces by 1 / (r mu), sources by
+// 1 / r^2).
 __global__ void __launch_bounds__(256) k_f64_uc2e(Pass P) {
   __shared__ int top;
   const int rows = P.nc * P.ns;
   const int32_t b = P.box0 + blockIdx.x;
-  if (threadIdx.x == 0) top = 0;
+  if (threadIdx.x == 0) top = -1;
   for (int i = threadIdx.x; i < rows; i += blockDim.x) UC2E()(P, (int64_t)blockIdx.x * rows + i);
   if (!P.ktab) return;
   __syncthreads();
   double c[3], r;
   box_geom(P.t, b, P.depth, c, r);
-  const double sf = 1.0 / r, sq = 1.0 / (r * r);
+  const double sf = P.csl / (0.5 * P.csrc) / r, sq = 1.0 / (r * r);
   const double *u = P.up + (size_t)b * rows;
-  int f = 0;
-  for (int i = threadIdx.x; i < rows; i += blockDim.x)
-    f = max(f, fx_field(u[i] * ((i % P.nc) < 3 ? sf : sq)));
+  int f = -1;  // -1: all zero; 0: subnormal
+  for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+    const double v = u[i] * ((i % P.nc) < 3 ? sf : sq);
+    if (v != 0.0 || u[i] != 0.0) f = max(f, fx_field(v));
+  }
   f = __reduce_max_sync(kFull, f);
   if ((threadIdx.x & 31) == 0) atomicMax(&top, f);
   __syncthreads();
-  const int e = top ? top - 1022 : 0;
+  const int e = top >= 0 ? top - 1022 : 0;
   const bool ok = in_range(e);  // so that the sums' FP64 exponents are
   if (threadIdx.x == 0) P.eexp[b] = ok ? e : kBadExp;
   for (int i = threadIdx.x; i < 4 * P.ns; i += blockDim.x) {
