@@ -329,8 +329,9 @@ __device__ __forceinline__ void copy16(void *dst, const void *src) {
 
 constexpr int kM2lBlock = 64;  // surface points per exact sum: 256 products of 2^52 fit 63 bits
 
-size_t m2l_buffer(int p, int ns) {
-  return sizeof(int2_t) * (9 * (size_t)table_pad(p) + 4 * (size_t)ns);
+// Two buffers of a table and a box's densities, and the points' lattice positions.
+size_t m2l_smem(int p, int ns) {
+  return 2 * sizeof(int2_t) * (9 * (size_t)table_pad(p) + 4 * (size_t)ns) + sizeof(int32_t) * ns;
 }
 
 // Adds the V-list densities of box b at its check point t (source points of
@@ -550,10 +551,13 @@ cudaError_t far_field_fp64(const Pass &P0, const int32_t *depth_ptr, int32_t max
   };
   k_f64_setup<<<P.ktab ? 344 : 1, kTableThreads, 0, st>>>(P);
   ++launches;
-  const size_t table_smem = P.ktab ? 2 * m2l_buffer(P.p, ns) + sizeof(int32_t) * ns : 0;
+  const size_t table_smem = P.ktab ? m2l_smem(P.p, ns) : 0;
   if (table_smem) {
+    // the limit belongs to the kernel, not to the call: one value for every order, so that
+    // host threads with plans of different orders do not lower each other's
     const cudaError_t e = cudaFuncSetAttribute(
-        k_f64_eval<E_DCHK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)table_smem);
+        k_f64_eval<E_DCHK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)m2l_smem(kTableMaxP, surface_count(kTableMaxP)));
     if (e != cudaSuccess) return e;
   }
   k_f64_eval<E_S2M><<<dim3(P.t.nleaf, nch), kEvalThreads, 0, st>>>(P);
