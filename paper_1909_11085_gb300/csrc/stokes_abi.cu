@@ -226,7 +226,9 @@ TileConfig form_tile(const stk_opts *o) {
   if (o->precision != STK_MIXED) t.item_max /= kFp64ItemDiv;
   return t;
 }
-// The smallest item size of a precision: bounds the item count of any tile.
+// The smallest item size of a precision: bounds the item count of any tile (the
+// autotuners run them all in one workspace; the direct sums, which have none, count
+// their own tile's).
 int least_item(bool mixed) { return mixed ? kMinItemMax : kMinItemMax / kFp64ItemDiv; }
 
 stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
@@ -252,7 +254,7 @@ stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
   if (p.nsplit < 1) p.nsplit = 1;
   if (p.mixed && o->source_splits == 0) p.nsub = split_parts(nt, ns, p.nsplit, di);
   p.nseg_ranges = p.nsplit * p.nsub;
-  p.max_items = ((nt + least_item(p.mixed) - 1) / least_item(p.mixed)) * p.nseg_ranges;
+  p.max_items = ((nt + p.tile.item_max - 1) / p.tile.item_max) * p.nseg_ranges;
   p.sort_targets = p.mixed;
   p.sort_items = false;
   p.ngroup = 0;
