@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_near(AdjParams A) {
 // ---------------------------------------------------------------- FP64 pass
 template <bool SRC>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_fp64(AdjParams A) {
-  if (fx_adj_use(*A.fx, A.nout + A.nin)) return;  // k_adj_fx does the call
+  if (A.fx && fx_adj_use(*A.fx, A.nout + A.nin)) return;  // k_adj_fx does the call
   constexpr int NA = NAcc<SRC>::value;
   __shared__ double sP[kAdjThreads][3];
   __shared__ double sA[kAdjThreads][3];
@@ -683,10 +683,13 @@ void launch_adj_nexp(int64_t ns, const double *nrm, int32_t *nexp, cudaStream_t 
 
 template <bool SRC>
 static void launch_adj_fx(const AdjParams &A, dim3 grid, cudaStream_t st) {
-  if (!A.has_dl) k_adj_fx<SRC, K_SL><<<grid, kAdjThreads, 0, st>>>(A);
-  else if (!A.has_sl) k_adj_fx<SRC, K_DL><<<grid, kAdjThreads, 0, st>>>(A);
-  else k_adj_fx<SRC, K_SLDL><<<grid, kAdjThreads, 0, st>>>(A);
-  k_adj_fp64<SRC><<<grid, kAdjThreads, 0, st>>>(A);  // the device picks one of them
+  if (A.fx) {
+    if (!A.has_dl) k_adj_fx<SRC, K_SL><<<grid, kAdjThreads, 0, st>>>(A);
+    else if (!A.has_sl) k_adj_fx<SRC, K_DL><<<grid, kAdjThreads, 0, st>>>(A);
+    else k_adj_fx<SRC, K_SLDL><<<grid, kAdjThreads, 0, st>>>(A);
+    count_launches(1);
+  }
+  k_adj_fp64<SRC><<<grid, kAdjThreads, 0, st>>>(A);  // with A.fx the device picks one of them
 }
 
 template <bool SRC>
@@ -714,7 +717,6 @@ cudaError_t launch_adjoint(bool mixed, bool src_major, const AdjParams &A, cudaS
   } else {
     if (src_major) launch_adj_fx<true>(A, grid, st);
     else launch_adj_fx<false>(A, grid, st);
-    count_launches(1);
   }
   count_launches(1);
   return cudaGetLastError();

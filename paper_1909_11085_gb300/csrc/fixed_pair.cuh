@@ -145,7 +145,7 @@ struct FxState {
 // What the FP64 engines need besides EngineParams.
 struct FxParams {
   const SrcFx *rec;
-  const FxState *state;
+  const FxState *state;          // NULL: the plain engine alone
   int64_t ns, nt;                // sources, targets
   const double *nrm, *phi, *w;   // the caller's (may be NULL where the kind has no use for it)
   double cdl;                    // double-layer factor

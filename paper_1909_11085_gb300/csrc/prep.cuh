@@ -90,7 +90,7 @@ struct AdjParams {
   int32_t near_cap;
   float *oframe;           // [nout][9]: local coordinates and the CTA frame origin (hi, lo)
   // FP64 form: fixed point records of both point sets, and the sources' normals'
-  // exponents
+  // exponents (fx NULL: the plain form alone)
   const FxState *fx;
   const SrcFx *out_fx, *in_fx;
   const int32_t *nexp;
@@ -113,7 +113,8 @@ inline int engine_mixed_form(const EngineParams &P) {
 }
 // Resident CTAs per SM by form.
 cudaError_t engine_mixed_occupancy(int (&blocks_per_sm)[kEngineForms]);
-// Launches both FP64 engines (grids of resident CTAs); *F.state picks one.
+// Launches both FP64 engines (grids of resident CTAs), of which *F.state picks one, or
+// without F.state the plain one.
 cudaError_t launch_engine_fp64(const EngineParams &P, const FxParams &F, int grid, int grid_fx,
                                cudaStream_t stream);
 cudaError_t engine_fp64_occupancy(int *blocks_per_sm, int *blocks_per_sm_fx);

@@ -122,6 +122,7 @@ struct Plan {
   bool sort_targets = false;
   bool sort_items = false;
   bool small = false;  // the small direct form (direct_small.cu)
+  bool fx = false;     // FP64: the fixed point engine where the inputs fit it
   int32_t ngroup = 0;
   // offsets (the counters always sit at offset 0 of the aligned workspace)
   size_t counters, rec, recfx = 0, keys_a, keys_b, vals_a, vals_b, ikeys_a, ikeys_b, ivals_a, ivals_b, hist,
@@ -189,7 +190,7 @@ void layout(Plan &p) {
     return;
   }
   p.rec = a.take((size_t)p.ns * (p.mixed ? sizeof(SrcRec) : sizeof(SrcRec64)));
-  if (!p.mixed) p.recfx = a.take((size_t)p.ns * sizeof(SrcFx));
+  if (p.fx) p.recfx = a.take((size_t)p.ns * sizeof(SrcFx));
   const int64_t nsort = p.sort_targets ? p.nt : 0;
   const int64_t nitem = p.sort_items ? p.max_items : 0;
   p.keys_a = a.take(sizeof(uint64_t) * (size_t)nsort);
@@ -219,6 +220,14 @@ void layout(Plan &p) {
     p.over = a.take(sizeof(int32_t) * mi);
   }
   p.total = a.off + 256;  // slack for re-alignment of an unaligned base
+}
+
+// FP64 sums of at most this many pairs run in the plain FP64 form alone: they are bound by
+// their launches, and fixed point and the choice on the device take more of them (24 points
+// on themselves 75 -> 57 us; from 25 on fixed point is the faster one, 65 against 75).
+constexpr double kPlainPairs = 576;
+bool takes_fx(bool mixed, int64_t ns, int64_t nt) {
+  return !mixed && (double)ns * (double)nt > kPlainPairs;
 }
 
 TileConfig form_tile(const stk_opts *o) {
@@ -258,6 +267,7 @@ stk_status plan_direct(int64_t ns, int64_t nt, const stk_opts *o, Plan &p) {
   p.sort_targets = p.mixed;
   p.sort_items = false;
   p.ngroup = 0;
+  p.fx = takes_fx(p.mixed, ns, nt);
   layout(p);
   return STK_OK;
 }
@@ -270,6 +280,7 @@ stk_status plan_p2p(int64_t n, int32_t nleaf, const stk_opts *o, Plan &p) {
   p.nsplit = 1;
   p.max_items = (int64_t)nleaf + n / least_item(p.mixed) + 1;
   p.nseg_ranges = nleaf;
+  p.fx = takes_fx(p.mixed, n, n);
   p.sort_targets = false;
   p.sort_items = true;
   p.ngroup = nleaf;
@@ -285,6 +296,7 @@ stk_status plan_batched(int64_t n, int32_t nsusp, const stk_opts *o, Plan &p) {
   p.nsplit = 1;
   p.max_items = (int64_t)nsusp + n / least_item(p.mixed) + 1;
   p.nseg_ranges = 2 * nsusp;
+  p.fx = takes_fx(p.mixed, n, n);
   p.sort_targets = p.mixed;
   p.sort_items = true;
   p.ngroup = nsusp;
@@ -418,8 +430,9 @@ stk_status run_engine(const Plan &p, void *ws, EngineParams &P, const double *nr
     CU(launch_engine_mixed(P, (int)grid, st));
   } else {
     P.rec64 = at<SrcRec64>(ws, p.rec);
-    const FxParams F{at<SrcFx>(ws, p.recfx), reinterpret_cast<const FxState *>(counters + kFxCounter),
-                     p.ns, P.trg64 == P.src64 ? 0 : p.nt, nrm, phi, w, kCdl};
+    const FxParams F{at<SrcFx>(ws, p.recfx),
+                     p.fx ? reinterpret_cast<const FxState *>(counters + kFxCounter) : nullptr, p.ns,
+                     P.trg64 == P.src64 ? 0 : p.nt, nrm, phi, w, kCdl};
     int64_t grid_fx = (int64_t)di.sms * di.occ_fx;
     if (grid_fx > need) grid_fx = need;
     CU(launch_engine_fp64(P, F, (int)grid, (int)(grid_fx < 1 ? 1 : grid_fx), st));
@@ -439,6 +452,8 @@ stk_status pack(const Plan &p, void *ws, const double *src, const double *f, con
   if (p.mixed)
     launch_pack_mixed(p.ns, src, f, nrm, phi, w, h, alpha, csl, cdl, src, at<SrcRec>(ws, p.rec),
                       st);
+  else if (!p.fx)
+    launch_pack_fp64(p.ns, src, f, nrm, phi, w, csl, cdl, at<SrcRec64>(ws, p.rec), st);
   else
     launch_pack_fx(p.ns, src, trg == src ? 0 : p.nt, trg, f, nrm, phi, w, csl, cdl,
                    reinterpret_cast<FxState *>(at<int32_t>(ws, p.counters) + kFxCounter),
@@ -547,12 +562,12 @@ stk_status direct_common(int32_t kinds, const double *src, const double *f, cons
 
 // ------------------------------------------------------------------ adjoint
 struct GradPlan {
-  bool mixed;
+  bool mixed, fx;
   int64_t ns, nt;
   int32_t nsplit_src, nsplit_trg;
   int32_t nsub_src = 1, nsub_trg = 1;
   size_t srec, trec, ska, skb, sva, svb, tka, tkb, tva, tvb, hist, hist_scan, bbox_part, bbox,
-      part_src, part_trg, counters, near_cnt = 0, near_idx = 0, oframe = 0, fx = 0, sfx = 0,
+      part_src, part_trg, counters, near_cnt = 0, near_idx = 0, oframe = 0, fxstate = 0, sfx = 0,
       tfx = 0, nexp = 0, total;
 };
 
@@ -594,6 +609,7 @@ stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
   DevInfo di;
   CU(dev_info(di));
   p.mixed = o->precision == STK_MIXED;
+  p.fx = takes_fx(p.mixed, ns, nt);
   p.ns = ns;
   p.nt = nt;
   p.nsplit_src = adj_splits(ns, nt, di);
@@ -630,8 +646,8 @@ stk_status plan_grad(int64_t ns, int64_t nt, const stk_opts *o, GradPlan &p) {
     p.near_cnt = a.take(sizeof(int32_t) * nmax);
     p.near_idx = a.take(sizeof(int32_t) * nmax * (size_t)kAdjNearCap);
     p.oframe = a.take(sizeof(float) * 9 * nmax);
-  } else {
-    p.fx = a.take(sizeof(FxState));
+  } else if (p.fx) {
+    p.fxstate = a.take(sizeof(FxState));
     p.sfx = a.take(sizeof(SrcFx) * (size_t)ns);
     p.tfx = a.take(sizeof(SrcFx) * (size_t)nt);
     p.nexp = a.take(sizeof(int32_t) * (size_t)ns);
@@ -931,13 +947,15 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
     launch_pack_fp64(ns, src, f, nrm, phi, w, csl, cdl, at<SrcRec64>(ws, p.srec), st);
     launch_pack_fp64(nt, trg, g, nullptr, nullptr, nullptr, 1.0, 0.0, at<SrcRec64>(ws, p.trec),
                      st);
-    FxState *fx = at<FxState>(ws, p.fx);
-    CU(cudaMemsetAsync(fx, 0, sizeof(FxState), st));
-    launch_fx_range(ns, src, nt, trg, fx, st);
-    launch_fx_records(ns, src, f, nrm, phi, w, csl, cdl, fx, at<SrcFx>(ws, p.sfx), st);
-    launch_fx_records(nt, trg, g, nullptr, nullptr, nullptr, 1.0, 0.0, fx, at<SrcFx>(ws, p.tfx),
-                      st);
-    if (phi) launch_adj_nexp(ns, nrm, at<int32_t>(ws, p.nexp), st);
+    if (p.fx) {
+      FxState *fx = at<FxState>(ws, p.fxstate);
+      CU(cudaMemsetAsync(fx, 0, sizeof(FxState), st));
+      launch_fx_range(ns, src, nt, trg, fx, st);
+      launch_fx_records(ns, src, f, nrm, phi, w, csl, cdl, fx, at<SrcFx>(ws, p.sfx), st);
+      launch_fx_records(nt, trg, g, nullptr, nullptr, nullptr, 1.0, 0.0, fx, at<SrcFx>(ws, p.tfx),
+                        st);
+      if (phi) launch_adj_nexp(ns, nrm, at<int32_t>(ws, p.nexp), st);
+    }
   }
   CU(cudaGetLastError());
   const int32_t *sperm = morton_perm(ns, src, ws, p.ska, p.skb, p.sva, p.svb, p.hist, p.hist_scan,
@@ -950,7 +968,7 @@ stk_status stokes_sldl_grad(const double *src, const double *f, const double *nr
   A.near_idx = p.mixed ? at<int32_t>(ws, p.near_idx) : nullptr;
   A.near_cap = kAdjNearCap;
   A.oframe = p.mixed ? at<float>(ws, p.oframe) : nullptr;
-  A.fx = at<FxState>(ws, p.fx);
+  A.fx = p.fx ? at<FxState>(ws, p.fxstate) : nullptr;
   A.nexp = at<int32_t>(ws, p.nexp);
   A.has_sl = f ? 1 : 0;
   A.has_dl = phi ? 1 : 0;
