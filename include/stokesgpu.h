@@ -55,7 +55,11 @@ typedef enum {
 
 typedef enum {
   /* FP64 accuracy: pair differences, dot products and 1/r in double or, where the
-   * inputs' range allows it, in 64-bit fixed point of no larger error. */
+   * inputs' range allows it, in 64-bit fixed point.  A fixed point pair's error is
+   * relative to its size (|q|/r, |d.psi||d.n|/r^3 or where larger products cancel in
+   * these, the products'): the sums meet double's bar of 1e-12, but a component of a
+   * pair far smaller than its others keeps fewer digits than in double.  Sums of at
+   * most 576 pairs run in double. */
   STK_FP64 = 0,
   /* FP32 pair arithmetic in per-work-item local frames with compensated
    * (two-sum) accumulation; pairs closer than near_ratio * h_j get their
@@ -84,7 +88,9 @@ void stokes_default_opts(stk_opts *opts);
  * near pairs queued per warp and evaluated in FP64 in the same launch) and one
  * that adds the splits in order (it has no waits that can run out, so its
  * workspace's status word stays 0); larger sums and any other
- * options take the work-item engine.  Both meet the same accuracy.
+ * options take the work-item engine.  Both meet the same accuracy.  With
+ * source_splits = 0 the engine cuts the sources into up to 64 x 32 parts, and its
+ * workspace holds 24 bytes per target and part and 2.1 KB per 128 targets and part.
  */
 stk_status stokes_sl_eval(const double *src, const double *f, const double *w, const double *h,
                           int64_t ns, const double *trg, int64_t nt, double mu, double *out,
@@ -213,8 +219,8 @@ stk_status stokes_graph_destroy(void *graph_exec);
  * FP64 by a second pass, in input order, so results are deterministic.  FP64: to double
  * accuracy, the pairs partly in 64-bit fixed point where the inputs' range allows it.  The
  * workspace (stokes_grad_workspace_size) holds the packed records, the
- * Morton orders, the per-split partial gradients and, for MIXED, the near-pair
- * lists.
+ * Morton orders, the partial gradients of up to 16 parts of each split and, for
+ * MIXED, the near-pair lists.
  */
 stk_status stokes_sldl_grad(const double *src, const double *f, const double *nrm,
                             const double *phi, const double *w, const double *h, int64_t ns,
@@ -294,23 +300,29 @@ stk_status stokes_upsample_patches(const double *coarse, int32_t npatch, int32_t
  * within d_eps of it, the closest point y = P(u*, v*), the unit normal
  * (dP/du x dP/dv)/|...| there and the distance (Sec. 3.2, the closest-point
  * search, steps a-e: inflated patch boxes, a spatial hash of the boxes and the
- * targets, sorted keys, Newton's method with a backtracking line search per
- * candidate patch, the nearest patch kept).  A patch is the degree-q
+ * targets, sorted keys, Newton's method per candidate patch, the nearest patch
+ * kept, ties to the lower index).  Its definition is a Gauss-Newton iteration in FP64
+ * with a backtracking line search on the barycentric interpolant; candidates are
+ * ranked in FP32 and finished in FP64 on the Chebyshev coefficients, and take the
+ * definition itself where FP32 does not settle them, where two distances or a
+ * distance and d_eps agree to rounding, and where a parameter lies 1e-9 to 1e-5 from
+ * a node's (there the definition's normals hold 1e-9 to 1e-5 and worse, as the
+ * distance from the node shrinks; elsewhere the normals are good to 1e-13).  A patch is the degree-q
  * tensor-product interpolant through its (q+1) x (q+1) Clenshaw-Curtis nodes,
  * ordered as for stokes_checkpoint_eval.  nodes [npatch (q+1)^2][3],
  * trg [nt][3]; outputs: patch [nt] (-1: none within d_eps), uv [nt][2],
  * y [nt][3], n [nt][3], dist [nt] (-1 for none).  Patch boxes are grown by
  * d_eps and 5% of their diagonal, so a target whose closest point lies
- * further outside its patch's node box than that is not found.  FP64 results; candidates
- * are ranked in FP32 and the closest points finished in FP64.
+ * further outside its patch's node box than that is not found.  FP64 results.
  * 2 <= q <= 12. */
 stk_status stokes_near_patch_search(const double *nodes, int32_t npatch, int32_t q,
                                     const double *trg, int64_t nt, double d_eps, int32_t *patch,
                                     double *uv, double *y, double *n, double *dist,
                                     void *workspace, size_t workspace_bytes, void *stream);
 /* Workspace of stokes_near_patch_search for npatch patches of order q and nt
- * targets (0 <= nt <= 2^31 - 1): the patch boxes, the sorted (cell, patch)
- * keys and a list of nt target indices. */
+ * targets (0 <= nt <= 2^31 - 1): the patch boxes, 64 bytes of coefficients and
+ * rounded coordinates per node, the sorted (cell, patch) keys, and cell, rank and
+ * list of the targets (12 bytes each). */
 stk_status stokes_near_search_workspace_size(int32_t npatch, int32_t q, int64_t nt,
                                              size_t *bytes);
 
