@@ -56,7 +56,7 @@ typedef enum {
 typedef enum {
   /* FP64 accuracy: pair differences, dot products and 1/r in double or, where the
    * inputs' range allows it, in 64-bit fixed point.  A fixed point pair's error is
-   * relative to its size (|q|/r, |d.psi||d.n|/r^3 or where larger products cancel in
+   * relative to its size (|q|/r, |d.psi||d.n|/r^4 or where larger products cancel in
    * these, the products'): the sums meet double's bar of 1e-12, but a component of a
    * pair far smaller than its others keeps fewer digits than in double.  Sums of at
    * most 576 pairs run in double. */
