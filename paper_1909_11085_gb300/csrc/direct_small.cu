@@ -15,17 +15,18 @@
 // pairs included) takes the FP64 difference and 1/|r| (near_contrib): each
 // warp queues them in shared memory and evaluates them 32 at a time, one per
 // lane, since GB300's FP64 pipe is only fed efficiently by full warps; the
-// values of one target are added in queue order (deterministic).  In the loop a warp only keeps its ballots (two words
-// per source pair and target slot); the queue is filled from them after the tile, so
-// the loop stays branch-free and unrolls (the smallest calls 20.3 -> 18.5 us).  The FP32
-// pairs run packed (two staged sources per instruction).  Each thread sums a
+// values of one target are added in queue order (deterministic).  In the loop
+// a warp only keeps its ballots (two words per source pair and target slot); the
+// queue is filled from them after the tile, so the loop stays branch-free and
+// unrolls.  The FP32 pairs run packed (two staged sources per instruction).  Each thread sums a
 // tile of 128 sources in FP32 and two-sums the tile into (hi, lo); the
 // split's (hi, lo) goes to part[split][target], and k_small_finish adds the
 // splits in order (FP32 two-sum, one conversion to FP64 at the end) and writes
 // out.  That second launch, on all SMs and overlapping the first one's end, takes
 // less than the last split of each target block adding them all did (a fence, a
-// counter cleared before every call, and one CTA reading a block's partials): a
-// call of 4,352 points on themselves 41.2 -> 34.9 us, 1,632 on themselves 22.6 -> 19.0.
+// counter cleared before every call, and one CTA reading a block's partials).  With
+// the ballots, a call of 4,352 points on themselves takes 34.9 us where it took 41.2,
+// and one of 1,632 points and 1,001 targets beside them, replayed in a graph, 19.0 (23.1).
 #include "common.cuh"
 #include "prep.cuh"
 

@@ -684,6 +684,3 @@ void launch_zero_ints(int32_t *p, int n, cudaStream_t st) {
 }
 
 }  // namespace stk
-
-namespace stk {
-}  // namespace stk
