@@ -928,7 +928,7 @@ struct NzWarpSmem {
   double res[kWarp][8];     // best so far: u, v, y, n
   double bd[kWarp];         //   distance
   int32_t bp[kWarp];        //   patch
-  int32_t bplain[kWarp];    //   whether the plain iteration gave it
+  int32_t bplain[kWarp];    //   bit 0: the distance is the plain iteration's, bit 1: only it may be
   float best[kWarp];        // no nearer patch can be further than this (FP32 bound)
   int32_t qp[kNzQueue];     // queued pairs: patch
   int32_t qs[kNzQueue];     //   target slot
@@ -1011,6 +1011,20 @@ __device__ __forceinline__ void nz_stage32(NzWarpSmem &sm, const NzPatches &Q, i
 // figures, which take the call from 1.02 to 1.27 ms (the Armijo test fails in the noise, so
 // such a pair takes all 40 iterations).
 constexpr double kNzNodeGap = 1e-5, kNzNodeNone = 1e-9;
+// kNzBeside: t lies that far from a node; kNzAtNode: closer (the ends of the square, which
+// the plain iteration meets exactly, aside).
+constexpr int kNzBeside = 1, kNzAtNode = 2;
+__device__ __forceinline__ int nz_by_node(int n1, const double *xkd, const float *xk, double t) {
+  int by = 0;
+  const float tf = (float)t;
+  for (int k = 0; k < n1; ++k)
+    if (fabsf(tf - xk[k]) < 2.f * (float)kNzNodeGap) {  // few: FP64 only for these
+      const double gap = fabs(t - xkd[k]);
+      if (gap < kNzNodeNone) by |= fabs(t) < 1.0 ? kNzAtNode : 0;
+      else if (gap < kNzNodeGap) by |= kNzBeside;
+    }
+  return by;
+}
 // Distances closer than this share of the coordinates' size could be equal, to each other
 // or to d_eps: some thirty times the rounding of the interpolants' sums.
 constexpr double kNzTie = 1e-13;
@@ -1033,30 +1047,51 @@ __device__ __forceinline__ bool nz_beside_node(int n1, const double *xkd, const 
 // thread per pair where there are many (a thread alone takes 1.8 ms for its 40 iterations,
 // a warp 0.25).
 constexpr int kNzPlainLanes = 8;
-__device__ __forceinline__ void nz_plain(NzWarpSmem &sm, const NzPatches &Q, int n1,
-                                         const double *xkd, const double *wkd, double d_eps,
-                                         bool plain, int p, int slot, int lane, double &d,
-                                         double (&res)[8]) {
+// keep: the distance alone.
+__device__ __noinline__ double nz_plain(const NzWarpSmem &sm, const NzPatches &Q, int n1,
+                                        const double *xkd, const double *wkd, double d_eps,
+                                        bool plain, bool keep, int p, int slot, int lane, double d,
+                                        double *res) {
   unsigned todo = __ballot_sync(kFull, plain);
   const size_t pn = (size_t)n1 * n1 * 3;
+  double r[8];
   if (__popc(todo) > kNzPlainLanes) {
     if (plain)
-      d = nz_pair_plain<false>(n1, Q.nodes + p * pn, xkd, wkd, sm.x[slot], d_eps, Q.rp[p], lane,
-                               res);
-    return;
+      d = nz_pair_plain<false>(n1, Q.nodes + p * pn, xkd, wkd, sm.x[slot], d_eps, Q.rp[p], lane, r);
+    if (plain && !keep)
+      for (int q = 0; q < 8; ++q) res[q] = r[q];
+    return d;
   }
   for (; todo; todo &= todo - 1) {
     const int l = __ffs(todo) - 1;
     const int lp = __shfl_sync(kFull, p, l), ls = __shfl_sync(kFull, slot, l);
-    double r[8];
     const double ld = nz_pair_plain<true>(n1, Q.nodes + lp * pn, xkd, wkd, sm.x[ls], d_eps,
                                           Q.rp[lp], lane, r);
-    if (lane == l) {
-      d = ld;
-#pragma unroll
+    if (lane == l) d = ld;
+    if (lane == l && !keep)
       for (int q = 0; q < 8; ++q) res[q] = r[q];
-    }
   }
+  return d;
+}
+
+// The distances of the lanes' pairs (p, slot) where `tie`, and of their targets' best patches so
+// far, by the plain iteration.
+__device__ __noinline__ double nz_tie(NzWarpSmem &sm, const NzPatches &Q, int n1, const double *xkd,
+                                      const double *wkd, double d_eps, bool tie, bool plain,
+                                      bool keep, int p, int slot, int lane, double d, double *res) {
+  d = nz_plain(sm, Q, n1, xkd, wkd, d_eps, tie && !plain, keep, p, slot, lane, d, res);
+  const int how = tie ? sm.bplain[slot] : 1;
+  const bool other = !(how & 1);
+  double bres[8];
+  const double bd = nz_plain(sm, Q, n1, xkd, wkd, d_eps, other, how & 2, other ? sm.bp[slot] : 0,
+                             slot, lane, 0.0, bres);
+  if (other) {
+    sm.bd[slot] = bd;
+    sm.bplain[slot] = how | 1;
+    if (!(how & 2))
+      for (int q = 0; q < 8; ++q) sm.res[slot][q] = bres[q];
+  }
+  return d;
 }
 
 // FP64 stage of the waiting pairs.
@@ -1095,7 +1130,7 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
     const bool act = e < n;
     double d = DBL_MAX, res[8];
     int p = 0, slot = -1 - lane;
-    bool plain = false;
+    bool plain = false, keep = false;
     if (act) {
       p = sm.rp[e];
       slot = sm.rs[e] & 31;
@@ -1104,11 +1139,14 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
       if (!plain) {
         d = nz_pair64<N1>(n1, Q.c32 + (size_t)p * n1 * n1, Q.c64 + 2 * (size_t)p * n1 * n1,
                           Q.meta[p], x, sm.ru[e], sm.rv[e], res);
-        plain = !(d >= 0.0) || fabs(d - d_eps) <= kNzTie * nz_size(Q.meta[p], x) ||
-                nz_beside_node(n1, xkd, xk, res[0]) || nz_beside_node(n1, xkd, xk, res[1]);
+        const int by = nz_by_node(n1, xkd, xk, res[0]) | nz_by_node(n1, xkd, xk, res[1]);
+        keep = d >= 0.0 && (by & kNzAtNode);
+        plain = !(d >= 0.0) || by == kNzBeside ||
+                fabs(d - d_eps) <= kNzTie * nz_size(Q.meta[p], x);
       }
     }
-    nz_plain(sm, Q, n1, xkd, wkd, d_eps, plain, p, slot, lane, d, res);
+    if (__any_sync(kFull, plain))
+      d = nz_plain(sm, Q, n1, xkd, wkd, d_eps, plain, keep, p, slot, lane, d, res);
     // the nearest patch of a target, ties to the lower index; pairs of one
     // target take turns.  Two patches that meet in an edge hold its nodes as the same
     // numbers, and the plain iteration finds the same distance to it from both; the
@@ -1121,25 +1159,16 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
       bool tie = false;
       if (now && sm.bp[slot] >= 0) {
         tie = fabs(d - sm.bd[slot]) <= kNzTie * nz_size(Q.meta[p], sm.x[slot]) &&
-              !(plain && sm.bplain[slot]);
+              !(plain && (sm.bplain[slot] & 1));
       }
       if (__any_sync(kFull, tie)) {
-        nz_plain(sm, Q, n1, xkd, wkd, d_eps, tie && !plain, p, slot, lane, d, res);
+        d = nz_tie(sm, Q, n1, xkd, wkd, d_eps, tie, plain, keep, p, slot, lane, d, res);
         plain = plain || tie;
-        const bool other = tie && !sm.bplain[slot];
-        double bd = 0.0, bres[8];
-        nz_plain(sm, Q, n1, xkd, wkd, d_eps, other, other ? sm.bp[slot] : 0, slot, lane, bd, bres);
-        if (other) {
-          sm.bd[slot] = bd;
-          sm.bplain[slot] = 1;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) sm.res[slot][q] = bres[q];
-        }
       }
       if (now && (d < sm.bd[slot] || (d == sm.bd[slot] && p < sm.bp[slot]))) {
         sm.bd[slot] = d;
         sm.bp[slot] = p;
-        sm.bplain[slot] = plain;
+        sm.bplain[slot] = (plain ? 1 : 0) | (keep ? 2 : 0);
 #pragma unroll
         for (int q = 0; q < 8; ++q) sm.res[slot][q] = res[q];
       }
