@@ -31,7 +31,13 @@
 // same order as by one warp for all of them, so the sums are the same; one warp
 // took up to 4.7 ms for such an item while the rest of the GPU had finished
 // (139,264 x 204,800 points, k_near: 4.73 -> 0.62 ms; 1.50 with the targets split
-// over warps that each scan the sources).
+// over warps that each scan the sources).  The U-list near field's items hold some 60
+// targets, four per warp of such a CTA, each of which tests all candidates: where so many of
+// its lists overflow that warps with an item each fill the GPU (alpha well above 1),
+// k_near_all takes all its items in one launch instead (1,048,928 points, alpha 8: 21.2 ms
+// a step with a CTA per item, 14.3 so; alpha 4: 4.93 and 4.14).
+#include <climits>
+
 #include "common.cuh"
 #include "prep.cuh"
 
@@ -210,13 +216,41 @@ __device__ __forceinline__ void finish_unit(NearSmem<TARGETS> &sm, const EngineP
   __syncwarp();
 }
 
-__global__ void __launch_bounds__(kNearWarps *kWarp, kNearMinBlocks) k_near(EngineParams P) {
+// Takes an item's listed candidates through its targets.
+__device__ __forceinline__ void test_listed(NearSmem<kItemMax> &sm, const EngineParams &P, int32_t id,
+                                            int32_t ncl, int32_t t0, int tn, const float (&oh)[3],
+                                            const float (&ol)[3], int &qn, int lane) {
+  const int32_t *cl = P.cand_list + (size_t)id * (size_t)P.cand_cap;
+  const int n_list = min(ncl, P.cand_cap);
+  for (int p0 = 0; p0 < n_list; p0 += kWarp) {
+    const int pp = p0 + lane;
+    float y[3] = {0.f, 0.f, 0.f}, hh = -1.f;  // hh < 0: idle lane, never near
+    int32_t j = -1;
+    uint32_t kb = 0;
+    if (pp < n_list) {
+      const uint32_t e = (uint32_t)cl[pp];
+      j = (int32_t)(e & 0x3fffffffu);
+      kb = e & 0xc0000000u;
+      const float4 yh = __ldg(&P.rec[j].yh);
+      y[0] = to_local(yh.x, __ldg(&P.rec[j].q.w), oh[0], ol[0]);
+      y[1] = to_local(yh.y, __ldg(&P.rec[j].n.w), oh[1], ol[1]);
+      y[2] = to_local(yh.z, __ldg(&P.rec[j].p.w), oh[2], ol[2]);
+      hh = yh.w;
+    }
+    test_candidates(sm, P, t0, tn, y, hh, j, kb, qn, lane);
+  }
+}
+
+// all_from: from this many overflowed items on, k_near_all takes all items.
+__global__ void __launch_bounds__(kNearWarps *kWarp, kNearMinBlocks) k_near(EngineParams P,
+                                                                          int all_from) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_near_over, as room comes free
   __shared__ NearSmem<kItemMax> smem[kNearWarps];
   NearSmem<kItemMax> &sm = smem[threadIdx.x / kWarp];
   const int lane = threadIdx.x & (kWarp - 1);
   const int n_items = *P.n_items;
-  if (*P.err_flag) return;  // the engine stopped early: its lists are incomplete
+  // (the engine stopped early: its lists are incomplete)
+  if (*P.err_flag || *P.over_cnt >= all_from) return;
   while (true) {
     int idx = 0;
     if (lane == 0) idx = atomicAdd(P.near_counter, 1);
@@ -236,25 +270,7 @@ __global__ void __launch_bounds__(kNearWarps *kWarp, kNearMinBlocks) k_near(Engi
     }
     load_targets(sm, P, it.t0, tn, lane);
     int qn = 0;
-    const int32_t *cl = P.cand_list + (size_t)id * (size_t)P.cand_cap;
-    const int n_list = min(ncl, P.cand_cap);
-    for (int p0 = 0; p0 < n_list; p0 += kWarp) {
-      const int pp = p0 + lane;
-      float y[3] = {0.f, 0.f, 0.f}, hh = -1.f;  // hh < 0: idle lane, never near
-      int32_t j = -1;
-      uint32_t kb = 0;
-      if (pp < n_list) {
-        const uint32_t e = (uint32_t)cl[pp];
-        j = (int32_t)(e & 0x3fffffffu);
-        kb = e & 0xc0000000u;
-        const float4 yh = __ldg(&P.rec[j].yh);
-        y[0] = to_local(yh.x, __ldg(&P.rec[j].q.w), oh[0], ol[0]);
-        y[1] = to_local(yh.y, __ldg(&P.rec[j].n.w), oh[1], ol[1]);
-        y[2] = to_local(yh.z, __ldg(&P.rec[j].p.w), oh[2], ol[2]);
-        hh = yh.w;
-      }
-      test_candidates(sm, P, it.t0, tn, y, hh, j, kb, qn, lane);
-    }
+    test_listed(sm, P, id, ncl, it.t0, tn, oh, ol, qn, lane);
     finish_unit(sm, P, it.t0, tn, it.tn_part >> 8, qn, lane);
   }
 }
@@ -279,10 +295,11 @@ struct OverSmem {
 };
 static_assert(sizeof(OverSmem) <= 48 * 1024, "no opt-in shared memory");
 
-__global__ void __launch_bounds__(kOverThreads, 2) k_near_over(EngineParams P) {
+__global__ void __launch_bounds__(kOverThreads, 2) k_near_over(EngineParams P, int all_from) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_near_all
   // (the engine's results only: complete before k_near began); it ends after k_near
   const int n_over = *P.over_cnt;
-  if (n_over == 0 || *P.err_flag) {
+  if (n_over == 0 || n_over >= all_from || *P.err_flag) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
@@ -403,18 +420,171 @@ __global__ void __launch_bounds__(kOverThreads, 2) k_near_over(EngineParams P) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// All items where many lists overflowed, an item per warp: the warp tests an overflowed item's
+// sources 32 at a time, first conservatively on the 16-byte position record; each candidate is
+// broadcast and every lane tests its targets.  (Taking these candidates through bit masks costs
+// more: most of a candidate's targets are near and would fill the queue several times.)
+constexpr int kScanT = kItemMax / kWarp;  // targets per lane
+constexpr int kScanMinBlocks = 8;
+
+struct ScanSmem {
+  NearSmem<kItemMax> n;
+  int32_t seg_start[kNearSegWin];    // window of segments, as in OverSmem
+  int32_t seg_pre[kNearSegWin];
+  int32_t seg_kind[kNearSegWin];
+};
+
+__global__ void __launch_bounds__(kNearWarps *kWarp, kScanMinBlocks) k_near_all(EngineParams P,
+                                                                                int all_from) {
+  __shared__ ScanSmem smem[kNearWarps];
+  const bool mine = *P.over_cnt >= all_from && !*P.err_flag;
+  ScanSmem &sm = smem[threadIdx.x / kWarp];
+  const int lane = threadIdx.x & (kWarp - 1);
+  const unsigned lt = (1u << lane) - 1u;
+  const int n_items = *P.n_items;
+  while (mine) {
+    int idx = 0;
+    if (lane == 0) idx = atomicAdd(P.over_head, 1);
+    idx = __shfl_sync(kFull, idx, 0);
+    if (idx >= n_items) break;
+    const int32_t id = P.item_order ? P.item_order[idx] : idx;
+    const int32_t ncl = P.cand_cnt[id];
+    const Item it = P.items[id];
+    const int tn = it.tn_part & 0xFF;
+    const float *fr = P.frames + 12 * (size_t)id;
+    float oh[3], ol[3], blo[3], bhi[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      oh[k] = fr[k];
+      ol[k] = fr[3 + k];
+      blo[k] = fr[6 + k];
+      bhi[k] = fr[9 + k];
+    }
+    const float tol0 = 4.8e-7f * (fabsf(oh[0]) + fabsf(oh[1]) + fabsf(oh[2]));
+    load_targets(sm.n, P, it.t0, tn, lane);
+    int qn = 0;
+    if (ncl >= 0) {
+      test_listed(sm.n, P, id, ncl, it.t0, tn, oh, ol, qn, lane);
+      finish_unit(sm.n, P, it.t0, tn, it.tn_part >> 8, qn, lane);
+      continue;
+    }
+    float x[kScanT][3];
+    int32_t self[kScanT];
+#pragma unroll
+    for (int t = 0; t < kScanT; ++t) {
+      const int li = lane + kWarp * t;
+      self[t] = li < tn ? sm.n.sid[li] : -1;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) x[t][k] = li < tn ? sm.n.xs[k][li] : 1e30f;
+    }
+    for (int32_t w0 = it.seg0; w0 < it.seg1; w0 += kNearSegWin) {
+      const int nw = min(kNearSegWin, it.seg1 - w0);
+      __syncwarp();
+      int32_t sz = 0;
+      if (lane < nw) {
+        const int32_t sid = P.seg_list ? P.seg_list[w0 + lane] : w0 + lane;
+        const int64_t a = P.range_ptr[sid];
+        sz = (int32_t)(P.range_ptr[sid + 1] - a);
+        sm.seg_start[lane] = (int32_t)a;
+        sm.seg_kind[lane] = seg_kind(P, sid) << 30;
+      }
+      int incl = sz;
+#pragma unroll
+      for (int o = 1; o < kWarp; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane < nw) sm.seg_pre[lane] = incl - sz;
+      const int total = __shfl_sync(kFull, incl, kWarp - 1);
+      __syncwarp();
+      for (int p0 = 0; p0 < total; p0 += kWarp) {
+        const int pp = p0 + lane;
+        bool cand = false;
+        int32_t j = 0;
+        uint32_t kb = 0;
+        float y[3] = {0.f, 0.f, 0.f}, hh = 0.f;
+        if (pp < total) {
+          int e = 0;  // last segment starting at or before pp
+#pragma unroll
+          for (int step = kNearSegWin / 2; step > 0; step >>= 1)
+            if (e + step < nw && sm.seg_pre[e + step] <= pp) e += step;
+          j = sm.seg_start[e] + (pp - sm.seg_pre[e]);
+          kb = (uint32_t)sm.seg_kind[e];
+          const SrcRec *r = P.rec + j;
+          const float4 yh = __ldg(&r->yh);
+          hh = yh.w;
+          // yh - oh differs from the local coordinate by less than tol (the dropped low parts
+          // and one rounding each)
+          const float tol = fmaf(4.8e-7f, fabsf(yh.x) + fabsf(yh.y) + fabsf(yh.z), tol0) + 1e-30f;
+          const float lo2[3] = {blo[0] - tol, blo[1] - tol, blo[2] - tol};
+          const float hi2[3] = {bhi[0] + tol, bhi[1] + tol, bhi[2] + tol};
+          if (box_dist2(yh.x - oh[0], yh.y - oh[1], yh.z - oh[2], lo2, hi2) <
+              hh * 1.0001f + 1e-30f) {
+            y[0] = to_local(yh.x, __ldg(&r->q.w), oh[0], ol[0]);
+            y[1] = to_local(yh.y, __ldg(&r->n.w), oh[1], ol[1]);
+            y[2] = to_local(yh.z, __ldg(&r->p.w), oh[2], ol[2]);
+            cand = is_candidate(box_dist2(y[0], y[1], y[2], blo, bhi), hh);
+          }
+        }
+        for (unsigned cm = __ballot_sync(kFull, cand); cm; cm &= cm - 1) {
+          const int l = __ffs(cm) - 1;
+          const float y0 = __shfl_sync(kFull, y[0], l), y1 = __shfl_sync(kFull, y[1], l),
+                      y2 = __shfl_sync(kFull, y[2], l), h2 = __shfl_sync(kFull, hh, l);
+          const int32_t jl = __shfl_sync(kFull, j, l);
+          const uint32_t kl = __shfl_sync(kFull, kb, l);
+          unsigned nm = 0;  // this lane's near targets
+#pragma unroll
+          for (int t = 0; t < kScanT; ++t)
+            if (t * kWarp < tn) {
+              const float r2 =
+                  pair_r2(__fsub_rn(x[t][0], y0), __fsub_rn(x[t][1], y1), __fsub_rn(x[t][2], y2));
+              if (is_near(r2, h2) && self[t] != jl) nm |= 1u << t;
+            }
+          if (!__any_sync(kFull, nm != 0)) continue;
+          // queue order: by lane, then by target slot
+          const int cnt = __popc(nm);
+          const unsigned b0 = __ballot_sync(kFull, cnt & 1), b1 = __ballot_sync(kFull, cnt & 2),
+                         b2 = __ballot_sync(kFull, cnt & 4);
+          int pos = qn + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
+          for (unsigned mm = nm; mm; mm &= mm - 1, ++pos) {
+            sm.n.qt[pos] = (uint8_t)(lane + kWarp * (__ffs(mm) - 1));
+            sm.n.qj[pos] = (int32_t)((uint32_t)jl | kl);
+          }
+          qn += __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+          if (qn > kNearQueue - kScanT * kWarp) {
+            __syncwarp();
+            eval_queue(sm.n, P, it.t0, qn, lane);
+            qn = 0;
+          }
+        }
+      }
+    }
+    finish_unit(sm.n, P, it.t0, tn, it.tn_part >> 8, qn, lane);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace
+
+// Overflowed items of the U-list near field from which on a warp each (k_near_all) beats a
+// CTA each: as many as its resident warps.  262,096 points, some 4,100 overflowed items at
+// alpha 8: 5.5 ms a step with a CTA each, 7.4 with a warp; 524,000 points, 8,300: 8.1 with a
+// warp.  Items of direct sums and batches hold 64 to 128 targets, and a CTA each stays the
+// better form (64 suspensions, alpha 8: 37.6 ms, 38.4 with a warp each).
+constexpr int kAllItems = 4864;
 
 // Runs after the engine on the same stream; P is the engine's parameter block
 // (items, segments, records, partial results) and P.near_counter is zeroed.
 void launch_near(const EngineParams &P, int sms, int64_t max_items, cudaStream_t st) {
-  int64_t grid = (int64_t)sms * 8;
+  int64_t grid = (int64_t)sms * kNearMinBlocks;
   const int64_t need = (max_items + kNearWarps - 1) / kNearWarps;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  k_near<<<(int)grid, kNearWarps * kWarp, 0, st>>>(P);
+  const bool all = P.seg_list && max_items >= kAllItems;
+  const int all_from = all ? kAllItems : INT_MAX;
+  k_near<<<(int)grid, kNearWarps * kWarp, 0, st>>>(P, all_from);
   // k_near_over reads and adds to nothing of k_near's: it starts as that one's CTAs end
-  // (2 to 6 us of a call when no list has overflowed)
+  // (2 to 6 us of a call when no list has overflowed); k_near_all likewise
   cudaLaunchAttribute early;
   early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   early.val.programmaticStreamSerializationAllowed = 1;
@@ -425,8 +595,14 @@ void launch_near(const EngineParams &P, int sms, int64_t max_items, cudaStream_t
   cfg.stream = st;
   cfg.attrs = &early;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_near_over, P);
+  cudaLaunchKernelEx(&cfg, k_near_over, P, all_from);
   count_launches(2);
+  if (!all) return;
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kNearWarps * kWarp);
+  cfg.dynamicSmemBytes = 0;
+  cudaLaunchKernelEx(&cfg, k_near_all, P, all_from);
+  count_launches(1);
 }
 
 }  // namespace stk
