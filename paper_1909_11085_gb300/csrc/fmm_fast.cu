@@ -1298,8 +1298,8 @@ __global__ void k_fast_dchk(Pass P) {
   for (int e0 = 0; e0 < neqs; e0 += neq) {
     const int nb = min(neq, neqs - e0);
     __syncthreads();
-    if ((int)threadIdx.x < nb) {
-      const int e = e0 + threadIdx.x;
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) {  // (64 boxes for 32 threads at p = 2)
+      const int e = e0 + k;
       EqSrc q;
       if (e < v1 - v0) {
         const int32_t a = P.t.v_idx[v0 + e];
@@ -1322,7 +1322,7 @@ __global__ void k_fast_dchk(Pass P) {
           q = eq_none(P);
         }
       }
-      src[threadIdx.x] = q;
+      src[k] = q;
     }
     __syncthreads();
     stage_eq_pairs(P, E, cap, src, nb);
