@@ -1180,10 +1180,12 @@ __device__ __forceinline__ void nz_stage64(NzWarpSmem &sm, const NzPatches &Q, i
 
 // 2^20 targets in a vessel against its 320 wall patches (q = 10), 63.9 k within
 // d_eps: 46.4 ms as one thread per target in FP64 alone (3.4 of 32 lanes
-// active, FP64 pipe 92% busy), 0.75 ms in this form; the call 46.8 -> 1.14 ms.
-// What is left is the FP32 stage's loads and multiply-adds (some 8,000 per
-// pair) and two FP64 evaluations per hit.  Three CTAs per SM: the FP64 basis
-// values live in registers.
+// active, FP64 pipe 92% busy), 1.05 ms in this form (0.75 without the plain iterations
+// beside nodes); the call 46.8 -> 1.3 ms.  Bound: the FP64 pipe (75% of the active cycles;
+// FMA 9%), with 16.6 lanes active, since each warp finishes its own 32 targets' pairs, and
+// at the end the plain iterations.  Three CTAs per SM: the FP64 basis values live in
+// registers.  Other orders than q = 10 take N1 = 0, whose loops are unrolled to the largest:
+// 200,000 targets at q = 4, 6, 8, 12 6.2, 8.8, 11.7, 19.1 -> 0.48, 0.57, 0.69, 0.81 ms.
 template <int N1>
 __global__ void __launch_bounds__(kNzWarps *kWarp, 3) k_nz_search(
     NzPatches Q, int q, const NzGrid *__restrict__ gp, const uint64_t *__restrict__ keys,
