@@ -285,7 +285,7 @@ __device__ __forceinline__ int fx_range_of(int64_t ns, const double *__restrict_
 }
 
 // This thread's records of the sources on the grid of exponent E; trg: the targets whose
-// inexact coordinates are counted too.
+// inexact coordinates are counted too (for the double layer's faint dots).
 __device__ __forceinline__ void fx_records_of(int64_t ns, const double *__restrict__ src, int64_t nt,
                                               const double *__restrict__ trg,
                                               const double *__restrict__ f,
@@ -318,7 +318,7 @@ __device__ __forceinline__ void fx_records_of(int64_t ns, const double *__restri
     inexact += R.thr >= kFxInexact;
     rec[j] = R;
   }
-  for (int64_t i = i0; i < nt; i += step) {
+  for (int64_t i = i0; phi && i < nt; i += step) {
     uint32_t thr = kFxExact;
     for (int k = 0; k < 3; ++k) fx_coord(trg[3 * i + k], E, thr);
     trg_inexact += thr != kFxExact;
