@@ -119,8 +119,8 @@ constexpr uint32_t kFxLow = 0x3fffffffu;  // the low part: 30 bits
 
 // A pair whose largest |d_k| has a high word below both points' thresholds
 // takes the FP64 form.
-constexpr uint32_t kFxExact = 1u;          // exact coordinates: |d| < 2^32 quanta (2^36 with)
-constexpr uint32_t kFxRoundQ = 2u, kFxRoundN = 4u, kFxRoundP = 8u;  // these: q, n, psi lost bits
+constexpr uint32_t kFxExact = 1u;          // exact coordinates: |d| < 2^32 quanta (2^36 with
+constexpr uint32_t kFxRoundQ = 2u, kFxRoundN = 4u, kFxRoundP = 8u;  //   these): q, n, psi lost bits
 constexpr uint32_t kFxInexact = 1u << 22;  // an inexact coordinate: |d| < 2^54 quanta
 constexpr uint32_t kFxNever = ~0u;         // nothing of the point fits
 
@@ -197,7 +197,8 @@ FX_HD int64_t fx_coord(double v, int E, uint32_t &thr) {
 FX_HD int fx_field(double v) { return (int)((fx_to_bits(v) >> 52) & 0x7ff); }
 
 // Block fixed point of a vector; returns its exponent e (|v_k| < 2^e; 0 for a
-// zero vector, -1022, which fits no form, for one of subnormals).  `flag` is added to thr where a component loses bits.
+// zero vector, -1022, which fits no form, for one of subnormals).  `flag` is
+// added to thr where a component loses bits.
 FX_HD int fx_block(const double (&v)[3], int32_t (&h)[3], int32_t (&l)[3], uint32_t &thr,
                    uint32_t flag) {
   int ef = 0;
